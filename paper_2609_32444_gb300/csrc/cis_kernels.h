@@ -88,7 +88,7 @@ cudaError_t launch_seq_weights(const double *lw64, const float *lw32, const floa
                                const int32_t *cu_seqlens, int64_t B, int64_t T,
                                const DevParams &P, float *w, uint8_t *trunc, cudaStream_t s);
 
-// Forward-only: lp (and lse) of the sampled token, one CTA per row.
+// Forward-only: lp (and lse, entropy) of the sampled token, any layout.
 cudaError_t launch_token_logprobs(const PassArgs &a, int dtype, cudaStream_t s);
 
 // Fused forward + backward, any layout: one CTA per row, second read from L2.

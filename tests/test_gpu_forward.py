@@ -1,0 +1,93 @@
+"""The forward kernel of cis_token_logprobs at the sizes where its row split
+and its ragged ends can go wrong, against fp64 log-softmaxes of the same rows.
+
+Tolerance of log p: 2e-5 plus four fp32 steps of it, as everywhere else; of
+the entropy, whose terms are bounded by log V, 2e-5 (1 + log V).
+"""
+import math
+
+import pytest
+import torch
+
+from paper_2609_32444_gb300 import binding
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+DEV = torch.device("cuda")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2609_32444_gb300 import build
+    build.build()
+    binding.lib()
+
+
+def _check(z, ids):
+    """Every output of the forward pass on rows z (a view of any stride)."""
+    T, V = z.shape
+    mask = torch.ones(T, dtype=torch.uint8, device=DEV)
+    mask[T // 2] = 0
+    plain = binding.cis_token_logprobs(z, ids, mask=mask)
+    lp, lse, ent = binding.cis_token_logprobs(z, ids, mask=mask, want_lse=True,
+                                              want_entropy=True)
+    on = mask != 0
+    x = z.double()
+    r = torch.arange(T, device=DEV)
+    zy = x[r, ids.long()]
+    rest = x.clone()
+    rest[r, ids.long()] = -math.inf
+    odds = zy - torch.logsumexp(rest, 1)
+    want = -torch.nn.functional.softplus(-odds).masked_fill(~on, 0)
+    want_lse = torch.logsumexp(x, 1).masked_fill(~on, 0)
+    ls = x - torch.logsumexp(x, 1, keepdim=True)
+    p = ls.exp()
+    want_ent = -torch.where(p > 0, p * ls, torch.zeros_like(p)).sum(1).masked_fill(~on, 0)
+    tol = 2e-5 + 2.0 ** -21 * want.abs()
+    assert bool(((lp.double() - want).abs() <= tol).all())
+    assert bool(((plain.double() - want).abs() <= tol).all())
+    assert bool(((lse.double() - want_lse).abs() <= 2e-5 + 2.0 ** -21 * want_lse.abs()).all())
+    assert bool(((ent.double() - want_ent).abs() <= 2e-5 * (1 + math.log(V))).all())
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("T,V", [
+    (5, 1), (5, 2), (4, 7), (4, 8), (4, 9), (6, 15), (3, 63), (3, 2049),   # 64 threads a row
+    (4, 4096), (4, 4097), (3, 4104), (700, 8200),                           # 256 threads a row
+    (300, 8207), (150, 16391), (3, 16391), (2, 40003)])                     # 2 to 8 CTAs a row
+def test_row_splits_and_ragged_ends(dtype, T, V):
+    """Rows that start at every offset from a 16-byte boundary (an odd stride
+    and an odd first element), the sampled token at either end and inside."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(V)
+    for pad, off in ((0, 0), (3, 1)):
+        buf = torch.randn(T * (V + pad) + off, generator=g, device=DEV).mul_(4).to(dtype)
+        z = buf[off:].view(T, V + pad)[:, :V]
+        ids = torch.randint(0, V, (T,), generator=g, device=DEV).int()
+        ids[0], ids[-1] = 0, V - 1
+        ids[T // 3] = min(V - 1, 9)
+        _check(z, ids)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("fill", ["lowest", "neg_inf"])
+def test_rows_of_masked_entries(dtype, fill):
+    """Rows with all but a few entries at the type's lowest value, or at -inf:
+    whole batches of a thread hold nothing else, and one row holds only its
+    sampled token; another is at the lowest value throughout."""
+    T, V = 4, 9000
+    low = torch.finfo(dtype).min if fill == "lowest" else -math.inf
+    z = torch.full((T, V), low, dtype=dtype, device=DEV)
+    ids = torch.tensor([17, 8999, 5000, 3], dtype=torch.int32, device=DEV)
+    z[0, 17:8000:900] = 1.5
+    z[1, 8990:] = -2.0
+    z[2, 5000] = 3.0
+    if fill == "lowest":
+        lp, lse = binding.cis_token_logprobs(z, ids, want_lse=True)
+        want = torch.tensor([-math.log(9), -math.log(10), 0.0, -math.log(V)], device=DEV)
+        assert bool(((lp - want).abs() <= 2e-5 + 2.0 ** -21 * want.abs()).all())
+        assert float(lse[3]) == low
+        return
+    z[3, :5] = 0.25
+    _check(z, ids)
