@@ -76,6 +76,22 @@ def test_binned_sums_bin_and_value_counts(nbins, nvalues):
     _compare(one_minus_p, edges, values)
 
 
+def test_keys_beside_edges_that_are_not_floats():
+    """Edges between two float32 values, three of them between the same two, and
+    beyond float32's range: keys on either side of each fall where fp64
+    comparisons put them."""
+    f = np.float32(0.3)
+    up = np.nextafter(f, np.float32(1))
+    mid = (float(f) + float(up)) / 2
+    edges = [-1e300, -1.0 - 1e-12, 0.1, float(f), mid - 1e-10, mid, mid + 1e-10, 0.7, 1e300]
+    key = np.array([f, up, 0.1, np.nextafter(np.float32(0.1), np.float32(0)), -1.0,
+                    np.nextafter(np.float32(-1), np.float32(-2)), 0.7, -np.inf, np.inf,
+                    np.finfo(np.float32).max, np.nan], np.float32)
+    key = np.tile(key, 41)
+    val = np.random.default_rng(3).standard_normal(key.size).astype(np.float32)
+    _compare(key, edges, [val])
+
+
 def test_binned_sums_are_deterministic():
     """Fixed-order sums: two calls give the same bits."""
     rng = np.random.default_rng(5)
