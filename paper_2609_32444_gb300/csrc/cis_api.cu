@@ -71,7 +71,10 @@ DevParams make_dev_params(const cis_params_t &p)
     d.log_rho_hi_f = (float)d.log_rho_hi;
     d.log_icepop_lo = log(p.icepop_lo);
     d.log_icepop_hi = log(p.icepop_hi);
+    d.log_icepop_lo_f = (float)d.log_icepop_lo;
+    d.log_icepop_hi_f = (float)d.log_icepop_hi;
     d.kpop_phi = p.kpop_phi;
+    d.kpop_phi_f = (float)p.kpop_phi;
     d.seq_cap = p.seq_cap;
     d.log_seq_cap = log(p.seq_cap);
     d.log_seq_lo = log(p.seq_lo);

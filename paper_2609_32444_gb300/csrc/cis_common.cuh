@@ -40,6 +40,7 @@ struct DevParams {
     float tis_cap_f, exact_lo_f, exact_hi_f;
     float rho_lo_f, rho_hi_f;  // 1 - c_low, 1 + c_high
     float log_tis_cap_f, log_exact_lo_f, log_exact_hi_f, log_rho_lo_f, log_rho_hi_f;
+    float log_icepop_lo_f, log_icepop_hi_f, kpop_phi_f;
     double lam, kappa;
     double log_tis_cap, log_exact_lo, log_exact_hi, log_rho_lo, log_rho_hi;
     double log_icepop_lo, log_icepop_hi, kpop_phi;
@@ -126,6 +127,50 @@ __device__ __forceinline__ int certain_cmp(float a, float b)
     return 0;
 }
 
+// e^{x + x_lo} as an unevaluated fp32 pair, within 2^-29 (2^-28 for x > 0),
+// for x <= 0 (x above 0.5, or NaN, takes fp64): x is reduced to n ln 2 + r,
+// |r| <= 0.35, with ln 2 in three parts whose products with n are exact or
+// negligible, and e^r is its Taylor series, the first two terms kept as a pair.
+__device__ __forceinline__ float exp_pair(float x, float x_lo, float &lo)
+{
+    if (!(x <= 0.5f)) {
+        const double e = exp((double)x + (double)x_lo);
+        const float h = (float)e;
+        lo = isfinite(h) ? (float)(e - (double)h) : 0.0f;
+        return h;
+    }
+    if (x < -80.0f) {  // below every use: 1 - p and (1 + p)/2 do not see it
+        lo = 0.0f;
+        return 0.0f;
+    }
+    const float n = rintf(x * kLog2e);
+    // ln 2 = 0x1.62ep-1 + 0x1.0bfbe8p-15 + 0x1.cf79acp-40 (+ 2^-65): n has 7
+    // bits, so n times the first part (13 bits) is exact, and x minus it as
+    // well (nearby values)
+    const float t0 = fmaf(n, -0x1.62ep-1f, x);
+    float e1;
+    const float p1 = n * -0x1.0bfbe8p-15f, p1e = fmaf(n, -0x1.0bfbe8p-15f, -p1);
+    const float r = two_sum(t0, p1, e1);
+    const float rl = e1 + (p1e + fmaf(n, -0x1.cf79acp-40f, x_lo));  // r + rl = x - n ln 2
+    // e^r - 1 - r - r^2/2, then r^2/2 as a pair
+    float q = 1.0f / 40320.0f;
+    q = fmaf(q, r, 1.0f / 5040.0f);
+    q = fmaf(q, r, 1.0f / 720.0f);
+    q = fmaf(q, r, 1.0f / 120.0f);
+    q = fmaf(q, r, 1.0f / 24.0f);
+    q = fmaf(q, r, 1.0f / 6.0f);
+    const float h = 0.5f * r, s2 = h * r, s2e = fmaf(h, r, -s2);
+    float a, b;
+    const float u = two_sum(r, s2, a);  // r + r^2/2
+    const float v = two_sum(1.0f, u, b);
+    const float w = b + (a + (fmaf(q * r, r * r, s2e) + rl * (1.0f + u)));
+    float c;
+    const float hi = two_sum(v, w, c);
+    const float sc = __int_as_float((127 + (int)n) << 23);
+    lo = c * sc;
+    return hi * sc;
+}
+
 struct TokenWeight {
     float w;
     float logk;
@@ -190,33 +235,64 @@ __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float
     }
     case CIS_MODE_BAND: {
         // Sec. 4.3: the CIS weight, lifted from below to (1 + p)/2 (the image
-        // of e^eps = 1/2); both decisions in fp64
-        const double phi = fmax(-expm1(lw64()), P.kappa);
-        const double lo = 0.5 * (1.0 + exp(lw64()));
-        const bool up = logk64() > log1p(P.lam * phi);
-        const bool low = logk64() < log(lo);
+        // of e^eps = 1/2).  Both comparisons as for CIS; k near (1 + p)/2 lies
+        // in [1/2, 1], where its error is smaller still
+        const float om = omp >= 0.0f ? omp : -expm1f(lw);
+        const float k = expf(logk);
+        const float lo = om < 0.5f ? 1.0f - 0.5f * om : 0.5f + 0.5f * expf(lw);
+        const int su = certain_cmp(k, 1.0f + P.lam_f * fmaxf(om, P.kappa_f));
+        const int sl = certain_cmp(lo, k);
+        const bool up =
+            su != 0 ? su > 0 : logk64() > log1p(P.lam * fmax(-expm1(lw64()), P.kappa));
+        const bool low = sl != 0 ? sl > 0 : logk64() < log(0.5 * (1.0 + exp(lw64())));
         r.trunc = up || low;
-        r.w = up ? (float)(1.0 + P.lam * phi) : (low ? (float)lo : expf(logk));
+        r.w = k;
+        if (up || low) {  // the bounds themselves, to fp32 rounding
+            float pl, e, ph = exp_pair(lw, lw_lo, pl);
+            const float half = two_sum(0.5f, 0.5f * ph, e);
+            r.w = up ? (float)(1.0 + P.lam * fmax((1.0 - (double)ph) - (double)pl, P.kappa))
+                     : half + fmaf(0.5f, pl, e);
+        }
         break;
     }
     case CIS_MODE_ICEPOP: {
         // Table 8: k on [lo, hi] (bounds included), else masked
-        const bool out = logk64() < P.log_icepop_lo || logk64() > P.log_icepop_hi;
+        const int sl = certain_cmp(P.log_icepop_lo_f, logk);
+        const int sh = certain_cmp(logk, P.log_icepop_hi_f);
+        const bool out = (sl != 0 ? sl > 0 : logk64() < P.log_icepop_lo) ||
+                         (sh != 0 ? sh > 0 : logk64() > P.log_icepop_hi);
         r.trunc = out;
         r.w = out ? 0.0f : expf(logk);
         break;
     }
     case CIS_MODE_KPOP: {
-        // Table 8 / App. D.5: binary KL both ways in fp64 on probabilities
-        // clamped to [1e-8, 1 - 1e-8]; masked when the larger exceeds phi
-        const double lo = 1e-8, hi = 1.0 - 1e-8;
-        double p = exp(lw64()), q = exp((double)linf);
-        p = p < lo ? lo : (p > hi ? hi : p);
-        q = q < lo ? lo : (q > hi ? hi : q);
-        const double kl_pq = p * log(p / q) + (1.0 - p) * log((1.0 - p) / (1.0 - q));
-        const double kl_qp = q * log(q / p) + (1.0 - q) * log((1.0 - q) / (1.0 - p));
-        const double m = kl_pq > kl_qp ? kl_pq : kl_qp;
-        const bool out = m > P.kpop_phi;
+        // Table 8 / App. D.5: binary KL both ways on probabilities clamped to
+        // [1e-8, 1 - 1e-8]; masked when the larger exceeds phi.  fp32 decides
+        // unless the two are close.  With L = log p - log q and M = log(1 - p)
+        // - log(1 - q) of the clamped values, |L|, |M| <= 18.5, the two KLs are
+        // p L + (1 - p) M and -(q L + (1 - q) M); p, 1 - p, q and 1 - q carry
+        // relative errors below 1e-6 and the four logs absolute errors below
+        // 6e-6, so each KL is off by less than 1e-6 (2 * 18.5) + 2 * 1.2e-5 <
+        // 7e-5; 2e-4 is taken.  (The clamps drop a NaN: fp64 keeps it.)
+        const float fl = 1e-8f, ll = -18.420681f;  // the clamp and its log
+        const float om = omp >= 0.0f ? omp : -expm1f(lw), oq = -expm1f(linf);
+        const float a = fminf(fmaxf(lw, ll), -fl), b = fminf(fmaxf(linf, ll), -fl);
+        const float p = expf(a), q = expf(b);
+        const float p1 = fminf(fmaxf(om, fl), 1.0f), q1 = fminf(fmaxf(oq, fl), 1.0f);
+        const float L = a - b, M = logf(p1) - logf(q1);
+        const float kl = fmaxf(p * L + p1 * M, -(q * L + q1 * M));
+        const float d = kl - P.kpop_phi_f;
+        bool out = d > 0.0f;
+        if (!(fabsf(d) > 2e-4f + 1e-6f * P.kpop_phi_f) || logk != logk) {
+            const double lo = 1e-8, hi = 1.0 - 1e-8;
+            double dp = exp(lw64()), dq = exp((double)linf);
+            dp = dp < lo ? lo : (dp > hi ? hi : dp);
+            dq = dq < lo ? lo : (dq > hi ? hi : dq);
+            const double kl_pq = dp * log(dp / dq) + (1.0 - dp) * log((1.0 - dp) / (1.0 - dq));
+            const double kl_qp = dq * log(dq / dp) + (1.0 - dq) * log((1.0 - dq) / (1.0 - dp));
+            const double m = kl_pq > kl_qp ? kl_pq : kl_qp;
+            out = m > P.kpop_phi;
+        }
         r.trunc = out;
         r.w = out ? 0.0f : expf(logk);
         break;

@@ -123,6 +123,49 @@ def test_token_operators_on_shared_fp32_inputs(mode):
     assert 0 < rtr.sum() < len(rtr)
 
 
+@pytest.mark.parametrize("phi", [1e-5, 0.1, 2.0])
+def test_kpop_decisions_close_to_the_threshold(phi):
+    """Pairs whose binary KL lies from 1e-9 to 3e-3 either side of phi (found by
+    bisection over log q in fp64), over all confidences: those within the fp32
+    margin are settled in fp64, so every decision is the oracle's."""
+    rng = np.random.default_rng(5)
+    n = 4000
+    lw = -np.exp(rng.uniform(np.log(1e-7), np.log(17.0), n)).astype(np.float32)
+    lo, hi = np.minimum(lw.astype(np.float64), -1e-9), np.full(n, -18.4)
+    for _ in range(60):  # the KL grows with the distance from log p
+        mid = 0.5 * (lo + hi)
+        over = _kpop_metric(lw.astype(np.float64), mid) > phi
+        hi, lo = np.where(over, mid, hi), np.where(over, lo, mid)
+    off = rng.choice([-1, 1], n) * 10.0 ** rng.uniform(-9, -2.5, n)
+    li = np.minimum(lo * (1 + off), -1e-30).astype(np.float32)
+    w, tr, _ = binding.cis_weights(torch.from_numpy(lw).to(DEV), torch.from_numpy(li).to(DEV),
+                                   binding.cis_default_params("kpop", kpop_phi=phi))
+    rw, rtr, _, _ = oracle.weights(lw.astype(np.float64), li.astype(np.float64),
+                                   oracle.params(mode=OMODE["kpop"], kpop_phi=phi))
+    m = _kpop_metric(lw.astype(np.float64), li.astype(np.float64))
+    clear = np.abs(m - phi) > 1e-9
+    tr = tr.cpu().numpy()
+    assert np.array_equal(tr[clear], rtr[clear])
+    assert 0 < rtr.sum() < n
+
+
+def test_band_bounds_are_rounded_once():
+    """The band's two bounds, formed from fp32 pairs, are the fp64 values rounded
+    to fp32: within half a step and 2^-28 of the bound (the pair's error)."""
+    rng = np.random.default_rng(6)
+    lw = -np.exp(rng.uniform(np.log(1e-8), np.log(30.0), 100_000)).astype(np.float32)
+    li = np.minimum(lw + np.where(rng.random(lw.size) < 0.5, -9.0, 9.0), -1e-9).astype(np.float32)
+    w, tr, _ = binding.cis_weights(torch.from_numpy(lw).to(DEV), torch.from_numpy(li).to(DEV),
+                                   binding.cis_default_params("band"))
+    rw, rtr, _, _ = oracle.weights(lw.astype(np.float64), li.astype(np.float64),
+                                   oracle.params(mode=OMODE["band"]))
+    tr, w = tr.cpu().numpy(), w.cpu().numpy().astype(np.float64)
+    on = (tr != 0) & (rtr != 0)
+    assert on.sum() > 1000
+    step = np.spacing(rw[on].astype(np.float32)).astype(np.float64)
+    assert np.all(np.abs(w[on] - rw[on]) <= 0.5 * step + 3.3 * 2.0 ** -28 * rw[on])
+
+
 @pytest.mark.parametrize("mode", SEQ)
 def test_sequence_operators_cis_weights(mode):
     """Responses of 1 to 300 tokens with masked tokens inside and tokens outside
