@@ -15,7 +15,9 @@
 //        and write it as dz [Tp, w];
 //   DH   dH (+)= dz W[v0 : v0 + w]   (K = w, fp32 accumulator);
 //   DW   dW[v0 : v0 + w] = dz^T H    (K = T);
-//   DH and DW of a chunk run as one launch with a balanced schedule.
+//   DH and DW of a chunk run as one launch with a balanced schedule; with few
+//   tokens DH's contraction is cut into ranges (split_for).
+// Masked tokens are left out of all four products (cis_lmhead_compact_kernel).
 //
 // dz exists one chunk at a time (the chunk width follows the workspace the
 // caller gives); z never exists outside TMEM.  Every operand is read where
@@ -41,11 +43,8 @@
 // to its end, so that TMEM is always released.
 #include <cuda.h>
 #include <cudaTypedefs.h>
-#include <array>
-#include <map>
-#include <memory>
+#include <algorithm>
 #include <mutex>
-#include <vector>
 
 #include "cis_kernels.h"
 #include "cis_tc.cuh"
@@ -126,8 +125,21 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 struct GemmArgs {
     int nMt, nNt, nK;
     int raster_n;  // 1: tile i -> (m = i % nMt, n = i / nMt); 0: (m = i / nNt, n = i % nNt)
+    // Batches with masked tokens: the valid ones' number, on the device (null:
+    // every token counts).  It replaces the host's row count, along M (FWD, DZ,
+    // DH: nMt, rows_valid) or along K (DW: nK).
+    const int *count;
+    int count_k;
+    // kStats, kDz: token of a row, for ids; kStore, kAccum: output row of a row
+    // (null: the row itself)
+    const int *rowmap;
+    // kStore, kAccum: the contraction in `splits` ranges of ksplit K blocks,
+    // range i stored split_stride elements after range i - 1
+    int splits, ksplit;
+    int64_t split_stride;
     int a_row0, a_k0, b_row0, b_k0;
-    // kStats, kDz: rows are tokens, columns vocabulary entries col0 + n 256 + c
+    // kStats, kDz: rows are tokens (rows_valid of them), columns vocabulary
+    // entries col0 + n 256 + c; T: row stride of part and part_u
     int T, V, col0;
     const int32_t *ids;
     const float *lse, *cvec;
@@ -198,29 +210,58 @@ __device__ __forceinline__ void tile_mn(const GemmArgs &g, int i, int &m, int &n
         n = i - m * g.nNt;
     }
 }
-// Work unit u of a launch: a tile, or with MC (2-CTA clusters) a pair of
+// The launch's arguments with the device's token count in place of the host's.
+// At least one row tile (one K block) is kept, so that every output is written
+// when no token is valid: its rows are dead, and their dz zero.
+__device__ __forceinline__ GemmArgs live_args(const GemmArgs &in)
+{
+    GemmArgs g = in;
+    if (in.count) {
+        const int n = *in.count;
+        if (in.count_k) {
+            g.nK = n > 0 ? (n + kBK - 1) / kBK : 1;
+            g.ksplit = g.nK;
+        } else {
+            g.nMt = n > 0 ? (n + kBM - 1) / kBM : 1;
+            g.rows_valid = n;
+        }
+    }
+    return g;
+}
+// Work unit u of a launch: a tile (in one K range), or with MC (2-CTA clusters) a pair of
 // tiles in row tiles 2 mp and 2 mp + 1 of one column tile, CTA `rank` of the
 // cluster taking row tile 2 mp + rank.  The pair shares its B tile: each CTA
 // loads one half of it and multicasts it to both.  With an odd number of row
 // tiles the last pair's second tile lies past the rows (m == nMt): its CTA
-// still loads and multicasts its half of B, and its A reads as zeros, but its
-// epilogue writes nothing.
-template <bool MC> __host__ __device__ __forceinline__ int n_units(const GemmArgs &g)
+// still loads and multicasts its half of B, and its A reads as zeros (or, with
+// masked tokens left out, whatever lies there), but its epilogue writes nothing.
+template <bool MC> __device__ __forceinline__ int n_tiles(const GemmArgs &g)
 {
     return MC ? ((g.nMt + 1) >> 1) * g.nNt : g.nMt * g.nNt;
 }
+// Unit u: its tile and its K range [k0, k0 + nk), in blocks.
+struct Unit {
+    int m, n, split, k0, nk;
+};
 template <bool MC>
-__device__ __forceinline__ void unit_mn(const GemmArgs &g, int u, int rank, int &m, int &n)
+__device__ __forceinline__ Unit unit_at(const GemmArgs &g, int u, int rank)
 {
+    Unit w;
+    const int tiles = n_tiles<MC>(g);
+    w.split = g.splits > 1 ? u / tiles : 0;
+    u -= w.split * tiles;
+    w.k0 = w.split * g.ksplit;
+    w.nk = g.nK - w.k0 < g.ksplit ? g.nK - w.k0 : g.ksplit;
     if (!MC) {
-        tile_mn(g, u, m, n);
-        return;
+        tile_mn(g, u, w.m, w.n);
+        return w;
     }
     GemmArgs gp = g;
     gp.nMt = (g.nMt + 1) >> 1;  // the pairs' own grid of (row pair, column) units
     int mp;
-    tile_mn(gp, u, mp, n);
-    m = 2 * mp + rank;
+    tile_mn(gp, u, mp, w.n);
+    w.m = 2 * mp + rank;
+    return w;
 }
 
 // Where the producer, or the MMA thread, is in the ring of stages.
@@ -236,16 +277,17 @@ struct Ring {
     }
 };
 
-// The producer's loads for tile (m, n): nK stages.  `used` and `last` record
+// The producer's loads for unit w: w.nk stages.  `used` and `last` record
 // per stage whether it was ever loaded and the parity of its last load, for
 // the drain before the CTA leaves.  Returns early once the CTA aborted.
 template <bool A_MN, bool B_MN, bool MC>
 __device__ __forceinline__ void load_tile(const CUtensorMap &tmA, const CUtensorMap &tmB,
-                                          const GemmArgs &g, int m, int n, int rank,
+                                          const GemmArgs &g, const Unit &w, int rank,
                                           uint8_t *ring, Barriers &bars, const Abort &ab,
                                           Ring &p, uint32_t &used, uint32_t &last)
 {
-    for (int kb = 0; kb < g.nK; ++kb) {
+    const int m = w.m, n = w.n;
+    for (int kb = w.k0; kb < w.k0 + w.nk; ++kb) {
         if (!ab.wait(&bars.empty[p.stage], p.phase ^ 1))
             return;
         uint64_t *full = &bars.full[p.stage];
@@ -283,10 +325,10 @@ __device__ __forceinline__ void load_tile(const CUtensorMap &tmA, const CUtensor
     }
 }
 
-// The MMAs of one tile into the accumulator at TMEM column d: nK stages of
+// The MMAs of one unit into the accumulator at TMEM column d: nk stages of
 // four K=16 steps.  Returns early once the CTA aborted.
 template <bool A_MN, bool B_MN, bool MC>
-__device__ __forceinline__ void mma_tile(const GemmArgs &g, uint32_t d, uint8_t *ring,
+__device__ __forceinline__ void mma_tile(int nk, uint32_t d, uint8_t *ring,
                                          Barriers &bars, const Abort &ab, Ring &p)
 {
     constexpr uint32_t kId =
@@ -302,7 +344,7 @@ __device__ __forceinline__ void mma_tile(const GemmArgs &g, uint32_t d, uint8_t 
     const uint64_t da0 = A_MN ? tc::desc_sw128_mn(s0, kMnBox) : tc::desc_sw128(s0);
     const uint64_t db0 =
         B_MN ? tc::desc_sw128_mn(s0 + kStageA, kMnBox) : tc::desc_sw128(s0 + kStageA);
-    for (int kb = 0; kb < g.nK; ++kb) {
+    for (int kb = 0; kb < nk; ++kb) {
         if (!ab.wait(&bars.full[p.stage], p.phase))
             return;
         tc::fence_after_sync();
@@ -324,12 +366,12 @@ __device__ __forceinline__ void mma_tile(const GemmArgs &g, uint32_t d, uint8_t 
 // first column of the tile's accumulator.
 template <int EPI>
 __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, uint32_t taddr, int m, int n,
-                                              int r, int half)
+                                              int split, int r, int half)
 {
     const int cbeg = half * kHalf;
     if (EPI == kStats) {
         const int row = m * kBM + r;  // token
-        const int y_r = row < g.T ? g.ids[row] : -1;
+        const int y_r = row < g.rows_valid ? g.ids[row] : -1;
         const bool ent = g.part_u != nullptr;
         float mx = -INFINITY, s = 0.0f, u = 0.0f, zyv = 0.0f;
         bool got_y = false;
@@ -380,7 +422,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, uint32_t taddr,
                 u += au;
             }
         }
-        if (row < g.T) {  // one (max, sum) per 128-column half
+        if (row < g.rows_valid) {  // one (max, sum) per 128-column half
             const int64_t pi = (int64_t)(2 * n + half) * g.T + row;
             g.part[pi] = make_float2(mx, s);
             if (ent)
@@ -390,12 +432,12 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, uint32_t taddr,
         }
     } else if (EPI == kDz) {
         const int row = m * kBM + r;  // token; rows up to Tp are allocated
-        const bool live = row < g.T;
-        // tokens with c = 0 (masked, clipped, past T) give 0 without
+        const bool live = row < g.rows_valid;
+        // tokens with c = 0 (masked, clipped, past the last) give 0 without
         // touching the exponential (their lse is a placeholder)
         const float c_r = live ? g.cvec[row] : 0.0f;
         const float lse_r = live ? g.lse[row] : 0.0f;
-        const int y_r = live ? g.ids[row] : -1;
+        const int y_r = live ? g.ids[g.rowmap ? g.rowmap[row] : row] : -1;
         const int cl0 = n * kBN;  // chunk-local column of the tile
         for (int c0 = cbeg; c0 < cbeg + kHalf; c0 += 32) {
             float v[32];
@@ -424,7 +466,9 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, uint32_t taddr,
     } else {
         const int lr = m * kBM + r;  // row of the output block
         const bool live = lr < g.rows_valid;
-        const int64_t o = (int64_t)lr * g.ld_out + (int64_t)n * kBN;
+        const int orow = live && g.rowmap ? g.rowmap[lr] : lr;
+        const int64_t o =
+            (int64_t)split * g.split_stride + (int64_t)orow * g.ld_out + (int64_t)n * kBN;
         for (int c0 = cbeg; c0 < cbeg + kHalf; c0 += 32) {
             float v[32];
             tc::tmem_ld32(taddr + c0, v);
@@ -562,7 +606,7 @@ template <bool MC> __device__ __forceinline__ void gemm_teardown(GemmShared &sh,
 // hand it back.  Warps 2..9: TMEM lane quadrant warp % 4 (one tile row per
 // thread), column half (warp - 2) / 4 of the 256-column tile.
 template <int EPI, bool MC>
-__device__ __forceinline__ void epilogue_unit(const GemmArgs &g, int m, int n, int i,
+__device__ __forceinline__ void epilogue_unit(const GemmArgs &g, const Unit &w, int i,
                                               uint32_t tmem, int warp, int lane, Barriers &bars,
                                               const Abort &ab)
 {
@@ -573,8 +617,9 @@ __device__ __forceinline__ void epilogue_unit(const GemmArgs &g, int m, int n, i
     ab.wait(&bars.accfull[acc], (i >> 1) & 1);
     tc::fence_after_sync();
     // with MC, the padding tile of an odd row count has nothing to write
-    if (!(MC && m >= g.nMt))
-        epilogue_tile<EPI>(g, tmem + lane_off + acc * kBN, m, n, lg * 32 + lane, half);
+    if (!(MC && w.m >= g.nMt))
+        epilogue_tile<EPI>(g, tmem + lane_off + acc * kBN, w.m, w.n, w.split, lg * 32 + lane,
+                           half);
     tc::fence_before_sync();
     tc::bar_arrive(&bars.accempty[acc]);
 }
@@ -582,27 +627,29 @@ __device__ __forceinline__ void epilogue_unit(const GemmArgs &g, int m, int n, i
 // The MMA thread's part of one tile: a free accumulator, the tile's MMAs,
 // then the accumulator handed to the epilogue.
 template <bool A_MN, bool B_MN, bool MC>
-__device__ __forceinline__ void mma_unit(const GemmArgs &g, int i, uint32_t tmem, uint8_t *ring,
+__device__ __forceinline__ void mma_unit(int nk, int i, uint32_t tmem, uint8_t *ring,
                                          Barriers &bars, const Abort &ab, Ring &p)
 {
     const int acc = i & 1;
     ab.wait(&bars.accempty[acc], ((i >> 1) & 1) ^ 1);
     tc::fence_after_sync();
-    mma_tile<A_MN, B_MN, MC>(g, tmem + acc * kBN, ring, bars, ab, p);
+    mma_tile<A_MN, B_MN, MC>(nk, tmem + acc * kBN, ring, bars, ab, p);
     tc::mma_commit(&bars.accfull[acc]);
 }
 
-template <int EPI, bool A_MN, bool B_MN, bool MC>
+// FWD and DZ: z tiles of H W^T, both operands K-major.
+template <int EPI, bool MC>
 __global__ void __launch_bounds__(kThreads, 1)
     cis_lmhead_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
-                           const __grid_constant__ CUtensorMap tmB, const GemmArgs g)
+                           const __grid_constant__ CUtensorMap tmB, const GemmArgs args)
 {
     extern __shared__ __align__(1024) uint8_t dsm[];
     uint8_t *ring = dsm + ((1024 - (tc::smem_addr(dsm) & 1023)) & 1023);
     __shared__ __align__(8) GemmShared sh;
 
+    const GemmArgs g = live_args(args);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nUnits = n_units<MC>(g);
+    const int nUnits = n_tiles<MC>(g);
     const int rank = MC ? (int)tc::cluster_ctarank() : 0;
     const int unit0 = MC ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
     const int ustep = MC ? (int)(gridDim.x >> 1) : (int)gridDim.x;
@@ -616,10 +663,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             Ring p;
             uint32_t used = 0, last = 0;
             for (int u = unit0; u < nUnits && !ab.on(); u += ustep) {
-                int m, n;
-                unit_mn<MC>(g, u, rank, m, n);
-                load_tile<A_MN, B_MN, MC>(tmA, tmB, g, m, n, rank, ring, sh.bars, ab, p, used,
-                                          last);
+                load_tile<false, false, MC>(tmA, tmB, g, unit_at<MC>(g, u, rank), rank, ring,
+                                            sh.bars, ab, p, used, last);
             }
             drain_loads(sh.bars, used, last);
         }
@@ -628,7 +673,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             Ring p;
             int i = 0;
             for (int u = unit0; u < nUnits && !ab.on(); u += ustep, ++i)
-                mma_unit<A_MN, B_MN, MC>(g, i, tmem, ring, sh.bars, ab, p);
+                mma_unit<false, false, MC>(g.nK, i, tmem, ring, sh.bars, ab, p);
             drain_mmas(sh.bars);
         }
     } else {  // epilogue
@@ -636,48 +681,82 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int u = unit0; u < nUnits; u += ustep, ++i) {
             if (__syncthreads_or_epi(ab.on()))
                 break;
-            int m, n;
-            unit_mn<MC>(g, u, rank, m, n);
-            epilogue_unit<EPI, MC>(g, m, n, i, tmem, warp, lane, sh.bars, ab);
+            epilogue_unit<EPI, MC>(g, unit_at<MC>(g, u, rank), i, tmem, warp, lane, sh.bars, ab);
         }
     }
     gemm_teardown<MC>(sh, warp);
 }
 
 // The dH and dW GEMMs of one vocabulary chunk in one launch.  Launched one
-// after the other, each ends in a partial wave: dH has 512 pair units of 512 K
-// blocks for 76 clusters (6.7 waves), dW 1024 of 256 (13.5 waves).  Here
-// every group (a cluster with MC, else a CTA) works through its own list of
-// units from both GEMMs: a greedy schedule made on the host, which hands the
-// units out in order (all of dH, then dW) to the group that frees up first, by
-// their K blocks.  The lists are kernel parameters.
-constexpr int kMaxSchedGroups = 160;
-constexpr int kMaxSchedUnits = 4096;
-constexpr uint16_t kSchedSecond = 0x8000;  // a unit of the second GEMM
-struct DualSched {
-    uint16_t off[kMaxSchedGroups + 1];  // group c takes unit[off[c]] .. unit[off[c + 1] - 1]
-    uint16_t unit[kMaxSchedUnits];      // unit index, | kSchedSecond for the second GEMM
+// after the other, each ends in a partial wave: at T=16384 dH has 512 pair units
+// of 512 K blocks for 76 clusters (6.7 waves), dW 1024 of 256 (13.5 waves), and
+// few tokens leave most clusters without any dH unit.  Here group c of G (a
+// cluster with MC, else a CTA) takes dH units c, c + G, ...; the L groups that
+// got one fewer then take dW units alone, until they have caught up by K blocks
+// (A units in all); the rest of dW goes round all groups, those L first.  The
+// units of one GEMM go out in order, so the groups at work at any time hold
+// neighbouring units, which share their operands in L2.  Every group works its
+// list out for itself, so the token count may be the device's.
+// A dW unit is taken to cost at least kDwBlocks K blocks: with few of them, what
+// its 256 KB of output costs (T=512: 5.7 us a unit, 8 blocks' worth being 2.7).
+constexpr int kDwBlocks = 16;
+struct DualList {
+    int c, G, n_dh, n_a, n_b, pos, L, A;
+    __device__ __forceinline__ int size() const { return n_dh + n_a + n_b; }
+    // Item i: a dH unit (true) or a dW unit, and its index.
+    __device__ __forceinline__ bool item(int i, int &u) const
+    {
+        if (i < n_dh) {
+            u = c + i * G;
+            return true;
+        }
+        i -= n_dh;
+        u = i < n_a ? pos + i * L : A + pos + (i - n_a) * G;
+        return false;
+    }
 };
+template <bool MC>
+__device__ __forceinline__ DualList dual_list(const GemmArgs &g0, const GemmArgs &g1, int c,
+                                              int G)
+{
+    const int n0 = n_tiles<MC>(g0) * g0.splits, n1 = n_tiles<MC>(g1) * g1.splits;
+    const int q = n0 / G, r = n0 - q * G;
+    DualList d;
+    d.c = c;
+    d.G = G;
+    d.L = r ? G - r : 0;
+    d.pos = c >= r ? c - r : c - r + G;
+    d.n_dh = q + (c < r);
+        const int cost1 = g1.ksplit > kDwBlocks ? g1.ksplit : kDwBlocks;
+    const int x = d.L ? g0.ksplit / cost1 : 0;
+    d.A = d.L * x < n1 ? d.L * x : n1;
+    d.n_a = d.pos < d.L && d.A > d.pos ? (d.A - d.pos + d.L - 1) / d.L : 0;
+    const int rest = n1 - d.A - d.pos;
+    d.n_b = rest > 0 ? (rest + G - 1) / G : 0;
+    return d;
+}
 
 // GEMM 0: dH (+)= dz W_c (A = dz K-major, B = W MN-major, EPI0 = kStore on
 // the first chunk, kAccum after); GEMM 1: dW_c = dz^T H (A = dz MN-major,
-// B = H MN-major, kStore).
+// B = H MN-major, kStore).  A GEMM without units (nNt = 0) is left out.
 template <int EPI0, bool MC>
 __global__ void __launch_bounds__(kThreads, 1)
     cis_lmhead_dual_kernel(const __grid_constant__ CUtensorMap tmA0,
                            const __grid_constant__ CUtensorMap tmB0,
                            const __grid_constant__ CUtensorMap tmA1,
-                           const __grid_constant__ CUtensorMap tmB1, const GemmArgs g0,
-                           const GemmArgs g1, const __grid_constant__ DualSched sc)
+                           const __grid_constant__ CUtensorMap tmB1, const GemmArgs args0,
+                           const GemmArgs args1)
 {
     extern __shared__ __align__(1024) uint8_t dsm[];
     uint8_t *ring = dsm + ((1024 - (tc::smem_addr(dsm) & 1023)) & 1023);
     __shared__ __align__(8) GemmShared sh;
 
+    const GemmArgs g0 = live_args(args0), g1 = live_args(args1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = MC ? (int)tc::cluster_ctarank() : 0;
-    const int grp = MC ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-    const int j0 = sc.off[grp], j1 = sc.off[grp + 1];
+    const DualList list = dual_list<MC>(g0, g1, MC ? (int)(blockIdx.x >> 1) : (int)blockIdx.x,
+                                        MC ? (int)(gridDim.x >> 1) : (int)gridDim.x);
+    const int items = list.size();
 
     gemm_setup<MC>(sh, warp);
     const uint32_t tmem = sh.tmem_base;
@@ -687,134 +766,286 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {  // producer
             Ring p;
             uint32_t used = 0, last = 0;
-            for (int j = j0; j < j1 && !ab.on(); ++j) {
-                const int u = sc.unit[j];
-                int m, n;
-                if (u & kSchedSecond) {
-                    unit_mn<MC>(g1, u & ~kSchedSecond, rank, m, n);
-                    load_tile<true, true, MC>(tmA1, tmB1, g1, m, n, rank, ring, sh.bars, ab, p,
-                                              used, last);
-                } else {
-                    unit_mn<MC>(g0, u, rank, m, n);
-                    load_tile<false, true, MC>(tmA0, tmB0, g0, m, n, rank, ring, sh.bars, ab, p,
-                                               used, last);
-                }
+            for (int i = 0; i < items && !ab.on(); ++i) {
+                int u;
+                if (list.item(i, u))
+                    load_tile<false, true, MC>(tmA0, tmB0, g0, unit_at<MC>(g0, u, rank), rank,
+                                               ring, sh.bars, ab, p, used, last);
+                else
+                    load_tile<true, true, MC>(tmA1, tmB1, g1, unit_at<MC>(g1, u, rank), rank,
+                                              ring, sh.bars, ab, p, used, last);
             }
             drain_loads(sh.bars, used, last);
         }
     } else if (warp == 1) {
         if (lane == 0) {  // MMA issue
             Ring p;
-            for (int j = j0; j < j1 && !ab.on(); ++j) {
-                if (sc.unit[j] & kSchedSecond)
-                    mma_unit<true, true, MC>(g1, j - j0, tmem, ring, sh.bars, ab, p);
+            for (int i = 0; i < items && !ab.on(); ++i) {
+                int u;
+                if (list.item(i, u))
+                    mma_unit<false, true, MC>(unit_at<MC>(g0, u, rank).nk, i, tmem, ring,
+                                              sh.bars, ab, p);
                 else
-                    mma_unit<false, true, MC>(g0, j - j0, tmem, ring, sh.bars, ab, p);
+                    mma_unit<true, true, MC>(g1.nK, i, tmem, ring, sh.bars, ab, p);
             }
             drain_mmas(sh.bars);
         }
     } else {  // epilogue
-        for (int j = j0; j < j1; ++j) {
+        for (int i = 0; i < items; ++i) {
             if (__syncthreads_or_epi(ab.on()))
                 break;
-            const int u = sc.unit[j];
-            int m, n;
-            if (u & kSchedSecond) {
-                unit_mn<MC>(g1, u & ~kSchedSecond, rank, m, n);
-                epilogue_unit<kStore, MC>(g1, m, n, j - j0, tmem, warp, lane, sh.bars, ab);
-            } else {
-                unit_mn<MC>(g0, u, rank, m, n);
-                epilogue_unit<EPI0, MC>(g0, m, n, j - j0, tmem, warp, lane, sh.bars, ab);
-            }
+            int u;
+            if (list.item(i, u))
+                epilogue_unit<EPI0, MC>(g0, unit_at<MC>(g0, u, rank), i, tmem, warp, lane,
+                                        sh.bars, ab);
+            else
+                epilogue_unit<kStore, MC>(g1, unit_at<MC>(g1, u, rank), i, tmem, warp, lane,
+                                          sh.bars, ab);
         }
     }
     gemm_teardown<MC>(sh, warp);
 }
 
-// dst[i] = bf16(src[i]) (round to nearest even)
-__global__ void cis_lmhead_to_bf16_kernel(const float *src, uint16_t *dst, int64_t n)
+// Masked tokens (the prompts and the padding of a batch) have no gradient, so
+// the products are formed over the valid ones only: their hidden states are
+// copied together, in token order, and every GEMM's tiles and K blocks are
+// counted from their number, which stays on the device.  At T=16384, H=2048,
+// V=151936 with 40% masked the call takes 15.8 ms against 25.0 for
+// multiplying the masked rows as well; the copy and the scan take 33 us.
+// Batches of one row tile have nothing to gain and are multiplied as they are.
+//
+// One CTA: pos[t] = the place of token t among the valid ones (-1: masked),
+// their ids in that order, and their number.
+constexpr int kCompactThreads = 1024;
+__global__ void __launch_bounds__(kCompactThreads)
+    cis_lmhead_compact_kernel(const uint8_t *mask, int T, const int32_t *ids, int *pos,
+                              int32_t *ids_c, int *count)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = __bfloat16_as_ushort(__float2bfloat16_rn(src[i]));
+    __shared__ int wsum[kCompactThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    // warp w takes `per` groups of 32 tokens from group w per on
+    const int groups = (T + 31) / 32;
+    const int per = (groups + kCompactThreads / 32 - 1) / (kCompactThreads / 32);
+    const int g0 = wid * per < groups ? wid * per : groups;
+    const int g1 = groups - g0 < per ? groups : g0 + per;
+    auto valid = [&](int grp) {
+        const int t = grp * 32 + lane;
+        return t < T && mask[t] != 0;
+    };
+    int n = 0;
+#pragma unroll 8
+    for (int grp = g0; grp < g1; ++grp)
+        n += valid(grp);
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0)
+        wsum[wid] = n;
+    __syncthreads();
+    int at = 0;
+    for (int w = 0; w < wid; ++w)
+        at += wsum[w];
+#pragma unroll 8
+    for (int grp = g0; grp < g1; ++grp) {
+        const int t = grp * 32 + lane;
+        const int32_t y = t < T ? ids[t] : 0;
+        const bool on = valid(grp);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        const int p = at + __popc(m & ((1u << lane) - 1));
+        if (t < T)
+            pos[t] = on ? p : -1;
+        if (on)
+            ids_c[p] = y;
+        at += __popc(m);
+    }
+    if (tid == kCompactThreads - 1)
+        *count = at;
 }
 
-// Per token: combine the FWD pairs, then log p, weight, loss, c_t (one warp).
-__global__ void cis_lmhead_token_kernel(const PassArgs a, const float2 *part, const float *part_u,
-                                        const float *zy, int nVt, float *lse_out, float *c_out)
+// The valid tokens' rows of src to their places in dst, one warp per token;
+// the rows after the last, up to the end of its row tile, are zeroed (dW's
+// last K block reads them against dz's zeros).
+__global__ void cis_lmhead_gather_kernel(const uint4 *src, const uint8_t *mask, const int *pos,
+                                         const int *count, int T, int row16, uint4 *dst)
 {
-    const int64_t t = blockIdx.x * (int64_t)(blockDim.x / 32) + (threadIdx.x >> 5);
+    const int r = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
     const int lane = threadIdx.x & 31;
-    if (t >= a.T)
+    if (r >= T)
         return;
-    const bool valid = a.mask == nullptr || a.mask[t] != 0;
-    const int64_t y = a.ids[t];
-    const bool id_ok = y >= 0 && y < a.V;
-    if (!valid || !id_ok) {
-        if (lane == 0) {
-            if (valid)
-                set_status(a.status, kStatusBadId);
-            const float lp = valid ? NAN : 0.0f;
-            if (a.lp_out) a.lp_out[t] = lp;
-            if (a.w_out) a.w_out[t] = 0.0f;
-            if (a.trunc_out) a.trunc_out[t] = 0;
-            a.ws_w[t] = 0.0f;
-            a.ws_trunc[t] = 0;
-            a.ws_logk[t] = 0.0f;
-            a.ws_terms[t] = valid ? (double)NAN : 0.0;
-            if (a.entropy_out) a.entropy_out[t] = lp;
-            lse_out[t] = 0.0f;
-            c_out[t] = 0.0f;
-        }
+    const int n = *count;
+    if (mask[r]) {
+        const uint4 *in = src + (int64_t)r * row16;
+        uint4 *out = dst + (int64_t)pos[r] * row16;
+        for (int c = lane; c < row16; c += 32)
+            out[c] = __ldcs(in + c);
+    }
+    if (r >= n && r < (n > 0 ? (n + kBM - 1) / kBM : 1) * kBM)
+        for (int c = lane; c < row16; c += 32)
+            dst[(int64_t)r * row16 + c] = make_uint4(0, 0, 0, 0);
+}
+
+// dhidden from the products' fp32 rows (splits of them, `stride` elements
+// apart, added in order), row r to row rowmap[r]; the masked tokens' rows are
+// zeroed.  parts null: only those.  A CTA takes kFinishCols columns of 8 rows.
+constexpr int kFinishCols = 256;
+__global__ void __launch_bounds__(256)
+    cis_lmhead_finish_kernel(const float *parts, int splits, int64_t stride, const int *rowmap,
+                             const int *count, const uint8_t *mask, int T, int H, void *out,
+                             int out_bf16)
+{
+    const int r = (int)(blockIdx.x * 8 + (threadIdx.x >> 5));
+    if (r >= T)
         return;
-    }
-    MaxSum o{-INFINITY, 0.0f};
-    MaxSumU ou{-INFINITY, 0.0f, 0.0f};
-    if (part_u) {
-        for (int j = lane; j < nVt; j += 32) {
-            const float2 q = part[(int64_t)j * a.T + t];
-            ou = msu_combine(ou, MaxSumU{q.x, q.y, part_u[(int64_t)j * a.T + t]});
+    const int c0 = (int)blockIdx.y * kFinishCols + 4 * (threadIdx.x & 31);
+    auto store = [&](int64_t row, int c, float4 v) {
+        const int64_t o = row * H + c;
+        if (out_bf16)
+            __stcs(reinterpret_cast<uint2 *>(static_cast<uint16_t *>(out) + o),
+                   make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w)));
+        else
+            __stcs(reinterpret_cast<float4 *>(static_cast<float *>(out) + o), v);
+    };
+    if (parts && r < (count ? *count : T)) {
+        const int64_t row = count ? rowmap[r] : r;
+#pragma unroll
+        for (int c = c0; c < c0 + kFinishCols; c += 128) {
+            const float *p = parts + (int64_t)r * H + c;
+            float4 v = __ldcs(reinterpret_cast<const float4 *>(p));
+#pragma unroll 4
+            for (int k = 1; k < splits; ++k) {
+                const float4 w = __ldcs(reinterpret_cast<const float4 *>(p + k * stride));
+                v.x += w.x;
+                v.y += w.y;
+                v.z += w.z;
+                v.w += w.w;
+            }
+            store(row, c, v);
         }
-        ou = warp_msu(ou);
-        o = MaxSum{ou.m, ou.s};
-    } else {
-        for (int j = lane; j < nVt; j += 32) {
-            const float2 q = part[(int64_t)j * a.T + t];
-            o = ms_combine(o, MaxSum{q.x, q.y});
-        }
-        o = warp_ms(o);
     }
-    if (lane == 0) {
-        const RowScalars rs = row_scalars(o, zy[t]);
-        if (part_u && a.entropy_out)
-            a.entropy_out[t] = row_entropy(ou, zy[t], rs.lp);
-        if (is_seq_mode(a.P.mode) && a.w_in == nullptr) {
-            // sequence operator, first sweep: log p only (the response's
-            // weight needs every token of the response)
-            if (a.lp64_out)
-                a.lp64_out[t] = rs.lp64();
+    if (count && mask[r] == 0)
+        for (int c = c0; c < c0 + kFinishCols; c += 128)
+            store(r, c, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+}
+
+// Per token: combine the FWD pairs, then log p, weight, loss, c_t.  A CTA takes
+// 8 tokens: lanes l, l + 8, ... of a warp hold the same token, so a warp's load
+// of one half tile's pairs covers whole sectors (one warp per token, each lane
+// a half tile of its own, read a sector per pair: 23 us at T=512, V=151936,
+// now 10).
+//
+// With masked tokens (pos): the pairs and zy lie at the token's place among
+// the valid ones, and so do lse and c; afterwards zy holds the token's index
+// (the row map of the later GEMMs).  pos shares its memory with a.ws_logk: each
+// token's place is read before its log k is written, by the same CTA.
+constexpr int kTokCta = 8;
+constexpr int kTokThreads = 256;
+__global__ void __launch_bounds__(kTokThreads)
+    cis_lmhead_token_kernel(const PassArgs a, const float2 *part, const float *part_u, float *zy,
+                            int nHalf, float *lse_out, float *c_out, const int *pos)
+{
+    constexpr int kGroups = kTokThreads / kTokCta;
+    __shared__ MaxSumU red[kTokThreads / 32][kTokCta];
+    const int tid = threadIdx.x, ti = tid & (kTokCta - 1), lane = tid & 31, wid = tid >> 5;
+    const int64_t t = blockIdx.x * (int64_t)kTokCta + ti;
+    const bool in = t < a.T;
+    const bool valid = in && (a.mask == nullptr || a.mask[t] != 0);
+    const int64_t y = in ? a.ids[t] : -1;
+    const bool live = valid && y >= 0 && y < a.V;
+    // the token's place; -1: none (past the end, or masked and left out)
+    const int64_t at = !in ? -1 : (pos == nullptr ? t : (valid ? pos[t] : -1));
+    MaxSumU o{-INFINITY, 0.0f, 0.0f};
+    if (live) {
+        constexpr int kU = 8;  // loads in flight
+        for (int j0 = tid / kTokCta; j0 < nHalf; j0 += kU * kGroups) {
+            float2 q[kU];
+            float u[kU];
+#pragma unroll
+            for (int k = 0; k < kU; ++k) {
+                const int j = j0 + k * kGroups;
+                q[k] = j < nHalf ? part[(int64_t)j * a.T + at] : make_float2(-INFINITY, 0.0f);
+                u[k] = part_u && j < nHalf ? part_u[(int64_t)j * a.T + at] : 0.0f;
+            }
+#pragma unroll
+            for (int k = 0; k < kU; ++k) {
+                if (part_u) {
+                    o = msu_combine(o, MaxSumU{q[k].x, q[k].y, u[k]});
+                } else {
+                    const MaxSum ms = ms_combine(MaxSum{o.m, o.s}, MaxSum{q[k].x, q[k].y});
+                    o.m = ms.m;
+                    o.s = ms.s;
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int d = kTokCta; d < 32; d <<= 1) {
+        MaxSumU w;
+        w.m = __shfl_xor_sync(0xffffffffu, o.m, d);
+        w.s = __shfl_xor_sync(0xffffffffu, o.s, d);
+        w.u = __shfl_xor_sync(0xffffffffu, o.u, d);
+        o = msu_combine(o, w);
+    }
+    if (lane < kTokCta)
+        red[wid][lane] = o;
+    __syncthreads();
+    if (tid >= kTokCta || !in)
+        return;
+    // a sequence operator's first sweep: log p only (the response's weight
+    // needs every token of the response)
+    const bool first = is_seq_mode(a.P.mode) && a.w_in == nullptr;
+    auto place = [&](float lse, float c) {
+        if (at < 0)
             return;
-        }
-        const bool has_old = a.lp_old != nullptr;
-        const float lold = has_old ? a.lp_old[t] : 0.0f;
-        TokenWeight tw = token_weight(has_old ? lold : rs.lp, has_old ? 0.0f : rs.lp_lo,
-                                      a.lp_inf[t], a.P, has_old ? -1.0f : rs.omp);
-        if (a.w_in) {
-            tw.w = a.w_in[t];
-            tw.trunc = a.trunc_in[t];
-        }
-        const TokenLoss tl =
-            token_loss(rs.lp, rs.lp_lo, has_old, lold, a.adv[t], a.scale[t], tw.w, a.P);
-        if (a.lp_out) a.lp_out[t] = rs.lp;
-        if (a.w_out) a.w_out[t] = tw.w;
-        if (a.trunc_out) a.trunc_out[t] = tw.trunc;
-        a.ws_w[t] = tw.w;
-        a.ws_trunc[t] = tw.trunc;
-        a.ws_logk[t] = tw.logk;
-        a.ws_terms[t] = tl.term;
-        lse_out[t] = rs.lse;
-        c_out[t] = tl.c;
+        lse_out[at] = lse;
+        c_out[at] = c;
+        if (pos)
+            zy[at] = __int_as_float((int)t);
+    };
+    if (!live) {
+        if (first)
+            return;
+        if (valid)
+            set_status(a.status, kStatusBadId);
+        const float lp = valid ? NAN : 0.0f;
+        if (a.lp_out) a.lp_out[t] = lp;
+        if (a.w_out) a.w_out[t] = 0.0f;
+        if (a.trunc_out) a.trunc_out[t] = 0;
+        a.ws_w[t] = 0.0f;
+        a.ws_trunc[t] = 0;
+        a.ws_logk[t] = 0.0f;
+        a.ws_terms[t] = valid ? (double)NAN : 0.0;
+        if (a.entropy_out) a.entropy_out[t] = lp;
+        place(0.0f, 0.0f);
+        return;
     }
+#pragma unroll
+    for (int w = 1; w < kTokThreads / 32; ++w)
+        o = msu_combine(o, red[w][ti]);
+    const float z = zy[at];
+    const RowScalars rs = row_scalars(MaxSum{o.m, o.s}, z);
+    if (part_u && a.entropy_out)
+        a.entropy_out[t] = row_entropy(o, z, rs.lp);
+    if (first) {
+        if (a.lp64_out)
+            a.lp64_out[t] = rs.lp64();
+        return;
+    }
+    const bool has_old = a.lp_old != nullptr;
+    const float lold = has_old ? a.lp_old[t] : 0.0f;
+    TokenWeight tw = token_weight(has_old ? lold : rs.lp, has_old ? 0.0f : rs.lp_lo, a.lp_inf[t],
+                                  a.P, has_old ? -1.0f : rs.omp);
+    if (a.w_in) {
+        tw.w = a.w_in[t];
+        tw.trunc = a.trunc_in[t];
+    }
+    const TokenLoss tl =
+        token_loss(rs.lp, rs.lp_lo, has_old, lold, a.adv[t], a.scale[t], tw.w, a.P);
+    if (a.lp_out) a.lp_out[t] = rs.lp;
+    if (a.w_out) a.w_out[t] = tw.w;
+    if (a.trunc_out) a.trunc_out[t] = tw.trunc;
+    a.ws_w[t] = tw.w;
+    a.ws_trunc[t] = tw.trunc;
+    a.ws_logk[t] = tw.logk;
+    a.ws_terms[t] = tl.term;
+    place(rs.lse, tl.c);
 }
 
 // ------------------------------------------------------------------ host side
@@ -851,76 +1082,18 @@ bool make_map(CUtensorMap *m, const void *ptr, int64_t inner, int64_t outer, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int EPI, bool A_MN = false, bool B_MN = false>
-cudaError_t launch_gemm(const CUtensorMap &a, const CUtensorMap &b, const GemmArgs &g,
-                        cudaStream_t s)
-{
-    const int tiles = g.nMt * g.nNt;
-    if (tiles <= 0 || g.nK <= 0)
-        return cudaSuccess;
-    auto k = cis_lmhead_gemm_kernel<EPI, A_MN, B_MN, false>;
-    const size_t smem = kSmemBytes;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess)
-        return e;
-    int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-        return e;
-    const int grid = tiles < sms ? tiles : sms;
-    k<<<grid, kThreads, smem, s>>>(a, b, g);
-    return cudaGetLastError();
-}
-
-// The same GEMM on 2-CTA clusters that share each B tile (multicast).  `b`
-// must be a map whose box is half of B's tile: 128 rows for a K-major B, the
-// 64-wide boxes of an MN-major one.
-template <int EPI, bool A_MN = false, bool B_MN = false>
-cudaError_t launch_gemm_mc(const CUtensorMap &a, const CUtensorMap &b, const GemmArgs &g,
-                           cudaStream_t s)
-{
-    const int units = ((g.nMt + 1) / 2) * g.nNt;
-    if (units <= 0 || g.nK <= 0)
-        return cudaSuccess;
-    auto k = cis_lmhead_gemm_kernel<EPI, A_MN, B_MN, true>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBytes);
-    if (e != cudaSuccess)
-        return e;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3(2);
-    int clusters = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters, k, &cfg)) != cudaSuccess)
-        return e;
-    if (clusters <= 0)
-        return cudaErrorNotSupported;
-    cfg.gridDim = dim3((unsigned)(2 * (units < clusters ? units : clusters)));
-    e = cudaLaunchKernelEx(&cfg, k, a, b, g);
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 // The groups that run at once: co-resident 2-CTA clusters (MC), else SMs.
 template <typename K> cudaError_t resident_groups(K kern, bool mc, int *groups)
 {
-    int dev = 0, sms = 0;
-    cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSmemBytes);
+    if (e != cudaSuccess)
         return e;
     if (!mc) {
-        *groups = sms;
-        return cudaSuccess;
+        int dev = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess)
+            return e;
+        return cudaDeviceGetAttribute(groups, cudaDevAttrMultiProcessorCount, dev);
     }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -938,98 +1111,68 @@ template <typename K> cudaError_t resident_groups(K kern, bool mc, int *groups)
     return *groups > 0 ? cudaSuccess : cudaErrorNotSupported;
 }
 
-// The greedy schedule of a dual launch: units n0 of GEMM 0 (c0 K blocks
-// each), then n1 of GEMM 1 (c1 each), each to the group whose list ends
-// earliest (ties: the lowest group).  The units of one GEMM go out in order,
-// so the groups at work at any time hold neighbouring units, which share their
-// operands in L2.  False if it does not fit a DualSched.
-static bool make_dual_sched(int n0, int c0, int n1, int c1, int groups, DualSched *s)
+// A persistent launch: one group (a cluster, or a CTA) per resident place, or
+// per unit where there are fewer.
+template <bool MC, typename K, typename... Args>
+cudaError_t launch_groups(K kern, int64_t units, cudaStream_t s, const Args &...args)
 {
-    if (groups < 1 || groups > kMaxSchedGroups || n0 + n1 > kMaxSchedUnits || n0 < 0 ||
-        n1 < 0 || n0 >= kSchedSecond || n1 >= kSchedSecond)
-        return false;
-    std::vector<int64_t> end(groups, 0);
-    std::vector<std::vector<uint16_t>> lists(groups);
-    for (int j = 0; j < n0 + n1; ++j) {
-        int best = 0;
-        for (int c = 1; c < groups; ++c)
-            if (end[c] < end[best])
-                best = c;
-        const bool second = j >= n0;
-        end[best] += second ? c1 : c0;
-        lists[best].push_back(second ? (uint16_t)((j - n0) | kSchedSecond) : (uint16_t)j);
-    }
-    int k = 0;
-    for (int c = 0; c < groups; ++c) {
-        s->off[c] = (uint16_t)k;
-        for (uint16_t u : lists[c])
-            s->unit[k++] = u;
-    }
-    for (int c = groups; c <= kMaxSchedGroups; ++c)
-        s->off[c] = (uint16_t)k;
-    return true;
-}
-
-// One launch of cis_lmhead_dual_kernel over both GEMMs' units; false (and no
-// launch) if the schedule does not fit, so that the caller launches them one
-// after the other.  Schedules are kept per shape: a call makes two (full
-// chunks, the last chunk).
-template <int EPI0, bool MC>
-cudaError_t launch_dual(const CUtensorMap &a0, const CUtensorMap &b0, const GemmArgs &g0,
-                        const CUtensorMap &a1, const CUtensorMap &b1, const GemmArgs &g1,
-                        cudaStream_t s, bool *launched)
-{
-    *launched = false;
-    auto k = cis_lmhead_dual_kernel<EPI0, MC>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBytes);
+    int groups = 0;
+    cudaError_t e = resident_groups(kern, MC, &groups);
     if (e != cudaSuccess)
         return e;
-    int groups = 0;
-    if ((e = resident_groups(k, MC, &groups)) != cudaSuccess)
-        return e;
-    const int n0 = MC ? n_units<true>(g0) : n_units<false>(g0);
-    const int n1 = MC ? n_units<true>(g1) : n_units<false>(g1);
-    if (g0.nK <= 0 || g1.nK <= 0 || n0 <= 0 || n1 <= 0)
+    if (units <= 0)
         return cudaSuccess;
-    static std::mutex mu;
-    static std::map<std::array<int, 5>, std::unique_ptr<DualSched>> cache;
-    std::unique_ptr<DualSched> sc(new DualSched());  // this call's copy
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        const std::array<int, 5> key = {n0, g0.nK, n1, g1.nK, groups};
-        auto it = cache.find(key);
-        if (it == cache.end()) {
-            std::unique_ptr<DualSched> p(new DualSched());
-            if (!make_dual_sched(n0, g0.nK, n1, g1.nK, groups, p.get()))
-                return cudaSuccess;
-            if (cache.size() >= 64)  // a process that sees many shapes keeps the last few
-                cache.clear();
-            it = cache.emplace(key, std::move(p)).first;
-        }
-        *sc = *it->second;
-    }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = MC ? 2 : 1;
+    attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(groups * (MC ? 2 : 1)));
+    cfg.gridDim = dim3((unsigned)((units < groups ? units : groups) * (MC ? 2 : 1)));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = MC ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, k, a0, b0, a1, b1, g0, g1, *sc);
-    if (e == cudaSuccess)
-        e = cudaGetLastError();
-    *launched = e == cudaSuccess;
-    return e;
+    e = cudaLaunchKernelEx(&cfg, kern, args...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// Units of a GEMM by the host's counts (the device's token count may lower
+// them).
+template <bool MC> int64_t host_units(const GemmArgs &g)
+{
+    return (int64_t)(MC ? (g.nMt + 1) / 2 : g.nMt) * g.nNt * g.splits;
+}
+
+// FWD and DZ.  With MC `b` must be a map whose box is half of B's tile.
+template <int EPI, bool MC>
+cudaError_t launch_gemm(const CUtensorMap &a, const CUtensorMap &b, const GemmArgs &g,
+                        cudaStream_t s)
+{
+    return launch_groups<MC>(cis_lmhead_gemm_kernel<EPI, MC>, host_units<MC>(g), s, a, b, g);
+}
+
+// dH and dW of a chunk in one launch.
+template <int EPI0, bool MC>
+cudaError_t launch_dual(const CUtensorMap &a0, const CUtensorMap &b0, const GemmArgs &g0,
+                        const CUtensorMap &a1, const CUtensorMap &b1, const GemmArgs &g1,
+                        cudaStream_t s)
+{
+    return launch_groups<MC>(cis_lmhead_dual_kernel<EPI0, MC>,
+                             host_units<MC>(g0) + host_units<MC>(g1), s, a0, b0, a1, b1, g0, g1);
+}
+template <bool MC>
+cudaError_t launch_dual(bool first, const CUtensorMap &a0, const CUtensorMap &b0,
+                        const GemmArgs &g0, const CUtensorMap &a1, const CUtensorMap &b1,
+                        const GemmArgs &g1, cudaStream_t s)
+{
+    return first ? launch_dual<kStore, MC>(a0, b0, g0, a1, b1, g1, s)
+                 : launch_dual<kAccum, MC>(a0, b0, g0, a1, b1, g1, s);
 }
 
 // Whether a chunk's dH and dW run as one launch (CIS_LMHEAD_DUAL=0: one after
-// the other; the results are the same either way).
+// the other, each with the other left out; the results are the same either way).
 static bool dual_on()
 {
     const char *e = getenv("CIS_LMHEAD_DUAL");
@@ -1113,6 +1256,56 @@ static int64_t chunk_for_bytes(int64_t T, int64_t V, int64_t Hd, size_t bytes)
     return c >= lm::kBN ? c : 0;
 }
 
+// dH has few, long units: (T / 256)(H / 256) pairs of tiles contracting the
+// whole chunk, so that with few tokens most SMs would wait for it (T=512,
+// H=2048, V=151936: 16 units of 2374 K blocks against dW's 4752 of 8, on 76
+// clusters).  Its contraction is then cut into ranges of at most half a
+// cluster's share of the launch, each with fp32 products of its own, added at
+// the end in order.  The products take the room of a narrower chunk's dz, or
+// what the caller's workspace has beyond the layout.  T=512, H=2048, V=151936:
+// dH and dW take 552 us (two chunks) against 1123 one after the other, the call
+// 1096 against 1600; ranges of a share took 578, of a third 626, of a sixth
+// 577.  T=300, H=1024, V=32003: 68 against 212.
+constexpr int64_t kSplitSms = 152;  // the split follows the shape alone
+constexpr int kMaxSplits = 16;
+struct Split {
+    int64_t Vc;
+    int splits;
+    size_t parts;  // offset of the products
+};
+static int split_count(int64_t T, int64_t w, int64_t Hd)
+{
+    const int64_t nH = Hd / lm::kBN, nM = (T + lm::kBM - 1) / lm::kBM;
+    const int64_t nV = (w + lm::kBM - 1) / lm::kBM;
+    const bool pairs = nM > 1;
+    const int64_t G = pairs ? kSplitSms / 2 : kSplitSms;
+    const int64_t n0 = (pairs ? (nM + 1) / 2 : nM) * nH, c0 = (w + lm::kBK - 1) / lm::kBK;
+    const int64_t n1 = (pairs ? (nV + 1) / 2 : nV) * nH, c1 = std::max<int64_t>((T + lm::kBK - 1) / lm::kBK, lm::kDwBlocks);
+    const int64_t share = (n0 * c0 + n1 * c1) / G;
+    int64_t S = (2 * c0 + share - 1) / share;
+    S = S < c0 / 16 ? S : c0 / 16;
+    S = S < kMaxSplits ? S : kMaxSplits;
+    return S > 1 ? (int)S : 1;
+}
+// The chunk and the split for a workspace that holds chunks of `widest` columns.
+static Split split_for(int64_t T, int64_t V, int64_t Hd, int64_t widest, size_t bytes)
+{
+    if (T <= 0 || split_count(T, widest < V ? widest : V, Hd) == 1)
+        return {widest, 1, 0};
+    for (int64_t chunks = 1; chunks <= 4; ++chunks) {
+        const int64_t Vc = round_up((V + chunks - 1) / chunks, lm::kBN);
+        const size_t base = lm_layout(T, V, Hd, Vc).total;
+        if (Vc > widest || base > bytes)
+            continue;
+        const int64_t want = split_count(T, Vc < V ? Vc : V, Hd);
+        const int64_t fit = (int64_t)((bytes - base) / (4 * (size_t)T * (size_t)Hd));
+        const int64_t S = want < fit ? want : fit;
+        if (S > 1 && 2 * S >= want)
+            return {Vc, (int)S, base};
+    }
+    return {widest, 1, 0};
+}
+
 }  // namespace cis
 
 using namespace cis;
@@ -1161,9 +1354,11 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
         return CIS_ERR_UNSUPPORTED;  // Hd in blocks of 256 (and so of the 64-wide K blocks)
     if (workspace == nullptr || (reinterpret_cast<uintptr_t>(workspace) & 1023))
         return CIS_ERR_INVALID_ARG;
-    const int64_t Vc = chunk_for_bytes(T, V, H, workspace_bytes);
-    if (Vc == 0)
+    const int64_t widest = chunk_for_bytes(T, V, H, workspace_bytes);
+    if (widest == 0)
         return CIS_ERR_INVALID_ARG;  // smaller than the layout for 256-column chunks
+    const Split sp = split_for(T, V, H, widest, workspace_bytes);
+    const int64_t Vc = sp.Vc;
     const LmLayout L = lm_layout(T, V, H, Vc);
     if (T > 0 && (hidden == nullptr || weight == nullptr || ids == nullptr ||
                   lp_infer == nullptr || adv == nullptr || dhidden == nullptr ||
@@ -1200,9 +1395,6 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
     float2 *part = reinterpret_cast<float2 *>(ws + L.part);
     float *part_u = entropy_out ? reinterpret_cast<float *>(ws + L.part_u) : nullptr;
     uint16_t *dz = reinterpret_cast<uint16_t *>(ws + L.dz);
-    float *dh_acc = grad_dtype == CIS_F32 ? static_cast<float *>(dhidden)
-                                          : reinterpret_cast<float *>(ws + L.dh);
-
     float *scale = reinterpret_cast<float *>(ws + L.base.scale);
     a.red_parts = ws + L.base.parts;
     a.red_ticket = reinterpret_cast<uint32_t *>(ws + L.base.ticket);
@@ -1214,21 +1406,55 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
         const int nTt = (int)((T + lm::kBM - 1) / lm::kBM);
         const int nVt = (int)((V + lm::kBN - 1) / lm::kBN);
         const int nHt = (int)(H / lm::kBN);
+        const bool bf16 = grad_dtype == CIS_BF16;
+        // one row tile has no partner to share B with
+        const int mc = nTt == 1 ? 0 : lm::mc_mask();
+        // Masked tokens are left out of the products where there is more than
+        // one row tile to save.  What that needs lives in memory that is free
+        // until the token step, each token's entry where the step itself writes
+        // that token's value: the places in ws_logk, the ids in lse, afterwards
+        // the row map in zy.  The valid tokens' hidden states take dH's fp32
+        // rows' room, or dhidden's own where those rows are in use.
+        // (A dhidden that shares memory with hidden is written last: not packed.)
+        const uintptr_t h0 = reinterpret_cast<uintptr_t>(hidden), hb = (uintptr_t)(T * H) * 2;
+        const uintptr_t d0 = reinterpret_cast<uintptr_t>(dhidden),
+                        db = (uintptr_t)(T * H) * (bf16 ? 2 : 4);
+        const bool packed = mask != nullptr && nTt > 1 && !(h0 < d0 + db && d0 < h0 + hb);
+        int *count = packed ? reinterpret_cast<int *>(ws + L.base.status + 128) : nullptr;
+        int *pos = packed ? reinterpret_cast<int *>(a.ws_logk) : nullptr;
+        int32_t *ids_c = reinterpret_cast<int32_t *>(lse);
+        const int *rowmap = packed ? reinterpret_cast<const int *>(zy) : nullptr;
+        const bool direct = sp.splits == 1 && !bf16;  // dH's products are dhidden's rows
+        float *dh_rows = direct ? static_cast<float *>(dhidden)
+                                : reinterpret_cast<float *>(ws + (sp.splits > 1 ? sp.parts : L.dh));
+        const void *h = hidden;
+        if (packed) {
+            void *hc = sp.splits == 1 && bf16 ? dhidden : static_cast<void *>(ws + L.dh);
+            lm::cis_lmhead_compact_kernel<<<1, lm::kCompactThreads, 0, s>>>(mask, (int)T, ids, pos,
+                                                                            ids_c, count);
+            if (cudaGetLastError() != cudaSuccess)
+                return CIS_ERR_CUDA;
+            lm::cis_lmhead_gather_kernel<<<(unsigned)((T + 7) / 8), 256, 0, s>>>(
+                static_cast<const uint4 *>(hidden), mask, pos, count, (int)T, (int)(H / 8),
+                static_cast<uint4 *>(hc));
+            if (cudaGetLastError() != cudaSuccess)
+                return CIS_ERR_CUDA;
+            h = hc;
+        }
         // K-major maps of H and W (FWD, DZ) and MN-major ones (boxes of 64
         // rows: W as DH's B operand, H as DW's)
         // (mWh: W in boxes of half a B tile, for the multicast clusters)
-        const int mc = lm::mc_mask();
         CUtensorMap mH, mW, mWh, mWmn, mHmn;
-        if (!lm::make_map(&mH, hidden, H, T, H, lm::kBM) ||
+        if (!lm::make_map(&mH, h, H, T, H, lm::kBM) ||
             !lm::make_map(&mW, weight, H, V, H, lm::kBN) ||
             !lm::make_map(&mWh, weight, H, V, H, lm::kBN / 2) ||
             !lm::make_map(&mWmn, weight, H, V, H, 64) ||
-            !lm::make_map(&mHmn, hidden, H, T, H, 64))
+            !lm::make_map(&mHmn, h, H, T, H, 64))
             return CIS_ERR_UNSUPPORTED;
         lm::GemmArgs g = {};
         g.T = (int)T;
         g.V = (int)V;
-        g.ids = ids;
+        g.ids = packed ? ids_c : ids;
         g.lse = lse;
         g.cvec = cv;
         g.part = part;
@@ -1236,16 +1462,21 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
         g.zy = zy;
         g.dz = dz;
         g.ld_dz = Vc;
+        g.rows_valid = (int)T;
+        g.count = count;
         g.status = a.status;
         // FWD: z tiles of H W^T, row statistics
         g.nMt = nTt;
         g.nNt = nVt;
         g.nK = (int)(H / lm::kBK);
+        g.splits = 1;
+        g.ksplit = g.nK;
         g.raster_n = 1;
-        if (((mc & 1) ? lm::launch_gemm_mc<lm::kStats>(mH, mWh, g, s)
-                      : lm::launch_gemm<lm::kStats>(mH, mW, g, s)) != cudaSuccess)
+        if (((mc & 1) ? lm::launch_gemm<lm::kStats, true>(mH, mWh, g, s)
+                      : lm::launch_gemm<lm::kStats, false>(mH, mW, g, s)) != cudaSuccess)
             return CIS_ERR_CUDA;
         // per-token scalars
+        const unsigned tok_grid = (unsigned)((T + lm::kTokCta - 1) / lm::kTokCta);
         if (is_seq_mode(P.mode)) {
             // sequence operator: log p of every token (fp64, into the terms
             // array, which the second sweep then overwrites), the responses'
@@ -1253,8 +1484,8 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
             if (lp_old == nullptr) {
                 PassArgs f = a;
                 f.lp64_out = a.ws_terms;
-                lm::cis_lmhead_token_kernel<<<(unsigned)((T + 7) / 8), 256, 0, s>>>(
-                    f, part, part_u, zy, 2 * nVt, lse, cv);
+                lm::cis_lmhead_token_kernel<<<tok_grid, lm::kTokThreads, 0, s>>>(
+                    f, part, part_u, zy, 2 * nVt, lse, cv, pos);
                 if ((e = cudaGetLastError()) != cudaSuccess)
                     return CIS_ERR_CUDA;
             }
@@ -1267,24 +1498,21 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
             a.w_in = a.ws_w;
             a.trunc_in = a.ws_trunc;
         }
-        lm::cis_lmhead_token_kernel<<<(unsigned)((T + 7) / 8), 256, 0, s>>>(a, part, part_u, zy,
-                                                                            2 * nVt, lse, cv);
+        lm::cis_lmhead_token_kernel<<<tok_grid, lm::kTokThreads, 0, s>>>(
+            a, part, part_u, zy, 2 * nVt, lse, cv, pos);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return CIS_ERR_CUDA;
+        g.ids = ids;
+        int splits = sp.splits;
         for (int64_t v0 = 0; v0 < V; v0 += Vc) {
             const int64_t w = V - v0 < Vc ? V - v0 : Vc;
             // DZ: recompute the chunk's z tiles, write dz
-            g.nMt = nTt;
             g.nNt = (int)((w + lm::kBN - 1) / lm::kBN);
-            g.nK = (int)(H / lm::kBK);
-            g.raster_n = 1;
-            g.a_row0 = 0;
-            g.a_k0 = 0;
+            g.rowmap = rowmap;
             g.b_row0 = (int)v0;
-            g.b_k0 = 0;
             g.col0 = (int)v0;
-            if (((mc & 2) ? lm::launch_gemm_mc<lm::kDz>(mH, mWh, g, s)
-                          : lm::launch_gemm<lm::kDz>(mH, mW, g, s)) != cudaSuccess)
+            if (((mc & 2) ? lm::launch_gemm<lm::kDz, true>(mH, mWh, g, s)
+                          : lm::launch_gemm<lm::kDz, false>(mH, mW, g, s)) != cudaSuccess)
                 return CIS_ERR_CUDA;
             // dz K-major (DH's A: rows are tokens) and MN-major (DW's A: its
             // M runs along dz's columns; rows past T read as zeros)
@@ -1293,70 +1521,68 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
                 !lm::make_map(&mDzmn, dz, w, T, Vc, 64))
                 return CIS_ERR_UNSUPPORTED;
             // DH (+)= dz W[chunk]: A = dz [Tp, w] K-major, B = W rows v0 .. v0 + w
-            // MN-major (N along Hd, K along the vocabulary)
+            // MN-major (N along Hd, K along the vocabulary), in `splits` ranges
+            // (as many as the first chunk fills)
             lm::GemmArgs gdh = g;
-            gdh.nMt = nTt;
             gdh.nNt = nHt;
             gdh.nK = (int)((w + lm::kBK - 1) / lm::kBK);
+            gdh.ksplit = (gdh.nK + splits - 1) / splits;
+            gdh.splits = (gdh.nK + gdh.ksplit - 1) / gdh.ksplit;
+            if (v0 == 0)
+                splits = gdh.splits;
+            gdh.split_stride = T * H;
             gdh.raster_n = 0;
-            gdh.a_row0 = 0;
-            gdh.a_k0 = 0;
             gdh.b_row0 = 0;
             gdh.b_k0 = (int)v0;
-            gdh.out = dh_acc;
+            gdh.rowmap = direct ? rowmap : nullptr;
+            gdh.out = dh_rows;
             gdh.out_bf16 = 0;
-            gdh.out_v8 = (reinterpret_cast<uintptr_t>(dh_acc) & 31) == 0;
-            gdh.rows_valid = (int)T;
+            gdh.out_v8 = (reinterpret_cast<uintptr_t>(dh_rows) & 31) == 0;
             gdh.ld_out = H;
             // DW[chunk] = dz^T H: A = dz MN-major (M along the chunk's columns,
             // K along the tokens), B = H MN-major (N along Hd, K along tokens)
-            lm::GemmArgs gdw = gdh;
+            lm::GemmArgs gdw = g;
+            gdw.count_k = 1;
+            gdw.rowmap = nullptr;
             gdw.nMt = (int)((w + lm::kBM - 1) / lm::kBM);
             gdw.nNt = nHt;
             gdw.nK = (int)((T + lm::kBK - 1) / lm::kBK);
+            gdw.ksplit = gdw.nK;
             gdw.raster_n = 0;
-            gdw.b_k0 = 0;
-            gdw.out = static_cast<uint8_t *>(dweight) +
-                      (size_t)v0 * (size_t)H * (grad_dtype == CIS_BF16 ? 2 : 4);
-            gdw.out_bf16 = grad_dtype == CIS_BF16;
+            gdw.b_row0 = 0;
+            gdw.out = static_cast<uint8_t *>(dweight) + (size_t)v0 * (size_t)H * (bf16 ? 2 : 4);
+            gdw.out_bf16 = bf16;
             gdw.out_v8 = (reinterpret_cast<uintptr_t>(gdw.out) & 31) == 0;
             gdw.rows_valid = (int)w;
-            // both in one launch where the schedule fits (and both take the
-            // same CTA grouping), else one after the other
-            bool done = false;
+            gdw.ld_out = H;
+            // both in one launch if both take the same CTA grouping, else each
+            // in one that leaves the other out
             if (lm::dual_on() && ((mc & 12) == 12 || (mc & 12) == 0)) {
-                const bool pair = (mc & 12) == 12;
-                if (v0 == 0)
-                    e = pair ? lm::launch_dual<lm::kStore, true>(mDz, mWmn, gdh, mDzmn, mHmn, gdw,
-                                                                 s, &done)
-                             : lm::launch_dual<lm::kStore, false>(mDz, mWmn, gdh, mDzmn, mHmn,
-                                                                  gdw, s, &done);
-                else
-                    e = pair ? lm::launch_dual<lm::kAccum, true>(mDz, mWmn, gdh, mDzmn, mHmn, gdw,
-                                                                 s, &done)
-                             : lm::launch_dual<lm::kAccum, false>(mDz, mWmn, gdh, mDzmn, mHmn,
-                                                                  gdw, s, &done);
-                if (e != cudaSuccess)
-                    return CIS_ERR_CUDA;
+                e = (mc & 12) ? lm::launch_dual<true>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, gdw, s)
+                              : lm::launch_dual<false>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, gdw,
+                                                       s);
+            } else {
+                lm::GemmArgs no_dh = gdh, no_dw = gdw;
+                no_dh.nNt = no_dw.nNt = 0;
+                e = (mc & 4) ? lm::launch_dual<true>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, no_dw,
+                                                     s)
+                             : lm::launch_dual<false>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, no_dw,
+                                                      s);
+                if (e == cudaSuccess)
+                    e = (mc & 8) ? lm::launch_dual<true>(true, mDz, mWmn, no_dh, mDzmn, mHmn, gdw,
+                                                         s)
+                                 : lm::launch_dual<false>(true, mDz, mWmn, no_dh, mDzmn, mHmn, gdw,
+                                                          s);
             }
-            if (!done) {
-                if (mc & 4)
-                    e = v0 == 0 ? lm::launch_gemm_mc<lm::kStore, false, true>(mDz, mWmn, gdh, s)
-                                : lm::launch_gemm_mc<lm::kAccum, false, true>(mDz, mWmn, gdh, s);
-                else
-                    e = v0 == 0 ? lm::launch_gemm<lm::kStore, false, true>(mDz, mWmn, gdh, s)
-                                : lm::launch_gemm<lm::kAccum, false, true>(mDz, mWmn, gdh, s);
-                if (e != cudaSuccess)
-                    return CIS_ERR_CUDA;
-                if (((mc & 8) ? lm::launch_gemm_mc<lm::kStore, true, true>(mDzmn, mHmn, gdw, s)
-                              : lm::launch_gemm<lm::kStore, true, true>(mDzmn, mHmn, gdw, s)) !=
-                    cudaSuccess)
-                    return CIS_ERR_CUDA;
-            }
+            if (e != cudaSuccess)
+                return CIS_ERR_CUDA;
         }
-        if (grad_dtype == CIS_BF16) {
-            lm::cis_lmhead_to_bf16_kernel<<<1184, 256, 0, s>>>(
-                dh_acc, static_cast<uint16_t *>(dhidden), T * H);
+        if (!direct || packed) {
+            lm::cis_lmhead_finish_kernel<<<dim3((unsigned)((T + 7) / 8),
+                                                (unsigned)(H / lm::kFinishCols)),
+                                           256, 0, s>>>(
+                direct ? nullptr : dh_rows, splits, T * H, rowmap, count, mask, (int)T, (int)H,
+                dhidden, bf16);
             if ((e = cudaGetLastError()) != cudaSuccess)
                 return CIS_ERR_CUDA;
         }
