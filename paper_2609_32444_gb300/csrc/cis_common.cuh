@@ -30,6 +30,9 @@ namespace cis {
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
+// Beyond this magnitude z log2e may overflow fp32, so exponents are formed
+// from z - m (rows of masked entries at the type's lowest value, for one).
+constexpr float kHugeLogit = 1e38f;
 
 // Hyper-parameters as the kernels use them: fp32 copies for the fast path and
 // fp64 values (with logs taken on the host) for the certified fallback.
@@ -181,7 +184,9 @@ struct TokenWeight {
 // for an fp32 input) and log q (linf, inference side).  Algorithm 1:
 // p = exp(lw), k = exp(lw - linf), phi = max(1-p, kappa),
 // w = min{k, 1 + lambda*phi}; Table 8 for the other modes.  omp is 1 - p
-// where the caller already has it (row_scalars), else negative.
+// where the caller already has it (row_scalars), else negative.  kAll false: the
+// band, IcePop and KPop are left out (the caller has none of them).
+template <bool kAll = true>
 __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float linf,
                                                     const DevParams &P, float omp = -1.0f)
 {
@@ -233,70 +238,6 @@ __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float
         r.w = hi ? P.exact_hi_f : (lo ? P.exact_lo_f : expf(logk));
         break;
     }
-    case CIS_MODE_BAND: {
-        // Sec. 4.3: the CIS weight, lifted from below to (1 + p)/2 (the image
-        // of e^eps = 1/2).  Both comparisons as for CIS; k near (1 + p)/2 lies
-        // in [1/2, 1], where its error is smaller still
-        const float om = omp >= 0.0f ? omp : -expm1f(lw);
-        const float k = expf(logk);
-        const float lo = om < 0.5f ? 1.0f - 0.5f * om : 0.5f + 0.5f * expf(lw);
-        const int su = certain_cmp(k, 1.0f + P.lam_f * fmaxf(om, P.kappa_f));
-        const int sl = certain_cmp(lo, k);
-        const bool up =
-            su != 0 ? su > 0 : logk64() > log1p(P.lam * fmax(-expm1(lw64()), P.kappa));
-        const bool low = sl != 0 ? sl > 0 : logk64() < log(0.5 * (1.0 + exp(lw64())));
-        r.trunc = up || low;
-        r.w = k;
-        if (up || low) {  // the bounds themselves, to fp32 rounding
-            float pl, e, ph = exp_pair(lw, lw_lo, pl);
-            const float half = two_sum(0.5f, 0.5f * ph, e);
-            r.w = up ? (float)(1.0 + P.lam * fmax((1.0 - (double)ph) - (double)pl, P.kappa))
-                     : half + fmaf(0.5f, pl, e);
-        }
-        break;
-    }
-    case CIS_MODE_ICEPOP: {
-        // Table 8: k on [lo, hi] (bounds included), else masked
-        const int sl = certain_cmp(P.log_icepop_lo_f, logk);
-        const int sh = certain_cmp(logk, P.log_icepop_hi_f);
-        const bool out = (sl != 0 ? sl > 0 : logk64() < P.log_icepop_lo) ||
-                         (sh != 0 ? sh > 0 : logk64() > P.log_icepop_hi);
-        r.trunc = out;
-        r.w = out ? 0.0f : expf(logk);
-        break;
-    }
-    case CIS_MODE_KPOP: {
-        // Table 8 / App. D.5: binary KL both ways on probabilities clamped to
-        // [1e-8, 1 - 1e-8]; masked when the larger exceeds phi.  fp32 decides
-        // unless the two are close.  With L = log p - log q and M = log(1 - p)
-        // - log(1 - q) of the clamped values, |L|, |M| <= 18.5, the two KLs are
-        // p L + (1 - p) M and -(q L + (1 - q) M); p, 1 - p, q and 1 - q carry
-        // relative errors below 1e-6 and the four logs absolute errors below
-        // 6e-6, so each KL is off by less than 1e-6 (2 * 18.5) + 2 * 1.2e-5 <
-        // 7e-5; 2e-4 is taken.  (The clamps drop a NaN: fp64 keeps it.)
-        const float fl = 1e-8f, ll = -18.420681f;  // the clamp and its log
-        const float om = omp >= 0.0f ? omp : -expm1f(lw), oq = -expm1f(linf);
-        const float a = fminf(fmaxf(lw, ll), -fl), b = fminf(fmaxf(linf, ll), -fl);
-        const float p = expf(a), q = expf(b);
-        const float p1 = fminf(fmaxf(om, fl), 1.0f), q1 = fminf(fmaxf(oq, fl), 1.0f);
-        const float L = a - b, M = logf(p1) - logf(q1);
-        const float kl = fmaxf(p * L + p1 * M, -(q * L + q1 * M));
-        const float d = kl - P.kpop_phi_f;
-        bool out = d > 0.0f;
-        if (!(fabsf(d) > 2e-4f + 1e-6f * P.kpop_phi_f) || logk != logk) {
-            const double lo = 1e-8, hi = 1.0 - 1e-8;
-            double dp = exp(lw64()), dq = exp((double)linf);
-            dp = dp < lo ? lo : (dp > hi ? hi : dp);
-            dq = dq < lo ? lo : (dq > hi ? hi : dq);
-            const double kl_pq = dp * log(dp / dq) + (1.0 - dp) * log((1.0 - dp) / (1.0 - dq));
-            const double kl_qp = dq * log(dq / dp) + (1.0 - dq) * log((1.0 - dq) / (1.0 - dp));
-            const double m = kl_pq > kl_qp ? kl_pq : kl_qp;
-            out = m > P.kpop_phi;
-        }
-        r.trunc = out;
-        r.w = out ? 0.0f : expf(logk);
-        break;
-    }
     case CIS_MODE_SEQ_TIS:
     case CIS_MODE_SEQ_MIS:
         // the weight is the response's (seq_weight); callers pass it in
@@ -304,6 +245,76 @@ __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float
         break;
     default:
         break;
+    }
+    if constexpr (kAll) {
+        switch (P.mode) {
+        case CIS_MODE_BAND: {
+            // Sec. 4.3: the CIS weight, lifted from below to (1 + p)/2 (the image
+            // of e^eps = 1/2).  Both comparisons as for CIS; k near (1 + p)/2 lies
+            // in [1/2, 1], where its error is smaller still
+            const float om = omp >= 0.0f ? omp : -expm1f(lw);
+            const float k = expf(logk);
+            const float lo = om < 0.5f ? 1.0f - 0.5f * om : 0.5f + 0.5f * expf(lw);
+            const int su = certain_cmp(k, 1.0f + P.lam_f * fmaxf(om, P.kappa_f));
+            const int sl = certain_cmp(lo, k);
+            const bool up =
+                su != 0 ? su > 0 : logk64() > log1p(P.lam * fmax(-expm1(lw64()), P.kappa));
+            const bool low = sl != 0 ? sl > 0 : logk64() < log(0.5 * (1.0 + exp(lw64())));
+            r.trunc = up || low;
+            r.w = k;
+            if (up || low) {  // the bounds themselves, to fp32 rounding
+                float pl, e, ph = exp_pair(lw, lw_lo, pl);
+                const float half = two_sum(0.5f, 0.5f * ph, e);
+                r.w = up ? (float)(1.0 + P.lam * fmax((1.0 - (double)ph) - (double)pl, P.kappa))
+                         : half + fmaf(0.5f, pl, e);
+            }
+            break;
+        }
+        case CIS_MODE_ICEPOP: {
+            // Table 8: k on [lo, hi] (bounds included), else masked
+            const int sl = certain_cmp(P.log_icepop_lo_f, logk);
+            const int sh = certain_cmp(logk, P.log_icepop_hi_f);
+            const bool out = (sl != 0 ? sl > 0 : logk64() < P.log_icepop_lo) ||
+                             (sh != 0 ? sh > 0 : logk64() > P.log_icepop_hi);
+            r.trunc = out;
+            r.w = out ? 0.0f : expf(logk);
+            break;
+        }
+        case CIS_MODE_KPOP: {
+            // Table 8 / App. D.5: binary KL both ways on probabilities clamped to
+            // [1e-8, 1 - 1e-8]; masked when the larger exceeds phi.  fp32 decides
+            // unless the two are close.  With L = log p - log q and M = log(1 - p)
+            // - log(1 - q) of the clamped values, |L|, |M| <= 18.5, the two KLs are
+            // p L + (1 - p) M and -(q L + (1 - q) M); p, 1 - p, q and 1 - q carry
+            // relative errors below 1e-6 and the four logs absolute errors below
+            // 6e-6, so each KL is off by less than 1e-6 (2 * 18.5) + 2 * 1.2e-5 <
+            // 7e-5; 2e-4 is taken.  (The clamps drop a NaN: fp64 keeps it.)
+            const float fl = 1e-8f, ll = -18.420681f;  // the clamp and its log
+            const float om = omp >= 0.0f ? omp : -expm1f(lw), oq = -expm1f(linf);
+            const float a = fminf(fmaxf(lw, ll), -fl), b = fminf(fmaxf(linf, ll), -fl);
+            const float p = expf(a), q = expf(b);
+            const float p1 = fminf(fmaxf(om, fl), 1.0f), q1 = fminf(fmaxf(oq, fl), 1.0f);
+            const float L = a - b, M = logf(p1) - logf(q1);
+            const float kl = fmaxf(p * L + p1 * M, -(q * L + q1 * M));
+            const float d = kl - P.kpop_phi_f;
+            bool out = d > 0.0f;
+            if (!(fabsf(d) > 2e-4f + 1e-6f * P.kpop_phi_f) || logk != logk) {
+                const double lo = 1e-8, hi = 1.0 - 1e-8;
+                double dp = exp(lw64()), dq = exp((double)linf);
+                dp = dp < lo ? lo : (dp > hi ? hi : dp);
+                dq = dq < lo ? lo : (dq > hi ? hi : dq);
+                const double kl_pq = dp * log(dp / dq) + (1.0 - dp) * log((1.0 - dp) / (1.0 - dq));
+                const double kl_qp = dq * log(dq / dp) + (1.0 - dq) * log((1.0 - dq) / (1.0 - dp));
+                const double m = kl_pq > kl_qp ? kl_pq : kl_qp;
+                out = m > P.kpop_phi;
+            }
+            r.trunc = out;
+            r.w = out ? 0.0f : expf(logk);
+            break;
+        }
+        default:
+            break;
+        }
     }
     return r;
 }

@@ -29,22 +29,18 @@ namespace {
 
 constexpr int kBatch = 4;  // 16-byte loads in flight per thread
 
-// Beyond this magnitude z log2e may overflow fp32, so exponents are formed
-// from z - m (rows of masked entries at the type's lowest value, for one).
-constexpr float kHuge = 1e38f;
-
 // Running (m, S[, U]) of one thread in the exponent form above; U = sum e x with
-// x = z log2e - c.  With |m| >= kHuge x = (z - m) log2e and c is not used.
+// x = z log2e - c.  With |m| >= kHugeLogit x = (z - m) log2e and c is not used.
 template <bool kEnt> struct ExpAcc {
     float m = -INFINITY, c = -INFINITY, S = 0.0f, U = 0.0f;
 
-    __device__ __forceinline__ bool fast() const { return fabsf(m) < kHuge; }
+    __device__ __forceinline__ bool fast() const { return fabsf(m) < kHugeLogit; }
     // Raise the offset to a larger (or NaN) maximum.
     __device__ __forceinline__ void raise(float mx)
     {
         if (mx > m || mx != mx) {
             const float c1 = mx * kLog2e;
-            const float d = fast() && fabsf(mx) < kHuge ? c - c1 : (m - mx) * kLog2e;
+            const float d = fast() && fabsf(mx) < kHugeLogit ? c - c1 : (m - mx) * kLog2e;
             const float f = ex2_ftz(d);
             if (kEnt)
                 U = f == 0.0f ? 0.0f : fmaf(d, S, U) * f;

@@ -95,8 +95,9 @@ cudaError_t launch_token_logprobs(const PassArgs &a, int dtype, cudaStream_t s);
 cudaError_t launch_rowwise_fwd_bwd(const PassArgs &a, int dtype, int out_dtype,
                                    cudaStream_t s);
 
-// Fused forward + backward, 16-byte aligned rows: a cluster of CTAs splits
-// each row, each CTA keeps its slice in shared memory (one HBM read).
+// Fused forward + backward, rows that a cluster's shared memory holds, any
+// alignment: a cluster of CTAs splits each row, each CTA keeps its slice in
+// shared memory (one HBM read).
 // Returns cudaErrorNotSupported when the shape does not fit the kernel.
 cudaError_t launch_cluster_fwd_bwd(const PassArgs &a, int dtype, int out_dtype,
                                    cudaStream_t s);

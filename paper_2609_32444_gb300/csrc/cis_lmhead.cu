@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(256)
 constexpr int kTokCta = 8;
 constexpr int kTokThreads = 256;
 __global__ void __launch_bounds__(kTokThreads)
-    cis_lmhead_token_kernel(const PassArgs a, const float2 *part, const float *part_u, float *zy,
+    cis_lmhead_token_kernel(const __grid_constant__ PassArgs a, const float2 *part, const float *part_u, float *zy,
                             int nHalf, float *lse_out, float *c_out, const int *pos)
 {
     constexpr int kGroups = kTokThreads / kTokCta;

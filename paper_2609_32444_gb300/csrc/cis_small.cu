@@ -143,8 +143,8 @@ __global__ void __launch_bounds__(kSmallThreads)
 }
 
 __global__ void cis_weights_kernel(const float *lp_w, const float *lp_inf, const uint8_t *mask,
-                               int64_t T, const DevParams P, float *w_out, uint8_t *trunc_out,
-                               float *eps_out)
+                               int64_t T, const __grid_constant__ DevParams P, float *w_out,
+                               uint8_t *trunc_out, float *eps_out)
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
          t += (int64_t)gridDim.x * blockDim.x) {
