@@ -302,8 +302,8 @@ CIS_API cis_status_t cis_loss_fwd_bwd(const void *logits, int32_t dtype, int64_t
             if ((e = launch_token_logprobs(f, dtype, s)) != cudaSuccess)
                 return cuda_status(e);
         }
-        if ((e = cudaMemsetAsync(a.ws_w, 0, 4 * (size_t)T, s)) != cudaSuccess ||
-            (e = cudaMemsetAsync(a.ws_trunc, 0, (size_t)T, s)) != cudaSuccess)
+        // the weight and flag arrays, which lie one after the other
+        if ((e = cudaMemsetAsync(a.ws_w, 0, L.trunc - L.w + (size_t)T, s)) != cudaSuccess)
             return cuda_status(e);
         if ((e = launch_seq_weights(lp_old ? nullptr : a.ws_terms, lp_old, lp_infer, ids, V, mask,
                                     cu_seqlens, B, T, a.P, a.ws_w, a.ws_trunc, s)) != cudaSuccess)
@@ -313,6 +313,9 @@ CIS_API cis_status_t cis_loss_fwd_bwd(const void *logits, int32_t dtype, int64_t
     }
     cudaEvent_t ev0 = g_prof_begin, ev1 = g_prof_end;
     g_prof_begin = g_prof_end = nullptr;
+    // The main kernel overlaps the small kernel before it, unless events are to
+    // bracket it, or no kernel comes between it and a memset.
+    a.overlap = ev0 == nullptr && !(is_seq_mode(params->mode) && B <= 0);
     if (ev0 && (e = cudaEventRecord(ev0, s)) != cudaSuccess)
         return cuda_status(e);
     if (T > 0) {

@@ -25,7 +25,6 @@
 #pragma once
 
 #include <cooperative_groups.h>
-#include <float.h>
 
 #include "cis_dsmem.cuh"
 #include "cis_kernels.h"
@@ -100,6 +99,9 @@ template <typename OutT, int kThreads> __device__ __forceinline__ void zero_run(
     else if ((int)threadIdx.x - head < n - tail)
         dst[tail + threadIdx.x - head] = from_f32<OutT>(0.0f);
 }
+
+// Below this, fl(m log2e) may be off by more than 2^7.
+constexpr float kFarLogit = -1.4e9f;
 
 // Ragged form, rows with maxima beyond z log2e's range (kHugeLogit), or NaN:
 // exponents from z - m.  Rare, and kept out of the kernel's own code (the same
@@ -182,6 +184,8 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     const bool valid = a.mask == nullptr || a.mask[t] != 0;
     const int64_t y = a.ids[t];
     const bool id_ok = y >= 0 && y < a.V;
+    if (threadIdx.x == 0)
+        allow_next_grid();
     if (!valid || !id_ok) {  // same branch in every CTA of the cluster
         if constexpr (kRagged) {
             zero_run<OutT, kThreads>(orow, (int)n);
@@ -190,6 +194,8 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
             for (int g = threadIdx.x; g < ng; g += kThreads)
                 store8<OutT>(orow + 8 * g, zero);
         }
+        if (threadIdx.x == 0)
+            grid_wait();  // in every CTA, so that this grid ends after the one before
         if (rank == 0 && threadIdx.x == 0) {
             const float lp = valid ? NAN : 0.0f;
             if (valid)
@@ -271,8 +277,11 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         linf = a.lp_inf[t];
         lold = a.lp_old ? a.lp_old[t] : 0.0f;
         adv = a.adv[t];
-        sc = a.scale[t];
         qinv = expf(-linf);  // 1 / q, off the row's serial path
+        // the workspace is the kernel before's until it has ended; with the
+        // launch gaps that saves 6 us of 94 at T=4096, V=32000
+        grid_wait();
+        sc = a.scale[t];
     }
     __syncthreads();  // barriers initialised before anyone polls them
 
@@ -305,10 +314,12 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     // the end, so the sum equals the one over (z - m) log2e.
     float s = 0.0f, u = 0.0f;
     if (kRagged ? fabsf(m) < kHugeLogit : m != -INFINITY) {
-        // (aligned form: a thread's entries may all lie at the type's lowest
-        // value, masked; with a finite cm they then count as 0, not NaN)
-        const float cm = kRagged ? m * kLog2e : fmaxf(m * kLog2e, -FLT_MAX);
-        const float cm_err = fmaf(m, kLog2e, -cm);  // m log2e - cm, exactly
+        // Aligned form: a thread's entries may all be masked ones, so low that
+        // the residual of cm leaves the exponential's range; their exponents
+        // are then taken from 0, which makes them count as 0, not NaN.
+        const bool far = !kRagged && m < kFarLogit;
+        const float cm = far ? 0.0f : m * kLog2e;
+        const float cm_err = far ? 0.0f : fmaf(m, kLog2e, -cm);  // m log2e - cm, exactly
 #pragma unroll 2
         for (int g = threadIdx.x; g < ng; g += kThreads) {
             float z[8];
@@ -388,8 +399,8 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
             bias_log2 = (float)J;
             scale = inv * __int_as_float((127 + J) << 23);
         } else {
-            // a row at the lowest value throughout has lost its count: NaN
-            if (!kRagged && o.s == 0.0f && !(fabsf(zy) < kHugeLogit))
+            // a row that low throughout has lost its count: NaN
+            if (!kRagged && o.s == 0.0f && zy < kFarLogit)
                 o.s = NAN;
             const RowScalars rs = row_scalars(o, zy);
             tw = token_weight<kAll>(has_old ? lold : rs.lp, has_old ? 0.0f : rs.lp_lo, linf, a.P,
@@ -528,13 +539,15 @@ cudaError_t launch_cluster_nt(const PassArgs &a, const ClusterPlan &p, cudaStrea
     cfg.blockDim = dim3(NT, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)p.cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = a.overlap ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, a, p.slice);
 }
 

@@ -30,9 +30,10 @@ namespace cis {
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-// Beyond this magnitude z log2e may overflow fp32, so exponents are formed
-// from z - m (rows of masked entries at the type's lowest value, for one).
-constexpr float kHugeLogit = 1e38f;
+// Exponents are formed as z log2e - fl(m log2e) while the rounding of that
+// offset stays below 2^-4, that is, for maxima up to this magnitude, and from
+// z - m beyond it (masked entries at -1e9, -1e30 or the type's lowest value).
+constexpr float kHugeLogit = 1e6f;
 
 // Hyper-parameters as the kernels use them: fp32 copies for the fast path and
 // fp64 values (with logs taken on the host) for the certified fallback.
@@ -63,6 +64,20 @@ constexpr int32_t kStatusBadId = CIS_ERR_BAD_TOKEN_ID;
 // wait gives up after kMaxPolls polls (about 2 s) and reports a timeout.
 constexpr uint32_t kPollSuspendNs = 1000;
 constexpr uint32_t kMaxPolls = 1u << 21;
+
+// Programmatic dependent launch.  A kernel launched with the attribute may start
+// once every CTA of the kernel before it has allowed it (or ended);
+// grid_wait() then holds a thread until that kernel has completed and its
+// writes are visible.  Kernels whose predecessor was launched without the
+// attribute may read what lay ready before it.
+__device__ __forceinline__ void allow_next_grid()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 __device__ __forceinline__ void set_status(int32_t *status, int32_t bits)
 {
@@ -436,6 +451,16 @@ struct MaxSumU {
     float u;
 };
 
+// u moved to the offset m.  The shift is held to a finite range: e^{a.m - m} is 0
+// long before it (masked entries at the type's lowest value).
+__device__ __forceinline__ float shift_u(MaxSumU a, float m)
+{
+    if (a.m == -INFINITY)
+        return a.u * 0.0f;
+    const float d = a.m - m;
+    return fmaf(fmaxf(d, -1e30f), a.s, a.u) * ex2_ftz(d * kLog2e);
+}
+
 // (m, s) comes from ms_combine itself, so the entropy variants of the kernels
 // reduce (m, s) exactly as the others do; u follows the same offsets.
 __device__ __forceinline__ MaxSumU msu_combine(MaxSumU a, MaxSumU b)
@@ -444,10 +469,7 @@ __device__ __forceinline__ MaxSumU msu_combine(MaxSumU a, MaxSumU b)
     const float m = r.m;
     if (m == -INFINITY)
         return {m, r.s, a.u + b.u};
-    const float ua = a.m == -INFINITY ? a.u * 0.0f
-                                      : fmaf(a.m - m, a.s, a.u) * ex2_ftz((a.m - m) * kLog2e);
-    const float ub = b.m == -INFINITY ? b.u * 0.0f
-                                      : fmaf(b.m - m, b.s, b.u) * ex2_ftz((b.m - m) * kLog2e);
+    const float ua = shift_u(a, m), ub = shift_u(b, m);
     return {m, r.s, ua + ub};
 }
 
@@ -500,9 +522,8 @@ __device__ __forceinline__ MaxSumU combine_flat(const float4 *part, unsigned n)
             S += q.y * 0.0f;
             U += q.z * 0.0f;
         } else {
-            const float f = ex2_ftz((q.x - M) * kLog2e);
-            S += q.y * f;
-            U += fmaf(q.x - M, q.y, q.z) * f;
+            S += q.y * ex2_ftz((q.x - M) * kLog2e);
+            U += shift_u(MaxSumU{q.x, q.y, q.z}, M);
         }
     }
     return {M, S, U};

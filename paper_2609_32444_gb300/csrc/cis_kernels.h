@@ -39,6 +39,10 @@ struct PassArgs {
     float *entropy_out;    // per-token entropy of the softmax (may be null)
     void *red_parts;       // the reduction's per-CTA partial sums (workspace)
     uint32_t *red_ticket;  // its completion counter (zeroed by the scales kernel)
+    // The fused cluster kernel may start while the kernel before it on the
+    // stream (the normaliser's, the sequence weights') still runs; host side
+    // only.  The kernels before that one were launched without overlap.
+    bool overlap;
 };
 
 // Host-side parameter checks and the kernels' copy of the parameters.

@@ -1489,8 +1489,7 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
                 if ((e = cudaGetLastError()) != cudaSuccess)
                     return CIS_ERR_CUDA;
             }
-            if (cudaMemsetAsync(a.ws_w, 0, 4 * (size_t)T, s) != cudaSuccess ||
-                cudaMemsetAsync(a.ws_trunc, 0, (size_t)T, s) != cudaSuccess)
+            if (cudaMemsetAsync(a.ws_w, 0, L.base.trunc - L.base.w + (size_t)T, s) != cudaSuccess)
                 return CIS_ERR_CUDA;
             if (launch_seq_weights(lp_old ? nullptr : a.ws_terms, lp_old, lp_infer, ids, V, mask,
                                    cu_seqlens, B, T, a.P, a.ws_w, a.ws_trunc, s) != cudaSuccess)

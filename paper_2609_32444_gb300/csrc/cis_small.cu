@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kSmallThreads)
     __shared__ long long part[kSmallThreads / 32];
     __shared__ int cnt[kMaxSeqInShared];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    allow_next_grid();
     if (threadIdx.x == 0 && status)
         *status = 0;
     if (threadIdx.x == 0 && ticket)  // the reduction at the end of this call counts from 0
@@ -177,6 +178,7 @@ __global__ void __launch_bounds__(kSeqThreads)
 {
     __shared__ double red[kSeqThreads];
     const int64_t i = blockIdx.x;
+    allow_next_grid();
     int64_t b = cu[i], e = cu[i + 1];
     b = b < 0 ? 0 : (b > T ? T : b);
     e = e < b ? b : (e > T ? T : e);
@@ -209,59 +211,62 @@ struct RedPart {
     float maxlk;
 };
 
-__device__ __forceinline__ RedPart red_add(RedPart a, const RedPart &b)
-{
-    a.loss += b.loss;
-    a.excess += b.excess;
-    a.ent += b.ent;
-    a.nvalid += b.nvalid;
-    a.ntrunc += b.ntrunc;
-    a.maxlk = fmaxf(a.maxlk, b.maxlk);
-    return a;
-}
-
-__device__ __forceinline__ RedPart red_shfl(const RedPart &v, int o)
-{
-    RedPart r;
-    r.loss = __shfl_xor_sync(0xffffffffu, v.loss, o);
-    r.excess = __shfl_xor_sync(0xffffffffu, v.excess, o);
-    r.ent = __shfl_xor_sync(0xffffffffu, v.ent, o);
-    r.nvalid = __shfl_xor_sync(0xffffffffu, v.nvalid, o);
-    r.ntrunc = __shfl_xor_sync(0xffffffffu, v.ntrunc, o);
-    r.maxlk = __shfl_xor_sync(0xffffffffu, v.maxlk, o);
-    return r;
-}
-
-__device__ __forceinline__ RedPart red_warp(RedPart v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        v = red_add(v, red_shfl(v, o));
-    return v;
-}
-
-// Sums over the tokens in fp64, deterministic and spread over many SMs (fp64
-// arithmetic runs at a small fraction of the fp32 rate here, so one CTA
-// summing every token was bound by its SM's fp64 pipe).  CTA b takes tokens
-// [256 b, 256 b + 256), one per thread, and reduces them in a fixed tree
-// (within each warp, then over the warps in order) into parts[b]; the last
-// CTA to finish (a ticket, zeroed by the scales kernel at the start of the
+// Sums over the tokens in fp64, deterministic and spread over many SMs: fp64
+// additions run at 2 a clock and SM here, so one CTA summing every token, or
+// butterflies in which every lane adds, are bound by them.  CTA b takes tokens
+// [256 b, 256 b + 256), one per thread, and leaves their sums in parts[b]; the
+// last CTA to finish (a ticket, zeroed by the scales kernel at the start of the
 // call) adds the parts in index order the same way and writes the results.
-__device__ __forceinline__ RedPart block_red(RedPart p, RedPart *sh)
+//
+// The CTA's sums, in thread 0: the values go through shared memory, warp 0 adds
+// the losses, warp 1 the excesses, warp 2 the entropies (lane l: threads l, l +
+// 32, ..., then a butterfly), warp 3 the rest.
+struct RedShared {
+    double v[3][kRedTokens];
+    long long n[2][kRedTokens];
+    float mx[kRedTokens];
+    RedPart out;
+};
+__device__ __forceinline__ RedPart block_red(const RedPart &p, RedShared &sh)
 {
-    constexpr int kWarps = kRedTokens / 32;
-    p = red_warp(p);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0)
-        sh[wid] = p;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    sh.v[0][tid] = p.loss;
+    sh.v[1][tid] = p.excess;
+    sh.v[2][tid] = p.ent;
+    sh.n[0][tid] = p.nvalid;
+    sh.n[1][tid] = p.ntrunc;
+    sh.mx[tid] = p.maxlk;
     __syncthreads();
-    RedPart r{0.0, 0.0, 0.0, 0, 0, 0.0f};
-    if (wid == 0) {
-        r = lane < kWarps ? sh[lane] : r;
-        r = red_warp(r);
+    if (wid < 3) {
+        double s = sh.v[wid][lane];
+#pragma unroll
+        for (int k = 32; k < kRedTokens; k += 32)
+            s += sh.v[wid][lane + k];
+        s = warp_sum(s);
+        if (lane == 0)
+            (wid == 0 ? sh.out.loss : wid == 1 ? sh.out.excess : sh.out.ent) = s;
+    } else if (wid == 3) {
+        long long n = 0, m = 0;
+        float mx = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kRedTokens; k += 32) {
+            n += sh.n[0][lane + k];
+            m += sh.n[1][lane + k];
+            mx = fmaxf(mx, sh.mx[lane + k]);
+        }
+        n = warp_sum(n);
+        m = warp_sum(m);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0) {
+            sh.out.nvalid = n;
+            sh.out.ntrunc = m;
+            sh.out.maxlk = mx;
+        }
     }
     __syncthreads();
-    return r;  // valid in thread 0
+    return sh.out;
 }
 
 __global__ void __launch_bounds__(kRedTokens)
@@ -270,10 +275,11 @@ __global__ void __launch_bounds__(kRedTokens)
                   const int32_t *status, RedPart *parts, uint32_t *ticket, cis_stats_t *stats,
                   double *loss_out)
 {
-    __shared__ RedPart sh[kRedTokens / 32];
+    __shared__ RedShared sh;
     __shared__ bool last;
     RedPart p{0.0, 0.0, 0.0, 0, 0, 0.0f};
     const int64_t t = (int64_t)blockIdx.x * kRedTokens + threadIdx.x;
+    grid_wait();
     if (t < T) {
         p.loss = terms[t];
         if (is_valid(mask, t)) {
@@ -308,8 +314,14 @@ __global__ void __launch_bounds__(kRedTokens)
         x.nvalid = vp[b].nvalid;
         x.ntrunc = vp[b].ntrunc;
         x.maxlk = vp[b].maxlk;
-        q = red_add(q, x);
+        q.loss += x.loss;
+        q.excess += x.excess;
+        q.ent += x.ent;
+        q.nvalid += x.nvalid;
+        q.ntrunc += x.ntrunc;
+        q.maxlk = fmaxf(q.maxlk, x.maxlk);
     }
+    __syncthreads();
     q = block_red(q, sh);
     if (threadIdx.x == 0) {
         if (loss_out)
@@ -368,10 +380,23 @@ cudaError_t launch_reduce(const PassArgs &a, cis_stats_t *stats, double *loss, c
         return cudaErrorInvalidValue;
     static_assert(sizeof(RedPart) <= kRedPartBytes, "a partial sum must fit its slot");
     const int64_t blocks = a.T > 0 ? (a.T + kRedTokens - 1) / kRedTokens : 1;
-    cis_reduce_kernel<<<(unsigned)blocks, kRedTokens, 0, s>>>(
-        a.mask, a.T, a.ws_terms, a.ws_logk, a.ws_w, a.ws_trunc, a.entropy_out, a.status,
-        static_cast<RedPart *>(a.red_parts), a.red_ticket, stats, loss);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kRedTokens);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];  // it waits for the kernel before it itself
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, cis_reduce_kernel, a.mask, a.T,
+                              static_cast<const double *>(a.ws_terms),
+                              static_cast<const float *>(a.ws_logk),
+                              static_cast<const float *>(a.ws_w),
+                              static_cast<const uint8_t *>(a.ws_trunc),
+                              static_cast<const float *>(a.entropy_out),
+                              static_cast<const int32_t *>(a.status),
+                              static_cast<RedPart *>(a.red_parts), a.red_ticket, stats, loss);
 }
 
 cudaError_t launch_seq_weights(const double *lw64, const float *lw32, const float *lp_inf,

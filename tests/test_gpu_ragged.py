@@ -99,18 +99,20 @@ def test_masked_and_bad_rows_are_zeroed_whole(dout, V):
 
 @pytest.mark.parametrize("dtype", [BF16, F32])
 @pytest.mark.parametrize("V", [9000, 9001])
-def test_rows_at_the_lowest_value(dtype, V):
-    """Masked vocabularies: all but a few entries at finfo.min, one row with
-    nothing but the sampled token, on the aligned and the ragged form; a row at
-    finfo.min throughout is uniform on the ragged form and NaN on the aligned
-    one, which keeps no count of such entries."""
-    T, low = 4, torch.finfo(dtype).min
+@pytest.mark.parametrize("low", [None, -1e30, -1e10, -1e9, -1e5])
+def test_rows_at_the_lowest_value(dtype, V, low):
+    """Masked vocabularies: all but a few entries at finfo.min or at a large
+    negative number, one row with nothing but the sampled token, on the aligned
+    and the ragged form; a row at that value throughout is uniform on the ragged
+    form and, below -1.4e9, NaN on the aligned one, which keeps no count of such
+    entries."""
+    T, low = 4, torch.finfo(dtype).min if low is None else low
     z = torch.full((T, V), low, dtype=dtype, device=DEV)
     z[0, 17:8000:900] = 1.5
     z[1, 8990:] = -2.0
     z[2, 5000] = 3.0
     ids = torch.tensor([17, 8999, 5000, 3], dtype=torch.int32, device=DEV)
-    n = T if V % 8 else 3
+    n = T if V % 8 or low >= -1e9 else 3
     for dout in (BF16, F32):
         _check(z[:n], ids[:n], torch.empty((n, V), dtype=dout, device=DEV), n, V, entropy=True)
     if n < T:
