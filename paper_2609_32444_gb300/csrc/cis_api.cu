@@ -71,6 +71,8 @@ DevParams make_dev_params(const cis_params_t &p)
     d.log_rho_hi_f = (float)d.log_rho_hi;
     d.log_icepop_lo = log(p.icepop_lo);
     d.log_icepop_hi = log(p.icepop_hi);
+    d.icepop_lo_f = (float)p.icepop_lo;
+    d.icepop_hi_f = (float)p.icepop_hi;
     d.log_icepop_lo_f = (float)d.log_icepop_lo;
     d.log_icepop_hi_f = (float)d.log_icepop_hi;
     d.kpop_phi = p.kpop_phi;

@@ -88,12 +88,12 @@ template <typename InT, typename OutT> struct Aligned {
     static cudaError_t run(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
     {
         if (a.entropy_out)  // the entropy variant is built for 256 threads only
-            return launch_cluster_nt<InT, OutT, 256, true, false, false>(a, p, s);
+            return launch_cluster_nt<InT, OutT, 256, true, false, Ops::kPlain>(a, p, s);
         switch (p.nt) {
-        case 512: return launch_cluster_nt<InT, OutT, 512, false, false, false>(a, p, s);
-        case 384: return launch_cluster_nt<InT, OutT, 384, false, false, false>(a, p, s);
-        case 128: return launch_cluster_nt<InT, OutT, 128, false, false, false>(a, p, s);
-        default: return launch_cluster_nt<InT, OutT, 256, false, false, false>(a, p, s);
+        case 512: return launch_cluster_nt<InT, OutT, 512, false, false, Ops::kPlain>(a, p, s);
+        case 384: return launch_cluster_nt<InT, OutT, 384, false, false, Ops::kPlain>(a, p, s);
+        case 128: return launch_cluster_nt<InT, OutT, 128, false, false, Ops::kPlain>(a, p, s);
+        default: return launch_cluster_nt<InT, OutT, 256, false, false, Ops::kPlain>(a, p, s);
         }
     }
 };
@@ -128,8 +128,11 @@ cudaError_t launch_cluster_fwd_bwd(const PassArgs &a, int dtype, int out_dtype, 
         p.nt = cluster_threads();
     const bool aligned = aligned_rows(a, dtype == CIS_BF16 ? 2 : 4, out_dtype == CIS_BF16 ? 2 : 4);
     const int m = a.P.mode;
+    // the smallest variant that can do the call
     if (m == CIS_MODE_BAND || m == CIS_MODE_ICEPOP || m == CIS_MODE_KPOP)
         return launch_cluster_all(a, dtype, out_dtype, aligned, p, s);
+    if (a.lp_old || a.w_in)
+        return launch_cluster_given(a, dtype, out_dtype, aligned, p, s);
     return aligned ? launch_cluster_aligned(a, dtype, out_dtype, p, s)
                    : launch_cluster_ragged(a, dtype, out_dtype, p, s);
 }

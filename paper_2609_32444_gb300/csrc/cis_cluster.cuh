@@ -1,5 +1,6 @@
 // cis_cluster.cuh -- the fused pass's cluster kernel and its launch; the launches
-// are instantiated in cis_cluster.cu, cis_cluster_ragged.cu and cis_cluster_all.cu.
+// are instantiated in cis_cluster.cu, cis_cluster_ragged.cu,
+// cis_cluster_given.cu and cis_cluster_all.cu.
 //
 // A bf16 row of the 151,936-entry vocabulary is 303,872 bytes, more than one
 // CTA's shared memory.  A cluster of CS CTAs (1 <= CS <= 8) therefore
@@ -42,15 +43,23 @@ struct ClusterPlan {
 };
 
 
-// The launches, by form and operators (one translation unit each): aligned rows
-// or any; the CIS, TIS, exact, none and sequence operators, or all of them.  The
-// code of operators that are not in use slows the others: the instructions of
-// the serial section compete for the cache (T=16384, V=1000, CIS: 109 us with all
-// of them, 88 without).
+// What a variant of the kernel can do, least code first.  The code of operators
+// that are not in use slows the others: the serial section's instructions
+// compete for the cache (T=16384, V=1000, CIS: 109 us with all of them, 88 without;
+// T=16384, V=151936: 1539 us a step with l_old's, 1463 without).
+enum class Ops {
+    kPlain,  // no l_old: CIS, TIS, exact, none
+    kGiven,  // those with l_old, and the sequence operators (weights given)
+    kAll     // every operator
+};
+
+// The launches, by form and operators, one translation unit each.
 cudaError_t launch_cluster_aligned(const PassArgs &a, int dtype, int out_dtype,
                                    const ClusterPlan &p, cudaStream_t s);
 cudaError_t launch_cluster_ragged(const PassArgs &a, int dtype, int out_dtype,
                                   const ClusterPlan &p, cudaStream_t s);
+cudaError_t launch_cluster_given(const PassArgs &a, int dtype, int out_dtype, bool aligned,
+                                 const ClusterPlan &p, cudaStream_t s);
 cudaError_t launch_cluster_all(const PassArgs &a, int dtype, int out_dtype, bool aligned,
                                const ClusterPlan &p, cudaStream_t s);
 
@@ -161,7 +170,7 @@ template <> struct ClusterShared<true> {
 // the 16-byte blocks that lie inside the slice, plain loads the few entries at
 // its two ends, and nothing outside the slice is read.  Groups of 8 then are
 // 16-byte aligned in the output too wherever its rows have the input's phase.
-template <typename InT, typename OutT, int kThreads, bool kEnt, bool kRagged, bool kAll>
+template <typename InT, typename OutT, int kThreads, bool kEnt, bool kRagged, Ops kOps>
 __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __grid_constant__ PassArgs a, int64_t slice)
 {
     extern __shared__ __align__(128) uint8_t dyn_smem[];
@@ -271,17 +280,34 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     cluster_arrive_relaxed();
 
     // Per-token inputs, fetched while the copy is in flight.
-    float zy = 0.0f, linf = 0.0f, lold = 0.0f, adv = 0.0f, sc = 0.0f, qinv = 0.0f;
+    // The weight is known here where it does not depend on the row (l_old, or a
+    // sequence operator's weight).
+    float zy = 0.0f, linf = 0.0f, lold = 0.0f, adv = 0.0f, sc = 0.0f, qinv = 0.0f, oinv = 0.0f;
+    TokenWeight tw{0.0f, 0.0f, 0};
+    KpopSide kq{0.0f, 0.0f, 0.0f, 0.0f};
+    constexpr bool kAll = kOps == Ops::kAll;
+    const bool has_old = kOps != Ops::kPlain && a.lp_old != nullptr;
+    const bool given = kOps != Ops::kPlain && a.w_in != nullptr;
     if (threadIdx.x == 0) {
         zy = to_f32(irow[y - v0]);
         linf = a.lp_inf[t];
-        lold = a.lp_old ? a.lp_old[t] : 0.0f;
         adv = a.adv[t];
         qinv = expf(-linf);  // 1 / q, off the row's serial path
+        if (has_old) {
+            lold = a.lp_old[t];
+            oinv = expf(-lold);
+            tw = token_weight<kAll>(lold, 0.0f, linf, a.P);
+        } else if (kAll && a.P.mode == CIS_MODE_KPOP) {
+            kq = kpop_side(linf);
+        }
         // the workspace is the kernel before's until it has ended; with the
         // launch gaps that saves 6 us of 94 at T=4096, V=32000
         grid_wait();
         sc = a.scale[t];
+        if (given) {  // a sequence operator: the response's weight
+            tw.w = a.w_in[t];
+            tw.trunc = a.trunc_in[t];
+        }
     }
     __syncthreads();  // barriers initialised before anyone polls them
 
@@ -362,14 +388,13 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     // Thread 0 forms the row's scalars: the serial part of every row, which
     // the other threads wait for, and which shares the SM's issue slots with
     // the other CTAs' streaming loops, so its instruction count sets its
-    // length.  In the common case (row_weight_direct) the weight comes from
-    // the row's statistics without logarithms, and log p, log k and the fp64
-    // loss term are formed after the barrier by rank 0 alone, which stores
-    // them.  Otherwise the log-domain path forms everything here.
+    // length.  In the common case (row_direct) the weight and the update ratio
+    // come from the row's statistics without logarithms, and log p, log k and
+    // the fp64 loss term are formed after the barrier by rank 0 alone, which
+    // stores them.  Otherwise the log-domain path forms everything here.
     MaxSumU ou{0.0f, 0.0f, 0.0f};
-    TokenWeight tw{0.0f, 0.0f, 0};
     double term = 0.0;
-    float lp = 0.0f, tdir = 0.0f;
+    float lp = 0.0f, tdir = 0.0f, obj = adv;  // obj: min(rho A, clip(rho) A)
     bool direct = false;
     if (threadIdx.x == 0) {
         MaxSum o;
@@ -379,16 +404,21 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         } else {
             o = cs == 4 ? combine4(sh.part) : combine_flat(sh.part, cs);
         }
-        const bool has_old = a.lp_old != nullptr;
         float c, omp, bias_log2, scale = 1.0f;
-        DirectWeight dw;
-        direct = !has_old && a.w_in == nullptr && row_weight_direct(o, zy, linf, qinv, a.P, dw);
+        DirectRow dw;
+        direct = row_direct(o, zy, dw);
+        if (direct && !has_old && !given)
+            direct = weight_direct<kAll>(dw, linf, qinv, kq, a.P, tw.w, tw.trunc);
+        float rho = 1.0f;
+        bool flows = true;  // the clip leaves the gradient
+        if (direct && has_old)
+            direct = ratio_direct(dw, lold, oinv, adv, a.P, rho, flows);
         if (direct) {
-            tw.w = dw.w;
-            tw.trunc = dw.trunc;
             omp = dw.omp;
             tdir = dw.t;
-            c = sc * tw.w * adv;  // s w A rho with rho = 1, g = 1 (Eq. 1 without l_old)
+            if (has_old)
+                obj = (flows ? rho : fminf(fmaxf(rho, a.P.rho_lo_f), a.P.rho_hi_f)) * adv;
+            c = flows ? sc * tw.w * adv * rho : 0.0f;  // s w A rho g
             // The softmax's 1 / (s' + e^{z_y - m'}) = e^{m' - z_y} p, in
             // [2^-102, 1] within the closed forms' range, replaces a logarithm:
             // its binary exponent -J goes into the exponent offset (as the
@@ -403,11 +433,13 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
             if (!kRagged && o.s == 0.0f && zy < kFarLogit)
                 o.s = NAN;
             const RowScalars rs = row_scalars(o, zy);
-            tw = token_weight<kAll>(has_old ? lold : rs.lp, has_old ? 0.0f : rs.lp_lo, linf, a.P,
-                              has_old ? -1.0f : rs.omp);
-            if (a.w_in) {  // a sequence operator: the response's weight
-                tw.w = a.w_in[t];
-                tw.trunc = a.trunc_in[t];
+            if (!has_old) {
+                const TokenWeight tn = token_weight<kAll>(rs.lp, rs.lp_lo, linf, a.P, rs.omp);
+                tw.logk = tn.logk;
+                if (!given) {
+                    tw.w = tn.w;
+                    tw.trunc = tn.trunc;
+                }
             }
             const TokenLoss tl = token_loss(rs.lp, rs.lp_lo, has_old, lold, adv, sc, tw.w, a.P);
             term = tl.term;
@@ -448,8 +480,9 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     if (threadIdx.x == 0 && rank == 0) {
         if (direct) {  // log p, log k and the loss term, off the serial path
             lp = -log1pf(tdir);  // p = 1 / (1 + t)
-            tw.logk = lp - linf;
-            term = -(double)sc * (double)tw.w * (double)adv;
+            if (!has_old)
+                tw.logk = lp - linf;
+            term = -(double)sc * (double)tw.w * (double)obj;
         }
         if (a.lp_out) a.lp_out[t] = lp;
         if (a.w_out) a.w_out[t] = tw.w;
@@ -524,10 +557,10 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     cluster_wait();
 }
 
-template <typename InT, typename OutT, int NT, bool kEnt, bool kRagged, bool kAll>
+template <typename InT, typename OutT, int NT, bool kEnt, bool kRagged, Ops kOps>
 cudaError_t launch_cluster_nt(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
 {
-    auto kern = cis_fused_cluster_kernel<InT, OutT, NT, kEnt, kRagged, kAll>;
+    auto kern = cis_fused_cluster_kernel<InT, OutT, NT, kEnt, kRagged, kOps>;
     // a ragged slice has up to 15 entries of padding
     const size_t smem = p.smem + (kRagged ? 16 * sizeof(InT) : 0);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -44,7 +44,7 @@ struct DevParams {
     float tis_cap_f, exact_lo_f, exact_hi_f;
     float rho_lo_f, rho_hi_f;  // 1 - c_low, 1 + c_high
     float log_tis_cap_f, log_exact_lo_f, log_exact_hi_f, log_rho_lo_f, log_rho_hi_f;
-    float log_icepop_lo_f, log_icepop_hi_f, kpop_phi_f;
+    float icepop_lo_f, icepop_hi_f, log_icepop_lo_f, log_icepop_hi_f, kpop_phi_f;
     double lam, kappa;
     double log_tis_cap, log_exact_lo, log_exact_hi, log_rho_lo, log_rho_hi;
     double log_icepop_lo, log_icepop_hi, kpop_phi;
@@ -195,6 +195,22 @@ struct TokenWeight {
     uint8_t trunc;
 };
 
+// What KPop needs of the inference side: log q, q, 1 - q (clamped as in
+// token_weight) and log(1 - q), formed ahead of the row.
+struct KpopSide {
+    float l, q, q1, l1;
+};
+constexpr float kKpopClamp = 1e-8f, kKpopLogClamp = -18.420681f;
+__device__ __forceinline__ KpopSide kpop_side(float linf)
+{
+    KpopSide r;
+    r.l = fminf(fmaxf(linf, kKpopLogClamp), -kKpopClamp);
+    r.q = expf(r.l);
+    r.q1 = fminf(fmaxf(-expm1f(linf), kKpopClamp), 1.0f);
+    r.l1 = logf(r.q1);
+    return r;
+}
+
 // Mismatch weight from log p (training side, the pair lw + lw_lo; lw_lo = 0
 // for an fp32 input) and log q (linf, inference side).  Algorithm 1:
 // p = exp(lw), k = exp(lw - linf), phi = max(1-p, kappa),
@@ -304,13 +320,12 @@ __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float
             // relative errors below 1e-6 and the four logs absolute errors below
             // 6e-6, so each KL is off by less than 1e-6 (2 * 18.5) + 2 * 1.2e-5 <
             // 7e-5; 2e-4 is taken.  (The clamps drop a NaN: fp64 keeps it.)
-            const float fl = 1e-8f, ll = -18.420681f;  // the clamp and its log
-            const float om = omp >= 0.0f ? omp : -expm1f(lw), oq = -expm1f(linf);
-            const float a = fminf(fmaxf(lw, ll), -fl), b = fminf(fmaxf(linf, ll), -fl);
-            const float p = expf(a), q = expf(b);
-            const float p1 = fminf(fmaxf(om, fl), 1.0f), q1 = fminf(fmaxf(oq, fl), 1.0f);
-            const float L = a - b, M = logf(p1) - logf(q1);
-            const float kl = fmaxf(p * L + p1 * M, -(q * L + q1 * M));
+            const KpopSide kq = kpop_side(linf);
+            const float om = omp >= 0.0f ? omp : -expm1f(lw);
+            const float a = fminf(fmaxf(lw, kKpopLogClamp), -kKpopClamp);
+            const float p = expf(a), p1 = fminf(fmaxf(om, kKpopClamp), 1.0f);
+            const float L = a - kq.l, M = logf(p1) - kq.l1;
+            const float kl = fmaxf(p * L + p1 * M, -(kq.q * L + kq.q1 * M));
             const float d = kl - P.kpop_phi_f;
             bool out = d > 0.0f;
             if (!(fabsf(d) > 2e-4f + 1e-6f * P.kpop_phi_f) || logk != logk) {
@@ -559,74 +574,117 @@ __device__ __forceinline__ MaxSumU block_msu(MaxSumU v, MaxSumU *sh)
     return r;
 }
 
-// The weight of the common case straight from a row's statistics, without
-// logarithms: the CIS, TIS, exact and no-correction operators with the
-// current log p as l_w (no l_old, no sequence weight).  From (m', s') over
-// j != y and z_y, with t = s' e^{m' - z_y} = (1 - p) / p:
-//   p = 1 / (1 + t),   1 - p = t p,   k = p / q = p e^{-l_inf},
-// each within ~8 ulp (expf, __fdividef: 2 ulp each), so k and the cap carry
-// relative errors near 2e-6, inside certain_cmp's 4e-6 (k + cap).  qinv is
-// e^{-l_inf}, formed by the caller ahead of time.  Returns false, deciding
-// nothing, where these forms would leave the normal fp32 range
-// (|m' - z_y| > 70, l_inf < -70, an empty or non-finite row) or the decision
-// is too close to call; the caller then takes the log-domain path
-// (row_scalars, token_weight), whose fp64 fallback settles it.
-struct DirectWeight {
-    float w;
+// The row's probabilities straight from its statistics, without logarithms.
+// From (m', s') over j != y and z_y, with t = s' e^{m' - z_y} = (1 - p) / p:
+//   p = 1 / (1 + t),   1 - p = t p,
+// each within ~8 ulp (expf, __fdividef: 2 ulp each), so that k = p e^{-l_inf}
+// and rho = p e^{-l_old} (the exponentials formed ahead of time) and the bounds
+// they are compared with carry relative errors near 2e-6, inside certain_cmp's
+// 4e-6 (a + b).  False where these forms would leave the normal fp32 range
+// (|m' - z_y| > 70, an empty or non-finite row): the caller then takes the
+// log-domain path (row_scalars, token_weight, token_loss), as it does where a
+// decision is too close to call; that path's fp64 fallback settles it.
+struct DirectRow {
     float omp;  // 1 - p
     float t;    // (1 - p) / p; log p = -log1p(t)
     float E;    // e^{m' - z_y}
     float p;
-    uint8_t trunc;
 };
-__device__ __forceinline__ bool row_weight_direct(MaxSum o, float zy, float linf, float qinv,
-                                                  const DevParams &P, DirectWeight &r)
+__device__ __forceinline__ bool row_direct(MaxSum o, float zy, DirectRow &r)
 {
     float dl;
     const float dh = two_sum(o.m, -zy, dl);  // m' - z_y = dh + dl exactly
-    if (!(fabsf(dh) <= 70.0f) || !(linf >= -70.0f) || !(o.s >= 1.0f) || !(o.s <= 3.0e38f))
+    if (!(fabsf(dh) <= 70.0f) || !(o.s >= 1.0f) || !(o.s <= 3.0e38f))
         return false;
     const float e = expf(dh);
     r.E = fmaf(e, dl, e);
-    const float t = o.s * r.E;
-    const float p = __fdividef(1.0f, 1.0f + t);
-    const float k = p * qinv;
-    r.t = t;
-    r.p = p;
-    r.omp = t * p;
-    r.trunc = 0;
-    r.w = 1.0f;
+    r.t = o.s * r.E;
+    r.p = __fdividef(1.0f, 1.0f + r.t);
+    r.omp = r.t * r.p;
+    return true;
+}
+
+// The weight with the current log p as l_w (no l_old, no sequence weight); qinv
+// is e^{-l_inf}.  kAll as in token_weight.  False where a decision is too close
+// to call, l_inf < -70, or the band's bounds are taken (they are rounded once,
+// from pairs, by token_weight).
+template <bool kAll>
+__device__ __forceinline__ bool weight_direct(const DirectRow &d, float linf, float qinv,
+                                              const KpopSide &kq, const DevParams &P, float &w,
+                                              uint8_t &trunc)
+{
+    if (!(linf >= -70.0f))
+        return false;
+    const float k = d.p * qinv;
+    trunc = 0;
+    w = k;
     switch (P.mode) {
     case CIS_MODE_CIS: {
-        const float cap = 1.0f + P.lam_f * fmaxf(r.omp, P.kappa_f);
+        const float cap = 1.0f + P.lam_f * fmaxf(d.omp, P.kappa_f);
         const int s = certain_cmp(k, cap);
-        if (s == 0)
-            return false;
-        r.trunc = s > 0;
-        r.w = s > 0 ? cap : k;
-        return true;
+        trunc = s > 0;
+        w = s > 0 ? cap : k;
+        return s != 0;
     }
     case CIS_MODE_TIS: {
         const int s = certain_cmp(k, P.tis_cap_f);
-        if (s == 0)
-            return false;
-        r.trunc = s > 0;
-        r.w = s > 0 ? P.tis_cap_f : k;
-        return true;
+        trunc = s > 0;
+        w = s > 0 ? P.tis_cap_f : k;
+        return s != 0;
     }
     case CIS_MODE_EXACT: {
         const int sh = certain_cmp(k, P.exact_hi_f), sl = certain_cmp(P.exact_lo_f, k);
-        if (sh == 0 || sl == 0)
-            return false;
-        r.trunc = sh > 0 || sl > 0;
-        r.w = sh > 0 ? P.exact_hi_f : (sl > 0 ? P.exact_lo_f : k);
-        return true;
+        trunc = sh > 0 || sl > 0;
+        w = sh > 0 ? P.exact_hi_f : (sl > 0 ? P.exact_lo_f : k);
+        return sh != 0 && sl != 0;
     }
     case CIS_MODE_NONE:
+        w = 1.0f;
         return true;
     default:
-        return false;
+        break;
     }
+    if constexpr (kAll) {
+        switch (P.mode) {
+        case CIS_MODE_BAND: {
+            const float cap = 1.0f + P.lam_f * fmaxf(d.omp, P.kappa_f);
+            return certain_cmp(k, cap) < 0 && certain_cmp(k, 1.0f - 0.5f * d.omp) > 0;
+        }
+        case CIS_MODE_ICEPOP: {
+            const int sl = certain_cmp(P.icepop_lo_f, k), sh = certain_cmp(k, P.icepop_hi_f);
+            trunc = sl > 0 || sh > 0;
+            w = trunc ? 0.0f : k;
+            return sl != 0 && sh != 0;
+        }
+        case CIS_MODE_KPOP: {
+            // the comparison of token_weight, with log p and log(1 - p) from t
+            const float lp = -log1pf(d.t);
+            const float a = fminf(fmaxf(lp, kKpopLogClamp), -kKpopClamp);
+            const float p = fminf(fmaxf(d.p, kKpopClamp), 1.0f);
+            const float p1 = fminf(fmaxf(d.omp, kKpopClamp), 1.0f);
+            const float L = a - kq.l, M = logf(p1) - kq.l1;
+            const float e = fmaxf(p * L + p1 * M, -(kq.q * L + kq.q1 * M)) - P.kpop_phi_f;
+            trunc = e > 0.0f;
+            w = trunc ? 0.0f : k;
+            return fabsf(e) > 2e-4f + 1e-6f * P.kpop_phi_f;
+        }
+        default:
+            break;
+        }
+    }
+    return false;
+}
+
+// rho = exp(l - l_old) and whether the PPO clip leaves the gradient (Eq. 1);
+// oinv is e^{-l_old}.  False where that is too close to call or l_old < -70.
+__device__ __forceinline__ bool ratio_direct(const DirectRow &d, float lold, float oinv, float A,
+                                             const DevParams &P, float &rho, bool &g)
+{
+    rho = d.p * oinv;
+    const int s = A > 0.0f ? certain_cmp(P.rho_hi_f, rho)
+                           : (A < 0.0f ? certain_cmp(rho, P.rho_lo_f) : 1);
+    g = s > 0;
+    return s != 0 && lold >= -70.0f && A == A;
 }
 
 // Per-row scalars from (m', s') over j != y and z_y.  With the log-odds

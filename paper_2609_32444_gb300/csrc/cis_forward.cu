@@ -332,6 +332,9 @@ __global__ void __launch_bounds__(NT) cis_logprob_kernel(const PassArgs a, unsig
 //   357 / 376, 8 loads 350 / 371.
 // - 64 threads for rows of at most 512 vectors, which 256 threads would not fill
 //   once: T=16384, V=4096 takes 26.6 us against 71.6.
+// - 128 threads where 256 would leave a last, part-empty round of rows among few
+//   (8 CTAs an SM, up to four rounds): T=2048, V=151936, a quarter masked, takes
+//   81.7 us against 92.8; T=2000, V=32003 23.5 against 25.7.
 // - A row is split over a cluster only while the clusters' CTAs stay within 608
 //   (four a SM), since the exchange costs more than it gives once the SMs are
 //   busy: V=151936 takes 33.2 us against 37.7 (one CTA a row, two) at T=512, 11.6
@@ -343,7 +346,7 @@ struct FwdPlan {
 FwdPlan fwd_plan(int64_t T, int64_t V, int in_bytes)
 {
     const int64_t nvec = V * in_bytes / 16;
-    FwdPlan p{1, nvec <= 512 ? 64 : 256};
+    FwdPlan p{1, nvec <= 512 ? 64 : (T > 1216 && T <= 4864 ? 128 : 256)};
     while (p.cs < kMaxCluster && T * p.cs * 2 <= 608 && nvec / (2 * p.cs) >= 512)
         p.cs *= 2;
     return p;
@@ -369,11 +372,15 @@ cudaError_t launch_fwd(const PassArgs &a, int cs, cudaStream_t s)
 template <typename InT> cudaError_t launch_fwd_t(const PassArgs &a, cudaStream_t s)
 {
     const FwdPlan p = fwd_plan(a.T, a.V, (int)sizeof(InT));
-    if (a.entropy_out)
-        return p.nt == 64 ? launch_fwd<InT, true, 64>(a, p.cs, s)
-                          : launch_fwd<InT, true, 256>(a, p.cs, s);
-    return p.nt == 64 ? launch_fwd<InT, false, 64>(a, p.cs, s)
-                      : launch_fwd<InT, false, 256>(a, p.cs, s);
+    const bool ent = a.entropy_out != nullptr;
+    switch (p.nt) {
+    case 64: return ent ? launch_fwd<InT, true, 64>(a, p.cs, s)
+                        : launch_fwd<InT, false, 64>(a, p.cs, s);
+    case 128: return ent ? launch_fwd<InT, true, 128>(a, p.cs, s)
+                         : launch_fwd<InT, false, 128>(a, p.cs, s);
+    default: return ent ? launch_fwd<InT, true, 256>(a, p.cs, s)
+                        : launch_fwd<InT, false, 256>(a, p.cs, s);
+    }
 }
 
 }  // namespace

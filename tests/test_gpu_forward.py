@@ -55,6 +55,7 @@ def _check(z, ids):
 @pytest.mark.parametrize("T,V", [
     (5, 1), (5, 2), (4, 7), (4, 8), (4, 9), (6, 15), (3, 63), (3, 2049),   # 64 threads a row
     (4, 4096), (4, 4097), (3, 4104), (700, 8200),                           # 256 threads a row
+    (1217, 4113),                                                           # 128
     (300, 8207), (150, 16391), (3, 16391), (2, 40003)])                     # 2 to 8 CTAs a row
 def test_row_splits_and_ragged_ends(dtype, T, V):
     """Rows that start at every offset from a 16-byte boundary (an odd stride
