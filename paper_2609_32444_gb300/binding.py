@@ -9,6 +9,7 @@ the compiled library and CUDA tensors, and raises otherwise.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import torch
@@ -66,6 +67,7 @@ class CisError(RuntimeError):
 
 
 _lib = None
+_native = None
 
 
 def library_path() -> str:
@@ -128,7 +130,23 @@ def lib():
                                   P]
     L.cis_binned_sums.restype = ctypes.c_int
     _lib = L
+    _load_native(path)
     return L
+
+
+def _load_native(path):
+    """The calls' native part (csrc/cis_native.cpp).  Each of its functions returns
+    the call's result, an int (the library's error), or None where its plain case
+    does not apply; the Python code below then makes the call."""
+    global _native
+    so = _build.native_path()
+    if not os.path.exists(so):
+        raise ImportError(f"{so} is not built; run __graft_entry__.build()")
+    spec = importlib.util.spec_from_file_location("_cis_native", so)
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    m.init(path)
+    _native = m
 
 
 def status_string(code: int) -> str:
@@ -222,6 +240,12 @@ def cis_token_logprobs(logits: torch.Tensor, ids: torch.Tensor, mask=None, V=Non
     """log p of the sampled tokens (fp32) -- and the row logsumexp and the
     softmax entropy if asked: returns lp, or a tuple (lp, lse, entropy) with
     None for what was not asked when either is."""
+    lib()
+    r = _native.token_logprobs(logits, ids, mask, V, want_lse, dev_status, want_entropy)
+    if r is not None:
+        if type(r) is int:
+            _check(r, "cis_token_logprobs")
+        return r
     _need_cuda(logits, ids, mask)
     T, ld = _rows(logits)
     V = logits.shape[1] if V is None else V
@@ -243,6 +267,12 @@ def cis_weights(lp_train: torch.Tensor, lp_infer: torch.Tensor, params: cis_para
                 mask=None, want_trunc=True, want_eps=False, cu_seqlens=None):
     """Weights of Algorithm 1 / Table 8 (the sequence operators need
     cu_seqlens).  Returns (w, trunc or None, eps or None)."""
+    lib()
+    r = _native.weights(lp_train, lp_infer, params, mask, want_trunc, want_eps, cu_seqlens)
+    if r is not None:
+        if type(r) is int:
+            _check(r, "cis_weights")
+        return r
     _need_cuda(lp_train, lp_infer, mask, cu_seqlens)
     T = lp_train.shape[0]
     _vec(lp_train, torch.float32, T, "lp_train")
@@ -276,6 +306,14 @@ def cis_loss_fwd_bwd(logits: torch.Tensor, ids: torch.Tensor, lp_infer: torch.Te
     """Fused forward + backward token pass.  Returns a dict with dlogits, lp, w,
     trunc, entropy (if asked), loss (device fp64 [1]), stats (device bytes of
     cis_stats_t) and the workspace (its first int32 is the device status word)."""
+    lib()
+    r = _native.loss_fwd_bwd(logits, ids, lp_infer, adv, params, lp_old, mask, cu_seqlens,
+                             dlogits, dlogits_dtype, V, want_lp, want_w, want_trunc, workspace,
+                             want_entropy)
+    if r is not None:
+        if type(r) is int:
+            _check(r, "cis_loss_fwd_bwd")
+        return r
     _need_cuda(logits, ids, lp_infer, adv, lp_old, mask, cu_seqlens, dlogits)
     T, ld = _rows(logits)
     V = logits.shape[1] if V is None else V
@@ -439,6 +477,12 @@ def cis_mismatch_diagnostics(logits_train: torch.Tensor, logits_infer: torch.Ten
                              dev_status=None):
     """Per-position mismatch diagnostics (App. A.5; Sec. 4.3, Fig. 5c-d): a dict
     of device float [T] tensors eps, logk, p, bias2, dvar."""
+    lib()
+    r = _native.mismatch_diagnostics(logits_train, logits_infer, ids, params, mask, V, dev_status)
+    if r is not None:
+        if type(r) is int:
+            _check(r, "cis_mismatch_diagnostics")
+        return r
     _need_cuda(logits_train, logits_infer, ids, mask)
     if logits_train.dtype != logits_infer.dtype:
         raise TypeError("both logit tensors must have the same type")
@@ -464,6 +508,12 @@ def cis_binned_sums(key: torch.Tensor, edges, values=(), mask=None):
     `key` and each of `values` are device float [T] tensors, `edges` a
     sequence of nbins + 1 strictly ascending floats.  Returns (counts int64
     [nbins], sums float64 [len(values), nbins]) on the device."""
+    lib()
+    r = _native.binned_sums(key, edges, values, mask)
+    if r is not None:
+        if type(r) is int:
+            _check(r, "cis_binned_sums")
+        return r
     _need_cuda(key, mask, *values)
     T = key.shape[0]
     _vec(key, torch.float32, T, "key")

@@ -1,0 +1,143 @@
+"""The binding's native calls against its Python ones: the same results where
+both make the call, and the same refusals (what the native part does not take
+goes on to the Python code, whose checks raise).
+"""
+import contextlib
+
+import pytest
+import torch
+
+from paper_2609_32444_gb300 import binding, synth
+
+DEV = torch.device("cuda")
+gpu = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2609_32444_gb300 import build
+    build.build()
+    binding.lib()
+
+
+class _Python:
+    """Stands in for the native module: every call goes on in Python."""
+
+    def __getattr__(self, name):
+        return lambda *a: None
+
+
+@contextlib.contextmanager
+def _python_only():
+    kept = binding._native
+    binding._native = _Python()
+    try:
+        yield
+    finally:
+        binding._native = kept
+
+
+def _same(a, b):
+    assert type(a) is type(b)
+    if isinstance(a, dict):
+        assert list(a) == list(b)
+        for k in a:
+            if k != "workspace":
+                _same(a[k], b[k])
+    elif isinstance(a, (tuple, list)):
+        assert len(a) == len(b)
+        for x, y in zip(a, b):
+            _same(x, y)
+    elif a is not None:
+        assert a.dtype == b.dtype and a.shape == b.shape and a.device == b.device
+        assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8))
+
+
+def _both(f):
+    x = f()
+    with _python_only():
+        y = f()
+    torch.cuda.synchronize()
+    _same(x, y)
+
+
+def _args():
+    b = synth.make_batch(2, T=200, V=1024)
+    b.mask[::3] = 0
+    return {k: getattr(b, k).to(DEV) for k in ("logits", "ids", "lp_infer", "adv", "mask",
+                                              "cu_seqlens")}
+
+
+class TestOnGpu:
+    pytestmark = gpu
+
+    @pytest.mark.parametrize("kw", [
+        {}, {"want_lp": False, "want_trunc": False}, {"want_w": False, "want_entropy": True},
+        {"dlogits_dtype": torch.float32}, {"V": 1000}, {"mask": None, "cu_seqlens": None}])
+    def test_loss(self, kw):
+        x = _args()
+        P = binding.cis_default_params("cis")
+        kw = dict({"mask": x["mask"], "cu_seqlens": x["cu_seqlens"]}, **kw)
+        _both(lambda: binding.cis_loss_fwd_bwd(x["logits"], x["ids"], x["lp_infer"], x["adv"], P,
+                                               **kw))
+        dz = torch.empty((200, 1030), dtype=torch.float32, device=DEV)
+        ws = torch.empty(1 << 20, dtype=torch.uint8, device=DEV)
+        _both(lambda: {k: v.clone() if k == "dlogits" else v for k, v in binding.cis_loss_fwd_bwd(
+            x["logits"], x["ids"], x["lp_infer"], x["adv"], P, lp_old=x["lp_infer"],
+            dlogits=dz.zero_(), workspace=ws, **{k: v for k, v in kw.items()
+                                                 if k in ("mask", "cu_seqlens")}).items()})
+
+    def test_other_calls(self):
+        x = _args()
+        P = binding.cis_default_params("tis")
+        lp = binding.cis_token_logprobs(x["logits"], x["ids"])
+        for kw in ({}, {"want_lse": True}, {"want_entropy": True, "mask": x["mask"]},
+                   {"want_lse": True, "want_entropy": True, "V": 1000}):
+            _both(lambda: binding.cis_token_logprobs(x["logits"], x["ids"], **kw))
+        for kw in ({}, {"want_trunc": False, "want_eps": True, "mask": x["mask"]}):
+            _both(lambda: binding.cis_weights(lp, x["lp_infer"], P, **kw))
+        _both(lambda: binding.cis_weights(lp, x["lp_infer"], binding.cis_default_params("seq_mis"),
+                                          cu_seqlens=x["cu_seqlens"]))
+        for e, v in (([0.0, 0.5, 1.0], (lp, lp)), ((0, 1), ()), ([-50.0, -1, 0.0], [lp])):
+            _both(lambda: binding.cis_binned_sums(lp, e, v, mask=x["mask"]))
+        _both(lambda: binding.cis_mismatch_diagnostics(x["logits"], x["logits"], x["ids"], P,
+                                                       mask=x["mask"]))
+
+    def test_refusals(self):
+        """Wrong kinds, types, shapes and strides, and the library's own errors."""
+        x = _args()
+        P = binding.cis_default_params("cis")
+        z, ids, li, adv = x["logits"], x["ids"], x["lp_infer"], x["adv"]
+        loss = binding.cis_loss_fwd_bwd
+        calls = [
+            lambda: loss(z.half(), ids, li, adv, P), lambda: loss(z, ids.long(), li, adv, P),
+            lambda: loss(z, ids, li[:-1], adv, P), lambda: loss(z.t(), ids, li, adv, P),
+            lambda: loss(z, ids, li, adv, bytes(200)), lambda: loss(z, ids, li, adv.cpu(), P),
+            lambda: loss(z, ids, li, adv, P, V=2000), lambda: loss(z, ids, li, adv, P, V=-1),
+            lambda: loss(z, ids, li, adv, P, dlogits_dtype=torch.float16),
+            lambda: loss(z, ids, li, adv, P, dlogits=torch.empty((200, 8), device=DEV)),
+            lambda: loss(z, ids, li, adv, binding.cis_default_params("seq_tis")),
+            lambda: loss(z, ids, li, adv, binding.cis_default_params("cis", lam=-1.0)),
+            lambda: binding.cis_token_logprobs(z[0], ids), lambda: binding.cis_weights(li, None, P),
+            lambda: binding.cis_binned_sums(li, [0.5, 0.5]),
+            lambda: binding.cis_binned_sums(li, [0.0, 1.0], (li.double(),)),
+            lambda: binding.cis_mismatch_diagnostics(z, z.float(), ids, P)]
+        for i, f in enumerate(calls):
+            errors = []
+            for python in (False, True):
+                with _python_only() if python else contextlib.nullcontext():
+                    with pytest.raises(Exception) as e:
+                        f()
+                    errors.append((type(e.value), str(e.value)))
+            assert errors[0] == errors[1], (i, errors)
+
+
+def test_host_tensors_are_refused_as_before():
+    z, ids, v = torch.zeros(4, 8), torch.zeros(4, dtype=torch.int32), torch.zeros(4)
+    P = binding.cis_default_params("cis")
+    for f in (lambda: binding.cis_loss_fwd_bwd(z, ids, v, v, P),
+              lambda: binding.cis_token_logprobs(z, ids), lambda: binding.cis_weights(v, v, P),
+              lambda: binding.cis_mismatch_diagnostics(z, z, ids, P),
+              lambda: binding.cis_binned_sums(v, [0.0, 1.0])):
+        with pytest.raises(ValueError, match="libcis takes CUDA tensors"):
+            f()
