@@ -812,7 +812,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // counted from their number, which stays on the device.  At T=16384, H=2048,
 // V=151936 with 40% masked the call takes 15.8 ms against 25.0 for
 // multiplying the masked rows as well; the copy and the scan take 33 us.
-// Batches of one row tile have nothing to gain and are multiplied as they are.
+// Smaller calls are multiplied as they are (kPackWork).
 //
 // One CTA: pos[t] = the place of token t among the valid ones (-1: masked),
 // their ids in that order, and their number.
@@ -1266,6 +1266,18 @@ static int64_t chunk_for_bytes(int64_t T, int64_t V, int64_t Hd, size_t bytes)
 // dH and dW take 552 us (two chunks) against 1123 one after the other, the call
 // 1096 against 1600; ranges of a share took 578, of a third 626, of a sixth
 // 577.  T=300, H=1024, V=32003: 68 against 212.
+// Leaving masked tokens out costs a call about 20 us (a scan, a copy, the zeroed
+// rows), whether or not many are masked: T=1244, V=1040, H=3072 with 40% masked took
+// 107 us against 93.  It is done from here on, where the products take 400 us.
+// (CIS_LMHEAD_PACK=1: always; =0: never.)
+constexpr double kPackWork = 8e10;  // tokens x vocabulary x hidden size
+static bool pack_on(int64_t T, int64_t V, int64_t Hd)
+{
+    const char *e = getenv("CIS_LMHEAD_PACK");
+    if (e && (e[0] == '0' || e[0] == '1'))
+        return e[0] == '1';
+    return (double)T * (double)V * (double)Hd >= kPackWork;
+}
 constexpr int64_t kSplitSms = 152;  // the split follows the shape alone
 constexpr int kMaxSplits = 16;
 struct Split {
@@ -1409,8 +1421,8 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
         const bool bf16 = grad_dtype == CIS_BF16;
         // one row tile has no partner to share B with
         const int mc = nTt == 1 ? 0 : lm::mc_mask();
-        // Masked tokens are left out of the products where there is more than
-        // one row tile to save.  What that needs lives in memory that is free
+        // Masked tokens are left out of the products of larger calls
+        // (kPackWork).  What that needs lives in memory that is free
         // until the token step, each token's entry where the step itself writes
         // that token's value: the places in ws_logk, the ids in lse, afterwards
         // the row map in zy.  The valid tokens' hidden states take dH's fp32
@@ -1419,7 +1431,8 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
         const uintptr_t h0 = reinterpret_cast<uintptr_t>(hidden), hb = (uintptr_t)(T * H) * 2;
         const uintptr_t d0 = reinterpret_cast<uintptr_t>(dhidden),
                         db = (uintptr_t)(T * H) * (bf16 ? 2 : 4);
-        const bool packed = mask != nullptr && nTt > 1 && !(h0 < d0 + db && d0 < h0 + hb);
+        const bool packed = mask != nullptr && nTt > 1 && pack_on(T, V, H) &&
+                            !(h0 < d0 + db && d0 < h0 + hb);
         int *count = packed ? reinterpret_cast<int *>(ws + L.base.status + 128) : nullptr;
         int *pos = packed ? reinterpret_cast<int *>(a.ws_logk) : nullptr;
         int32_t *ids_c = reinterpret_cast<int32_t *>(lse);

@@ -24,6 +24,11 @@ def _built():
     binding.lib()
 
 
+@pytest.fixture(autouse=True)
+def _packed(monkeypatch):
+    monkeypatch.setenv("CIS_LMHEAD_PACK", "1")  # these sizes are below the rule's
+
+
 @pytest.mark.parametrize("grad", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("T,V,H,valid", [
     (129, 1000, 256, 1), (300, 1000, 512, 128), (300, 1000, 512, 129),  # one tile, just over one
