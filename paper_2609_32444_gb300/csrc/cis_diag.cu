@@ -18,9 +18,8 @@
 //   Var(f g) - Var(g) = C1 + P2 C2 - [C4 - (2 + C3) C5 - C3 C6 + C3 (2 + C3) P2]
 //   with C6 = sum q (f + 1) p = C5 + 2 QP.
 // Every term but P2 is proportional to f - 1 or to q f - p, so neither result
-// is a small difference of O(1) numbers.  Per-thread sums are fp32; the
-// one-CTA kernel adds the threads' sums in fp64, the streaming kernel adds a
-// warp's in fp32 and the warps' in fp64.
+// is a small difference of O(1) numbers.  Per-thread and warp sums are fp32, the
+// warps' are added in fp64.
 //
 // Two kernels compute this:
 //   - cis_mismatch_stream_kernel (bf16 rows, V a multiple of 8, 16-byte
@@ -31,13 +30,13 @@
 //     forming each row's outputs while the consumer warps go on; pass 2
 //     forms two candidates per instruction with the packed f32x2 FMA, add
 //     and multiply;
-//   - cis_mismatch_kernel (any row): one CTA per position streaming both rows
-//     from global memory with vector loads, twice.
+//   - cis_mismatch_split_kernel (any row): a CTA, or for few rows a cluster, per
+//     position reading both rows from global memory with vector loads, twice.
 #include <stdlib.h>
 
 #include "cis_dsmem.cuh"
 #include "cis_kernels.h"
-#include "cis_rowops.cuh"
+#include "cis_expacc.cuh"
 #include "cis_nvtx.h"
 
 namespace cis {
@@ -86,134 +85,6 @@ __device__ __forceinline__ float elem_weight(float xp, float xq, float p, float 
     }
     return 1.0f;  // CIS_MODE_NONE
 }
-
-struct DiagShared {
-    MaxSum red[kDiagThreads / 32];
-    double sums[kDiagThreads / 32][kNSums];
-    float lse_p, lse_q;
-};
-
-template <typename InT, int MODE>
-__global__ void __launch_bounds__(kDiagThreads)
-    cis_mismatch_kernel(const InT *zt, const InT *zi, int64_t T, int64_t V, int64_t ld_t,
-                        int64_t ld_i, const int32_t *ids, const uint8_t *mask,
-                        const DevParams P, float *eps_out, float *logk_out, float *p_out,
-                        float *bias2_out, float *dvar_out, int32_t *status)
-{
-    __shared__ DiagShared sh;
-    const int64_t t = blockIdx.x;
-    const bool valid = mask == nullptr || mask[t] != 0;
-    const int64_t y = ids[t];
-    const bool id_ok = y >= 0 && y < V;
-    if (!valid || !id_ok) {
-        if (threadIdx.x == 0) {
-            const float v = valid ? NAN : 0.0f;
-            if (valid)
-                set_status(status, kStatusBadId);
-            eps_out[t] = v;
-            if (logk_out) logk_out[t] = v;
-            if (p_out) p_out[t] = v;
-            if (bias2_out) bias2_out[t] = v;
-            if (dvar_out) dvar_out[t] = v;
-        }
-        return;
-    }
-    const InT *rt = zt + t * ld_t;
-    const InT *ri = zi + t * ld_i;
-    // pass 1: each engine's (max, sum) over j != y
-    const MaxSum ot = block_ms<kDiagThreads>(row_stats<InT, false, MaxSum, kDiagThreads>(rt, V, y),
-                                             sh.red);
-    const MaxSum oi = block_ms<kDiagThreads>(row_stats<InT, false, MaxSum, kDiagThreads>(ri, V, y),
-                                             sh.red);
-    if (threadIdx.x == 0) {
-        const float zyt = to_f32(rt[y]), zyi = to_f32(ri[y]);
-        const RowScalars st = row_scalars(ot, zyt), si = row_scalars(oi, zyi);
-        // eps = logit p - logit q: Lemma 3.1's -delta_y + log sum_{j != y} w_j e^{delta_j}
-        // in the normalised gauge, from the log-odds of each engine
-        const double dp = ((double)zyt - (double)ot.m) - (double)logf(ot.s);
-        const double dq = ((double)zyi - (double)oi.m) - (double)logf(oi.s);
-        eps_out[t] = (float)(dp - dq);
-        if (logk_out) logk_out[t] = (float)(st.lp64() - si.lp64());
-        if (p_out) p_out[t] = expf(st.lp);
-        sh.lse_p = st.lse;
-        sh.lse_q = si.lse;
-    }
-    __syncthreads();
-    // the exponents in log2 units, x = z log2e - lse log2e (one FMA each);
-    // probabilities that flush to 0 add nothing measurable to the sums
-    const float op = sh.lse_p * kLog2e, oq = sh.lse_q * kLog2e;
-    // pass 2: the sums over every candidate j
-    float acc[kNSums] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    auto add = [&](float a, float b) {
-        const float xp = fmaf(a, kLog2e, -op), xq = fmaf(b, kLog2e, -oq);
-        const float p = ex2_ftz(xp), q = ex2_ftz(xq);
-        const float k = ex2_ftz(xp - xq);
-        // a candidate with q = 0 is never drawn: only r = -p counts, so f = 1
-        const float f = q > 0.0f ? elem_weight<MODE>(xp, xq, p, k, P) : 1.0f;
-        const float fm1 = f - 1.0f;
-        const float t1 = q * (fm1 * (f + 1.0f));   // q (f^2 - 1)
-        const float t2 = q * fm1;                  // q (f - 1)
-        const float r = fmaf(q, f, -p);
-        acc[0] = fmaf(p, p, acc[0]);                       // P2
-        acc[1] = fmaf(r, r, acc[1]);                       // R2
-        acc[2] = fmaf(r, p, acc[2]);                       // RP
-        acc[3] = fmaf(t1, fmaf(-2.0f, p, 1.0f), acc[3]);   // C1
-        acc[4] += t1;                                      // C2
-        acc[5] += t2;                                      // C3
-        acc[6] = fmaf(t1, q, acc[6]);                      // C4
-        acc[7] = fmaf(t2, p, acc[7]);                      // C5
-        acc[8] = fmaf(q, p, acc[8]);                       // QP
-    };
-    constexpr int EV = 16 / sizeof(InT);
-    int64_t j0 = 0;
-    if ((reinterpret_cast<uintptr_t>(rt) & 15) == 0 && (reinterpret_cast<uintptr_t>(ri) & 15) == 0) {
-        const int64_t nvec = V / EV;
-        const uint4 *vt = reinterpret_cast<const uint4 *>(rt);
-        const uint4 *vi = reinterpret_cast<const uint4 *>(ri);
-        for (int64_t v = threadIdx.x; v < nvec; v += kDiagThreads) {
-            float a[EV], b[EV];
-            unpack(__ldg(vt + v), a);
-            unpack(__ldg(vi + v), b);
-#pragma unroll
-            for (int e = 0; e < EV; ++e)
-                add(a[e], b[e]);
-        }
-        j0 = nvec * EV;
-    }
-    for (int64_t j = j0 + threadIdx.x; j < V; j += kDiagThreads)
-        add(to_f32(rt[j]), to_f32(ri[j]));
-    // block sums in fp64, fixed order
-    double d[kNSums];
-#pragma unroll
-    for (int i = 0; i < kNSums; ++i) {
-        double v = (double)acc[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            v += __shfl_xor_sync(0xffffffffu, v, o);
-        d[i] = v;
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < kNSums; ++i)
-            sh.sums[wid][i] = d[i];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double S[kNSums];
-        for (int i = 0; i < kNSums; ++i) {
-            S[i] = 0.0;
-            for (int w = 0; w < kDiagThreads / 32; ++w)
-                S[i] += sh.sums[w][i];
-        }
-        const double P2 = S[0], R2 = S[1], RP = S[2], C1 = S[3], C2 = S[4], C3 = S[5],
-                     C4 = S[6], C5 = S[7], C6 = C5 + 2.0 * S[8];
-        const double bias2 = R2 - 2.0 * C3 * RP + C3 * C3 * P2;
-        const double dvar = C1 + P2 * C2 - (C4 - (2.0 + C3) * C5 - C3 * C6 + C3 * (2.0 + C3) * P2);
-        if (bias2_out) bias2_out[t] = (float)bias2;
-        if (dvar_out) dvar_out[t] = (float)dvar;
-    }
-}
-
 
 // ---------------------------------------------------------------------------
 // Streaming kernel.
@@ -308,7 +179,7 @@ __device__ __forceinline__ float2 sum8_exp2_pk(uint4 w, float2 noff, float2 acc)
 }
 
 struct DiagArgs {
-    const __nv_bfloat16 *zt, *zi;
+    const void *zt, *zi;
     int64_t T, V, ld_t, ld_i;
     const int32_t *ids;
     const uint8_t *mask;
@@ -316,6 +187,234 @@ struct DiagArgs {
     float *eps, *logk, *p, *bias2, *dvar;
     int32_t *status;
 };
+
+// Masked rows give 0; valid ones with a bad id NaN, and the status bit.
+__device__ __forceinline__ void no_row(const DiagArgs &a, int64_t t, bool valid)
+{
+    const float v = valid ? NAN : 0.0f;
+    if (valid)
+        set_status(a.status, kStatusBadId);
+    a.eps[t] = v;
+    if (a.logk) a.logk[t] = v;
+    if (a.p) a.p[t] = v;
+    if (a.bias2) a.bias2[t] = v;
+    if (a.dvar) a.dvar[t] = v;
+}
+
+// bias2 and dvar from the nine sums in diag_pair's signs.
+__device__ __forceinline__ void finish_sums(const DiagArgs &a, int64_t t,
+                                            const double (&S)[kNSums])
+{
+    const double P2 = S[0], R2 = S[1], RP = -S[2], D = S[3], C2 = -S[4], C3 = -S[5], C4 = -S[6],
+                 C5 = -S[7], QP = S[8];
+    const double C1 = C2 + 2.0 * D, C6 = C5 + 2.0 * QP;
+    const double bias2 = R2 - 2.0 * C3 * RP + C3 * C3 * P2;
+    const double dvar = C1 + P2 * C2 - (C4 - (2.0 + C3) * C5 - C3 * C6 + C3 * (2.0 + C3) * P2);
+    if (a.bias2) a.bias2[t] = (float)bias2;
+    if (a.dvar) a.dvar[t] = (float)dvar;
+}
+
+// ---------------------------------------------------------------------------
+// Split kernel: any type and alignment, and few rows.  A cluster of cs CTAs
+// shares a row; both passes read global memory with aligned 16-byte loads (two
+// vectors of each tensor in flight per thread), the second mostly from L2.  Both
+// rows must start at the same offset from a 16-byte boundary, else they are read
+// entry by entry.  Bound: instruction issue for many rows, as the streaming
+// kernel; the latency of a row for few.  T=2048, V=151935 bf16 takes 465 us against
+// 1068 for the kernel before it (one CTA a row, unaligned rows entry by entry, fp64
+// butterflies for the sums), V=151936 fp32 769 against 816.
+template <int NT> struct SplitShared {
+    MaxSum red[2][NT / 32];
+    MaxSum part[2][kMaxCluster];     // [engine][CTA] this row's pairs, in every CTA
+    double sums[kMaxCluster][kNSums];  // the CTAs' sums, in the first one
+    float wsum[NT / 32][kNSums];
+    float lse[2];
+};
+
+template <typename InT, int MODE, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT)
+    cis_mismatch_split_kernel(const __grid_constant__ DiagArgs a, unsigned cs)
+{
+    constexpr int EV = Vec<InT>::kN, kU = 2;
+    __shared__ SplitShared<NT> sh;
+    const int64_t t = blockIdx.x / cs;
+    const unsigned rank = blockIdx.x - (unsigned)t * cs;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const bool valid = a.mask == nullptr || a.mask[t] != 0;
+    const int64_t y = a.ids[t];
+    if (!valid || y < 0 || y >= a.V) {  // same branch in every CTA of the row
+        if (rank == 0 && tid == 0)
+            no_row(a, t, valid);
+        return;
+    }
+    if (cs > 1)
+        cluster_arrive_relaxed();  // waited for before the first store to a peer
+    const InT *rt = static_cast<const InT *>(a.zt) + t * a.ld_t;
+    const InT *ri = static_cast<const InT *>(a.zi) + t * a.ld_i;
+    const int V = (int)a.V;
+    const bool same = ((reinterpret_cast<uintptr_t>(rt) ^ reinterpret_cast<uintptr_t>(ri)) & 15) == 0;
+    const int head = same ? row_head(rt, V) : 0;
+    const int nvec = same ? (V - head) / EV : 0;
+    const int tail = head + nvec * EV;  // entries [0, head) and [tail, V) one by one
+    const int v0 = (int)((int64_t)nvec * rank / cs), v1 = (int)((int64_t)nvec * (rank + 1) / cs);
+    const uint4 *vt = reinterpret_cast<const uint4 *>(rt + head);
+    const uint4 *vi = reinterpret_cast<const uint4 *>(ri + head);
+    const int nend = head + V - tail;
+    const int yb = (int)y - head;
+    const int vy = yb >= 0 ? yb / EV : -1, iy = yb - vy * EV;
+
+    // pass 1: each engine's (max, sum) over j != y
+    ExpAcc<false> xt, xi;
+    for (int v = v0 + tid; v < v1; v += kU * NT) {
+        Vec<InT> u[kU], w[kU];
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+            const bool in = v + k * NT < v1;
+            const uint4 n4 = make_uint4(Vec<InT>::kNone, Vec<InT>::kNone, Vec<InT>::kNone,
+                                        Vec<InT>::kNone);
+            u[k].q = in ? __ldg(vt + v + k * NT) : n4;
+            w[k].q = in ? __ldg(vi + v + k * NT) : n4;
+        }
+#pragma unroll
+        for (int k = 0; k < kU; ++k)
+            if (v + k * NT == vy) {
+                u[k].drop(iy);
+                w[k].drop(iy);
+            }
+        take<false, kU>(xt, u);
+        take<false, kU>(xi, w);
+    }
+    for (int k = (int)rank * NT + tid; k < nend; k += (int)cs * NT) {
+        const int j = k < head ? k : tail + (k - head);
+        if (j != (int)y) {
+            const float z[2] = {to_f32(rt[j]), to_f32(ri[j])};
+            xt.raise(z[0]);
+            xi.raise(z[1]);
+            if (xt.m != -INFINITY)
+                xt.add_entry(z[0]);
+            if (xi.m != -INFINITY)
+                xi.add_entry(z[1]);
+        }
+    }
+    const MaxSumU bt = xt.result(), bi = xi.result();
+    MaxSum ot = warp_ms(MaxSum{bt.m, bt.s}), oi = warp_ms(MaxSum{bi.m, bi.s});
+    if (lane == 0) {
+        sh.red[0][wid] = ot;
+        sh.red[1][wid] = oi;
+    }
+    __syncthreads();
+    ot = sh.red[0][0];
+    oi = sh.red[1][0];
+#pragma unroll
+    for (int w = 1; w < NT / 32; ++w) {
+        ot = ms_combine(ot, sh.red[0][w]);
+        oi = ms_combine(oi, sh.red[1][w]);
+    }
+    if (cs > 1) {  // every CTA's pairs to every CTA, combined in rank order
+        cluster_wait();
+        if (tid < (int)cs) {
+            const uint32_t d0 = map_rank(smem_u32(&sh.part[0][rank]), tid);
+            const uint32_t d1 = map_rank(smem_u32(&sh.part[1][rank]), tid);
+            asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(d0), "f"(ot.m),
+                         "f"(ot.s)
+                         : "memory");
+            asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(d1), "f"(oi.m),
+                         "f"(oi.s)
+                         : "memory");
+        }
+        __syncwarp();
+        cluster_sync_data();
+        ot = sh.part[0][0];
+        oi = sh.part[1][0];
+        for (unsigned r = 1; r < cs; ++r) {
+            ot = ms_combine(ot, sh.part[0][r]);
+            oi = ms_combine(oi, sh.part[1][r]);
+        }
+    }
+    if (tid == 0) {
+        const float zyt = to_f32(rt[y]), zyi = to_f32(ri[y]);
+        const RowScalars st = row_scalars(ot, zyt), si = row_scalars(oi, zyi);
+        sh.lse[0] = st.lse;
+        sh.lse[1] = si.lse;
+        if (rank == 0) {
+            // eps = logit p - logit q: Lemma 3.1's -delta_y + log sum_{j != y} w_j
+            // e^{delta_j} in the normalised gauge, from the log-odds of each engine
+            const double dp = ((double)zyt - (double)ot.m) - (double)logf(ot.s);
+            const double dq = ((double)zyi - (double)oi.m) - (double)logf(oi.s);
+            a.eps[t] = (float)(dp - dq);
+            if (a.logk) a.logk[t] = (float)(st.lp64() - si.lp64());
+            if (a.p) a.p[t] = expf(st.lp);
+        }
+    }
+    __syncthreads();
+    // pass 2: the sums over every candidate, the exponents in log2 units (one FMA
+    // each); probabilities that flush to 0 add nothing measurable
+    const float op = sh.lse[0] * kLog2e, oq = sh.lse[1] * kLog2e;
+    const float2 nop = make_float2(-op, -op), noq = make_float2(-oq, -oq);
+    float2 acc[kNSums];
+#pragma unroll
+    for (int i = 0; i < kNSums; ++i)
+        acc[i] = make_float2(0.0f, 0.0f);
+    Vec<InT> u, w;  // the next vectors are fetched while these are summed
+    if (v0 + tid < v1) {
+        u.q = __ldg(vt + v0 + tid);
+        w.q = __ldg(vi + v0 + tid);
+    }
+    for (int v = v0 + tid; v < v1; v += NT) {
+        const Vec<InT> x = u, z = w;
+        if (v + NT < v1) {
+            u.q = __ldg(vt + v + NT);
+            w.q = __ldg(vi + v + NT);
+        }
+#pragma unroll
+        for (int i = 0; i < EV; i += 2)
+            diag_pair<MODE>(make_float2(x.entry(i), x.entry(i + 1)),
+                            make_float2(z.entry(i), z.entry(i + 1)), nop, noq, a.P, acc);
+    }
+    for (int k = (int)rank * NT + tid; k < nend; k += (int)cs * NT) {
+        const int j = k < head ? k : tail + (k - head);
+        diag_pair<MODE>(make_float2(to_f32(rt[j]), -INFINITY),
+                        make_float2(to_f32(ri[j]), -INFINITY), nop, noq, a.P, acc);
+    }
+    // warp sums in fp32 (fp64 additions run at 2 a clock and SM), the warps' and
+    // the CTAs' in fp64, in order
+#pragma unroll
+    for (int i = 0; i < kNSums; ++i) {
+        float v = acc[i].x + acc[i].y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0)
+            sh.wsum[wid][i] = v;
+    }
+    __syncthreads();
+    if (tid < kNSums) {
+        double v = sh.wsum[0][tid];
+        for (int w = 1; w < NT / 32; ++w)
+            v += sh.wsum[w][tid];
+        if (cs > 1 && rank != 0) {
+            const uint32_t d = map_rank(smem_u32(&sh.sums[rank][tid]), 0);
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(d), "d"(v) : "memory");
+        } else {
+            sh.sums[0][tid] = v;
+        }
+    }
+    if (cs > 1) {
+        __syncwarp();
+        cluster_sync_data();
+    } else {
+        __syncthreads();
+    }
+    if (rank == 0 && tid == 0) {
+        double S[kNSums];
+        for (int i = 0; i < kNSums; ++i) {
+            S[i] = sh.sums[0][i];
+            for (unsigned r = 1; r < cs; ++r)
+                S[i] += sh.sums[r][i];
+        }
+        finish_sums(a, t, S);
+    }
+}
 
 // The layout for NW consumer warps (plus a producer and an epilogue warp)
 // and CPS CTAs per SM: a ring slot holds four groups per consumer thread of
@@ -525,8 +624,8 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
             const int64_t y = a.ids[t];
             if ((a.mask != nullptr && a.mask[t] == 0) || y < 0 || y >= a.V)
                 continue;
-            const uint8_t *rp = reinterpret_cast<const uint8_t *>(a.zt + t * a.ld_t);
-            const uint8_t *rq = reinterpret_cast<const uint8_t *>(a.zi + t * a.ld_i);
+            const uint8_t *rp = static_cast<const uint8_t *>(a.zt) + t * a.ld_t * 2;
+            const uint8_t *rq = static_cast<const uint8_t *>(a.zi) + t * a.ld_i * 2;
             // Pass 1's bytes are prefetched into L2 kPrefetchSlots slots ahead
             // of their copies: this row's slot st + kPrefetchSlots with
             // pass-1 slot st, and the first slots of this CTA's next row with
@@ -544,9 +643,9 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
                     break;
             }
             const uint8_t *np =
-                tn < a.T ? reinterpret_cast<const uint8_t *>(a.zt + tn * a.ld_t) : nullptr;
+                tn < a.T ? static_cast<const uint8_t *>(a.zt) + tn * a.ld_t * 2 : nullptr;
             const uint8_t *nq =
-                tn < a.T ? reinterpret_cast<const uint8_t *>(a.zi + tn * a.ld_i) : nullptr;
+                tn < a.T ? static_cast<const uint8_t *>(a.zi) + tn * a.ld_i * 2 : nullptr;
             for (int pass = 0; pass < 2 && !ab.on(); ++pass)
                 for (int st = 0; st < nst; ++st, ++k) {
                     const uint32_t s = k % kRing, u = k / kRing;
@@ -629,14 +728,7 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
                 a.eps[t] = (float)(dp - dq);
                 if (a.logk) a.logk[t] = (float)(rs.lp64() - lp64_q);
                 if (a.p) a.p[t] = expf(rs.lp);
-                const double P2 = S[0], R2 = S[1], RP = -S[2], D = S[3], C2 = -S[4], C3 = -S[5],
-                             C4 = -S[6], C5 = -S[7], QP = S[8];
-                const double C1 = C2 + 2.0 * D, C6 = C5 + 2.0 * QP;
-                const double bias2 = R2 - 2.0 * C3 * RP + C3 * C3 * P2;
-                const double dvar =
-                    C1 + P2 * C2 - (C4 - (2.0 + C3) * C5 - C3 * C6 + C3 * (2.0 + C3) * P2);
-                if (a.bias2) a.bias2[t] = (float)bias2;
-                if (a.dvar) a.dvar[t] = (float)dvar;
+                finish_sums(a, t, S);
             }
             ++rr;
         }
@@ -650,16 +742,8 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
         const bool valid = a.mask == nullptr || a.mask[t] != 0;
         const int64_t y = a.ids[t];
         if (!valid || y < 0 || y >= a.V) {
-            if (ct == 0) {
-                const float v = valid ? NAN : 0.0f;
-                if (valid)
-                    set_status(a.status, kStatusBadId);
-                a.eps[t] = v;
-                if (a.logk) a.logk[t] = v;
-                if (a.p) a.p[t] = v;
-                if (a.bias2) a.bias2[t] = v;
-                if (a.dvar) a.dvar[t] = v;
-            }
+            if (ct == 0)
+                no_row(a, t, valid);
             continue;
         }
         const int b = rr & 1;
@@ -667,7 +751,8 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
         // training row's, lane 16 the inference row's
         float zy = 0.0f;
         if ((lane & 15) == 0)
-            zy = to_f32(lane == 0 ? a.zt[t * a.ld_t + y] : a.zi[t * a.ld_i + y]);
+            zy = to_f32(lane == 0 ? static_cast<const __nv_bfloat16 *>(a.zt)[t * a.ld_t + y]
+                                  : static_cast<const __nv_bfloat16 *>(a.zi)[t * a.ld_i + y]);
         const int gy = (int)(y >> 3), iy = (int)(y & 7);
 
         // pass 1
@@ -837,16 +922,26 @@ int diag_warps()
     return (v == 24 || v == 8 || v == 4) ? v : 16;
 }
 
-bool diag_stream_applies(const void *zt, const void *zi, int dtype, int64_t V, int64_t ld_t,
-                         int64_t ld_i)
+// The streaming kernel gives an SM whole rows, one at a time: it is the better one
+// for long rows (T=4096, V=151936: 717 us against 891 for the split kernel; T=100:
+// 32 against 39) but for a few very long ones (T=48: 31.2 against 25.7), and for
+// short rows while each SM has one (T=60, V=16000: 9.9 against 11.5; T=400: 20.6
+// against 15.7).  CIS_DIAG_KERNEL=row (stream) forces the split (streaming) kernel
+// where both apply, and the streaming kernel's tuning variables imply it.
+bool diag_stream_applies(const DiagArgs &a, int dtype)
 {
-    if (dtype != CIS_BF16 || V % 8 != 0)
+    if (dtype != CIS_BF16 || a.V % 8 != 0)
         return false;
-    if ((reinterpret_cast<uintptr_t>(zt) & 15) || (reinterpret_cast<uintptr_t>(zi) & 15) ||
-        (ld_t * 2) % 16 || (ld_i * 2) % 16)
+    if ((reinterpret_cast<uintptr_t>(a.zt) & 15) || (reinterpret_cast<uintptr_t>(a.zi) & 15) ||
+        (a.ld_t * 2) % 16 || (a.ld_i * 2) % 16)
         return false;
     const char *e = getenv("CIS_DIAG_KERNEL");
-    return !(e && e[0] == 'r');
+    if (e && (e[0] == 'r' || e[0] == 's'))
+        return e[0] == 's';
+    if (getenv("CIS_DIAG_SLOT_GROUPS") || getenv("CIS_DIAG_WARPS"))
+        return true;
+    const int64_t nvec = a.V / 8;
+    return nvec > 2048 ? a.T >= 64 || nvec < 8192 : a.T <= 152;
 }
 
 template <int MODE, int NW, int CPS>
@@ -882,15 +977,52 @@ cudaError_t launch_stream_mode(const DiagArgs &a, cudaStream_t s)
 // ---------------------------------------------------------------------------
 // Dispatch on the operator (a template parameter of both kernels).
 
-template <typename InT, int MODE>
-void launch_mode(const void *zt, const void *zi, int64_t T, int64_t V, int64_t ld_t,
-                 int64_t ld_i, const int32_t *ids, const uint8_t *mask, const DevParams &P,
-                 float *eps, float *logk, float *p, float *bias2, float *dvar, int32_t *status,
-                 cudaStream_t s)
+// The split kernel's CTAs per row and their width.
+// - 128 threads for rows that 512 would not give four vectors each (eight rows an
+//   SM hide one another's latencies: T=3710, V=2488 bf16 takes 29.4 us against
+//   107, T=8192, V=4001 fp32 82 against 252), and up to twice that length with rows
+//   enough for every place (T=4096, V=32003: 196 against 265).
+// - Few rows are shared by clusters while those leave two CTAs an SM at most, a CTA
+//   keeping 512 vectors (T=24, V=151936: 21.5 us against 30.9 for one CTA a row of the
+//   streaming kernel; four CTAs an SM 21.5, but 65 against 44 at T=152).
+struct DiagSplit {
+    unsigned cs;
+    int nt;
+};
+DiagSplit diag_split(int64_t T, int64_t V, int bytes, int sms)
 {
-    cis_mismatch_kernel<InT, MODE><<<(unsigned)T, kDiagThreads, 0, s>>>(
-        static_cast<const InT *>(zt), static_cast<const InT *>(zi), T, V, ld_t, ld_i, ids, mask,
-        P, eps, logk, p, bias2, dvar, status);
+    const int64_t nvec = V * bytes / 16;
+    const bool narrow = nvec <= 2048 || (nvec <= 4096 && T >= 8 * (int64_t)sms);
+    DiagSplit d{1, narrow ? 128 : kDiagThreads};
+    while (d.cs < kMaxCluster && nvec / (2 * d.cs) >= 512 && T * d.cs * 2 <= 2 * (int64_t)sms)
+        d.cs *= 2;
+    return d;
+}
+
+template <typename InT, int MODE> cudaError_t launch_split(const DiagArgs &a, cudaStream_t s)
+{
+    int dev = 0, sms = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return e;
+    const DiagSplit d = diag_split(a.T, a.V, (int)sizeof(InT), sms);
+    const unsigned cs = d.cs;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.T * cs), 1, 1);
+    cfg.blockDim = dim3((unsigned)d.nt, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cs > 1 ? 1 : 0;
+    return d.nt == 128
+               ? cudaLaunchKernelEx(&cfg, cis_mismatch_split_kernel<InT, MODE, 128>, a, cs)
+               : cudaLaunchKernelEx(&cfg, cis_mismatch_split_kernel<InT, MODE, kDiagThreads>, a,
+                                    cs);
 }
 
 #define CIS_DIAG_MODES(X)  \
@@ -901,22 +1033,13 @@ void launch_mode(const void *zt, const void *zi, int64_t T, int64_t V, int64_t l
     X(CIS_MODE_ICEPOP)     \
     X(CIS_MODE_KPOP)
 
-template <typename InT>
-void launch_type(const void *zt, const void *zi, int64_t T, int64_t V, int64_t ld_t,
-                 int64_t ld_i, const int32_t *ids, const uint8_t *mask, const DevParams &P,
-                 float *eps, float *logk, float *p, float *bias2, float *dvar, int32_t *status,
-                 cudaStream_t s)
+template <typename InT> cudaError_t launch_split_type(const DiagArgs &a, cudaStream_t s)
 {
-#define CIS_DIAG_CASE(M)                                                                          \
-    case M:                                                                                      \
-        launch_mode<InT, M>(zt, zi, T, V, ld_t, ld_i, ids, mask, P, eps, logk, p, bias2, dvar,    \
-                            status, s);                                                          \
-        break;
-    switch (P.mode) {
+#define CIS_DIAG_CASE(M) \
+    case M: return launch_split<InT, M>(a, s);
+    switch (a.P.mode) {
         CIS_DIAG_MODES(CIS_DIAG_CASE)
-    default:
-        launch_mode<InT, CIS_MODE_NONE>(zt, zi, T, V, ld_t, ld_i, ids, mask, P, eps, logk, p,
-                                        bias2, dvar, status, s);
+    default: return launch_split<InT, CIS_MODE_NONE>(a, s);
     }
 #undef CIS_DIAG_CASE
 }
@@ -942,19 +1065,11 @@ cudaError_t launch_mismatch(const void *zt, const void *zi, int dtype, int64_t T
 {
     if (T == 0)
         return cudaSuccess;
-    if (diag_stream_applies(zt, zi, dtype, V, ld_t, ld_i)) {
-        const DiagArgs a{static_cast<const __nv_bfloat16 *>(zt),
-                         static_cast<const __nv_bfloat16 *>(zi),
-                         T, V, ld_t, ld_i, ids, mask, P, eps, logk, p, bias2, dvar, status};
+    const DiagArgs a{zt, zi, T, V, ld_t, ld_i, ids, mask, P, eps, logk, p, bias2, dvar, status};
+    if (diag_stream_applies(a, dtype))
         return launch_stream(a, s);
-    }
-    if (dtype == CIS_BF16)
-        launch_type<__nv_bfloat16>(zt, zi, T, V, ld_t, ld_i, ids, mask, P, eps, logk, p, bias2,
-                                   dvar, status, s);
-    else
-        launch_type<float>(zt, zi, T, V, ld_t, ld_i, ids, mask, P, eps, logk, p, bias2, dvar,
-                           status, s);
-    return cudaGetLastError();
+    return dtype == CIS_BF16 ? launch_split_type<__nv_bfloat16>(a, s)
+                             : launch_split_type<float>(a, s);
 }
 
 }  // namespace cis

@@ -81,6 +81,13 @@ __device__ __forceinline__ void cluster_wait()
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
 
+// Every thread of the cluster, with the stores before it visible after it.
+__device__ __forceinline__ void cluster_sync_data()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // 8 consecutive entries from shared memory as floats.
 template <typename InT> __device__ __forceinline__ void load8(const uint8_t *sm, int g,
                                                               float (&z)[8]);

@@ -1,0 +1,197 @@
+// cis_expacc.cuh -- sums of exponentials over one row read straight into
+// registers with aligned 16-byte loads (the forward kernel, the diagnostics).
+//
+// Per batch of vectors a thread takes one maximum (bf16 entries compared in
+// pairs), moves its offset at most once, and then spends per entry an unpack,
+// half a packed FMA, an exponential and half a packed add:
+//   S = sum 2^{z log2e - c},  c = fl(m log2e),
+// the rounding residual of c being taken out once at the end.
+#pragma once
+
+#include "cis_common.cuh"
+
+namespace cis {
+namespace {
+
+// Running (m, S[, U]) of one thread in the exponent form above; U = sum e x with
+// x = z log2e - c.  With |m| >= kHugeLogit x = (z - m) log2e and c is not used.
+template <bool kEnt> struct ExpAcc {
+    float m = -INFINITY, c = -INFINITY, S = 0.0f, U = 0.0f;
+
+    __device__ __forceinline__ bool fast() const { return fabsf(m) < kHugeLogit; }
+    // Raise the offset to a larger (or NaN) maximum.
+    __device__ __forceinline__ void raise(float mx)
+    {
+        if (mx > m || mx != mx) {
+            const float c1 = mx * kLog2e;
+            const float d = fast() && fabsf(mx) < kHugeLogit ? c - c1 : (m - mx) * kLog2e;
+            const float f = ex2_ftz(d);
+            if (kEnt)
+                U = f == 0.0f ? 0.0f : fmaf(d, S, U) * f;
+            S = f == 0.0f ? 0.0f : S * f;
+            m = mx;
+            c = c1;
+        }
+    }
+    // Add 8 entries (those left out are -inf); the offset covers them.
+    __device__ __forceinline__ void add8(const float2 (&z)[4])
+    {
+        const float2 l2 = make_float2(kLog2e, kLog2e), nc = make_float2(-c, -c);
+        float2 e[4], u = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 x = __ffma2_rn(z[i], l2, nc);
+            e[i] = make_float2(ex2_ftz(x.x), ex2_ftz(x.y));
+            if (kEnt)  // an entry at -inf adds 0, not 0 * -inf
+                u = __ffma2_rn(e[i], make_float2(fmaxf(x.x, -1024.0f), fmaxf(x.y, -1024.0f)), u);
+        }
+        const float2 s = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
+        S += s.x + s.y;
+        if (kEnt)
+            U += u.x + u.y;
+    }
+    // One entry, covered by the offset, in either form.
+    __device__ __forceinline__ void add_entry(float z)
+    {
+        const float x = fast() ? fmaf(z, kLog2e, -c) : (z - m) * kLog2e, e = ex2_ftz(x);
+        S += e;
+        if (kEnt)
+            U = fmaf(e, fmaxf(x, -1024.0f), U);
+    }
+    // As sums of e^{z - m}: the residual of c is exact (an FMA).
+    __device__ __forceinline__ MaxSumU result() const
+    {
+        if (m == -INFINITY)
+            return {m, 0.0f, 0.0f};
+        const float err = fast() ? fmaf(m, kLog2e, -c) : 0.0f, f = ex2_ftz(-err);
+        return {m, S * f, kEnt ? f * kLn2 * fmaf(-err, S, U) : 0.0f};
+    }
+};
+
+// One 16-byte vector: 8 bf16 or 4 fp32 entries.
+template <typename InT> struct Vec;
+template <> struct Vec<__nv_bfloat16> {
+    static constexpr int kN = 8;
+    static constexpr uint32_t kNone = 0xff80ff80u;  // entries at -inf
+    uint4 q;
+    __device__ __forceinline__ float entry(int i) const
+    {
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+        return (i & 1) ? bf16_hi(w[i >> 1]) : bf16_lo(w[i >> 1]);
+    }
+    __device__ __forceinline__ void drop(int i)  // entry i to -inf
+    {
+        uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((i >> 1) == k)
+                w[k] = (i & 1) ? (w[k] & 0x0000ffffu) | 0xff800000u
+                               : (w[k] & 0xffff0000u) | 0x0000ff80u;
+        q = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+};
+template <> struct Vec<float> {
+    static constexpr int kN = 4;
+    static constexpr uint32_t kNone = 0xff800000u;
+    uint4 q;
+    __device__ __forceinline__ float entry(int i) const
+    {
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+        return __uint_as_float(w[i]);
+    }
+    __device__ __forceinline__ void drop(int i)
+    {
+        const uint32_t ninf = 0xff800000u;
+        q.x = i == 0 ? ninf : q.x;
+        q.y = i == 1 ? ninf : q.y;
+        q.z = i == 2 ? ninf : q.z;
+        q.w = i == 3 ? ninf : q.w;
+    }
+};
+
+__device__ __forceinline__ __nv_bfloat162 as_bf2(uint32_t w)
+{
+    return *reinterpret_cast<const __nv_bfloat162 *>(&w);
+}
+
+// Maximum of N vectors (NaN propagates).
+template <int N> __device__ __forceinline__ float vec_max(const Vec<__nv_bfloat16> (&v)[N])
+{
+    __nv_bfloat162 a = __hmax2_nan(as_bf2(v[0].q.x), as_bf2(v[0].q.y));
+    __nv_bfloat162 b = __hmax2_nan(as_bf2(v[0].q.z), as_bf2(v[0].q.w));
+#pragma unroll
+    for (int k = 1; k < N; ++k) {
+        a = __hmax2_nan(a, __hmax2_nan(as_bf2(v[k].q.x), as_bf2(v[k].q.y)));
+        b = __hmax2_nan(b, __hmax2_nan(as_bf2(v[k].q.z), as_bf2(v[k].q.w)));
+    }
+    a = __hmax2_nan(a, b);
+    return max_nan(__low2float(a), __high2float(a));
+}
+template <int N> __device__ __forceinline__ float vec_max(const Vec<float> (&v)[N])
+{
+    float m = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        m = max_nan(m, max_nan(__uint_as_float(v[k].q.x), __uint_as_float(v[k].q.y)));
+        m = max_nan(m, max_nan(__uint_as_float(v[k].q.z), __uint_as_float(v[k].q.w)));
+    }
+    return m;
+}
+
+template <bool kEnt, int N>
+__device__ __forceinline__ void add_vecs(ExpAcc<kEnt> &acc, const Vec<__nv_bfloat16> (&v)[N])
+{
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const uint4 q = v[k].q;
+        const float2 z[4] = {make_float2(bf16_lo(q.x), bf16_hi(q.x)),
+                             make_float2(bf16_lo(q.y), bf16_hi(q.y)),
+                             make_float2(bf16_lo(q.z), bf16_hi(q.z)),
+                             make_float2(bf16_lo(q.w), bf16_hi(q.w))};
+        acc.add8(z);
+    }
+}
+template <bool kEnt, int N>
+__device__ __forceinline__ void add_vecs(ExpAcc<kEnt> &acc, const Vec<float> (&v)[N])
+{
+    const float2 none = make_float2(-INFINITY, -INFINITY);
+#pragma unroll
+    for (int k = 0; k < N; k += 2) {
+        const uint4 a = v[k].q, b = v[k + 1 < N ? k + 1 : k].q;
+        const float2 z[4] = {make_float2(__uint_as_float(a.x), __uint_as_float(a.y)),
+                             make_float2(__uint_as_float(a.z), __uint_as_float(a.w)),
+                             k + 1 < N ? make_float2(__uint_as_float(b.x), __uint_as_float(b.y))
+                                       : none,
+                             k + 1 < N ? make_float2(__uint_as_float(b.z), __uint_as_float(b.w))
+                                       : none};
+        acc.add8(z);
+    }
+}
+
+template <bool kEnt, int N, typename InT>
+__device__ __forceinline__ void take(ExpAcc<kEnt> &acc, const Vec<InT> (&v)[N])
+{
+    acc.raise(vec_max<N>(v));
+    if (acc.fast()) {
+        add_vecs<kEnt, N>(acc, v);
+    } else if (acc.m != -INFINITY) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int i = 0; i < Vec<InT>::kN; ++i)
+                acc.add_entry(v[k].entry(i));
+    }
+}
+
+// Where row's 16-byte vectors lie: the entries before the first whole one, and
+// the number of whole ones.
+template <typename InT>
+__device__ __forceinline__ int row_head(const InT *row, int V)
+{
+    const int head =
+        (int)((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) / (int)sizeof(InT);
+    return head < V ? head : V;
+}
+
+}  // namespace
+}  // namespace cis

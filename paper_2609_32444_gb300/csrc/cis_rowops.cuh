@@ -1,6 +1,5 @@
-// cis_rowops.cuh -- row-streaming building blocks shared by the row kernels
-// (cis_rowwise.cu) and the mismatch diagnostics (cis_diag.cu): a running
-// (max, sum of exponentials) -- optionally with the entropy term -- over the
+// cis_rowops.cuh -- row-streaming building blocks of the row kernel
+// (cis_rowwise.cu): a running (max, sum of exponentials) -- optionally with the entropy term -- over the
 // entries j != y of one row, read with 16-byte vector loads.
 #pragma once
 
