@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     // Per-token inputs, fetched while the copy is in flight.
     // The weight is known here where it does not depend on the row (l_old, or a
     // sequence operator's weight).
-    float zy = 0.0f, linf = 0.0f, lold = 0.0f, adv = 0.0f, sc = 0.0f, qinv = 0.0f, oinv = 0.0f;
+    float zy = 0.0f, linf = 0.0f, lold = 0.0f, adv = 0.0f, sc = 0.0f, qinv = 0.0f, qinv_lo = 0.0f;
     TokenWeight tw{0.0f, 0.0f, 0};
     KpopSide kq{0.0f, 0.0f, 0.0f, 0.0f};
     constexpr bool kAll = kOps == Ops::kAll;
@@ -295,10 +295,17 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         qinv = expf(-linf);  // 1 / q, off the row's serial path
         if (has_old) {
             lold = a.lp_old[t];
-            oinv = expf(-lold);
             tw = token_weight<kAll>(lold, 0.0f, linf, a.P);
-        } else if (kAll && a.P.mode == CIS_MODE_KPOP) {
-            kq = kpop_side(linf);
+        } else if (kAll) {
+            // 1 / q as a pair: q as one, its reciprocal's residual from FMAs
+            float ql;
+            const float qh = exp_pair(linf, 0.0f, ql);
+            if (qh > 0.0f && linf >= -70.0f) {
+                qinv = 1.0f / qh;
+                qinv_lo = -qinv * fmaf(ql, qinv, fmaf(qh, qinv, -1.0f));
+            }
+            if (a.P.mode == CIS_MODE_KPOP)
+                kq = kpop_side(linf);
         }
         // the workspace is the kernel before's until it has ended; with the
         // launch gaps that saves 6 us of 94 at T=4096, V=32000
@@ -388,13 +395,13 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     // Thread 0 forms the row's scalars: the serial part of every row, which
     // the other threads wait for, and which shares the SM's issue slots with
     // the other CTAs' streaming loops, so its instruction count sets its
-    // length.  In the common case (row_direct) the weight and the update ratio
-    // come from the row's statistics without logarithms, and log p, log k and
-    // the fp64 loss term are formed after the barrier by rank 0 alone, which
-    // stores them.  Otherwise the log-domain path forms everything here.
+    // length.  Without l_old the weight comes from the row's statistics without
+    // logarithms (row_direct) in the common case, and log p, log k and the fp64
+    // loss term are formed after the barrier by rank 0 alone, which stores them.
+    // Otherwise the log-domain path forms everything here.
     MaxSumU ou{0.0f, 0.0f, 0.0f};
     double term = 0.0;
-    float lp = 0.0f, tdir = 0.0f, obj = adv;  // obj: min(rho A, clip(rho) A)
+    float lp = 0.0f, tdir = 0.0f;
     bool direct = false;
     if (threadIdx.x == 0) {
         MaxSum o;
@@ -406,19 +413,13 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         }
         float c, omp, bias_log2, scale = 1.0f;
         DirectRow dw;
-        direct = row_direct(o, zy, dw);
-        if (direct && !has_old && !given)
-            direct = weight_direct<kAll>(dw, linf, qinv, kq, a.P, tw.w, tw.trunc);
-        float rho = 1.0f;
-        bool flows = true;  // the clip leaves the gradient
-        if (direct && has_old)
-            direct = ratio_direct(dw, lold, oinv, adv, a.P, rho, flows);
+        direct = !has_old && row_direct(o, zy, dw);
+        if (direct && !given)
+            direct = weight_direct<kAll>(dw, linf, qinv, qinv_lo, kq, a.P, tw.w, tw.trunc);
         if (direct) {
             omp = dw.omp;
             tdir = dw.t;
-            if (has_old)
-                obj = (flows ? rho : fminf(fmaxf(rho, a.P.rho_lo_f), a.P.rho_hi_f)) * adv;
-            c = flows ? sc * tw.w * adv * rho : 0.0f;  // s w A rho g
+            c = sc * tw.w * adv;  // s w A rho with rho = 1, g = 1 (Eq. 1 without l_old)
             // The softmax's 1 / (s' + e^{z_y - m'}) = e^{m' - z_y} p, in
             // [2^-102, 1] within the closed forms' range, replaces a logarithm:
             // its binary exponent -J goes into the exponent offset (as the
@@ -480,9 +481,8 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     if (threadIdx.x == 0 && rank == 0) {
         if (direct) {  // log p, log k and the loss term, off the serial path
             lp = -log1pf(tdir);  // p = 1 / (1 + t)
-            if (!has_old)
-                tw.logk = lp - linf;
-            term = -(double)sc * (double)tw.w * (double)obj;
+            tw.logk = lp - linf;
+            term = -(double)sc * (double)tw.w * (double)adv;
         }
         if (a.lp_out) a.lp_out[t] = lp;
         if (a.w_out) a.w_out[t] = tw.w;

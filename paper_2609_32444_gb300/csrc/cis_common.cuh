@@ -577,10 +577,9 @@ __device__ __forceinline__ MaxSumU block_msu(MaxSumU v, MaxSumU *sh)
 // The row's probabilities straight from its statistics, without logarithms.
 // From (m', s') over j != y and z_y, with t = s' e^{m' - z_y} = (1 - p) / p:
 //   p = 1 / (1 + t),   1 - p = t p,
-// each within ~8 ulp (expf, __fdividef: 2 ulp each), so that k = p e^{-l_inf}
-// and rho = p e^{-l_old} (the exponentials formed ahead of time) and the bounds
-// they are compared with carry relative errors near 2e-6, inside certain_cmp's
-// 4e-6 (a + b).  False where these forms would leave the normal fp32 range
+// each within ~8 ulp (expf, __fdividef: 2 ulp each), so that k = p e^{-l_inf} (the
+// exponential formed ahead of time) and the bounds it is compared with carry
+// relative errors near 2e-6, inside certain_cmp's 4e-6 (a + b).  False where these forms would leave the normal fp32 range
 // (|m' - z_y| > 70, an empty or non-finite row): the caller then takes the
 // log-domain path (row_scalars, token_weight, token_loss), as it does where a
 // decision is too close to call; that path's fp64 fallback settles it.
@@ -605,17 +604,19 @@ __device__ __forceinline__ bool row_direct(MaxSum o, float zy, DirectRow &r)
 }
 
 // The weight with the current log p as l_w (no l_old, no sequence weight); qinv
-// is e^{-l_inf}.  kAll as in token_weight.  False where a decision is too close
+// (+ qinv_lo with kAll) is e^{-l_inf}.  kAll as in token_weight.  False where a decision is too close
 // to call, l_inf < -70, or the band's bounds are taken (they are rounded once,
 // from pairs, by token_weight).
 template <bool kAll>
 __device__ __forceinline__ bool weight_direct(const DirectRow &d, float linf, float qinv,
-                                              const KpopSide &kq, const DevParams &P, float &w,
-                                              uint8_t &trunc)
+                                              float qinv_lo, const KpopSide &kq,
+                                              const DevParams &P, float &w, uint8_t &trunc)
 {
     if (!(linf >= -70.0f))
         return false;
-    const float k = d.p * qinv;
+    // the other operators' weights come from log k, rounded less often than
+    // p / q: 1 / q as a pair makes up for it
+    const float k = kAll ? fmaf(d.p, qinv, d.p * qinv_lo) : d.p * qinv;
     trunc = 0;
     w = k;
     switch (P.mode) {
@@ -675,18 +676,6 @@ __device__ __forceinline__ bool weight_direct(const DirectRow &d, float linf, fl
     return false;
 }
 
-// rho = exp(l - l_old) and whether the PPO clip leaves the gradient (Eq. 1);
-// oinv is e^{-l_old}.  False where that is too close to call or l_old < -70.
-__device__ __forceinline__ bool ratio_direct(const DirectRow &d, float lold, float oinv, float A,
-                                             const DevParams &P, float &rho, bool &g)
-{
-    rho = d.p * oinv;
-    const int s = A > 0.0f ? certain_cmp(P.rho_hi_f, rho)
-                           : (A < 0.0f ? certain_cmp(rho, P.rho_lo_f) : 1);
-    g = s > 0;
-    return s != 0 && lold >= -70.0f && A == A;
-}
-
 // Per-row scalars from (m', s') over j != y and z_y.  With the log-odds
 //   d = z_y - log sum_{j != y} e^{z_j} = (z_y - m') - log s',
 // log p = -softplus(-d) is accurate for p near 0 and near 1 (Sec. 3.3 notes
@@ -705,7 +694,20 @@ struct RowScalars {
     __device__ __forceinline__ double lp64() const { return (double)lp + (double)lp_lo; }
 };
 
-__device__ __forceinline__ RowScalars row_scalars(MaxSum o, float zy)
+// log s - ls for ls near log s, from e^{-ls} as a pair: s e^{-ls} - 1.
+__device__ __forceinline__ float log_residual(float s, float ls)
+{
+    if (!(ls >= 0.0f && ls < 79.0f))
+        return 0.0f;
+    float el;
+    const float eh = exp_pair(-ls, 0.0f, el);
+    const float p = s * eh;
+    return (p - 1.0f) + (fmaf(s, eh, -p) + s * el);
+}
+
+// exact_log: log s' as a pair too (its fp32 rounding, up to half an ulp of 12, is
+// the largest error of log p where tokens' log p are added up).
+__device__ __forceinline__ RowScalars row_scalars(MaxSum o, float zy, bool exact_log = false)
 {
     RowScalars r;
     if (o.m == -INFINITY && o.s == 0.0f) {
@@ -722,6 +724,8 @@ __device__ __forceinline__ RowScalars row_scalars(MaxSum o, float zy)
     const float dh = two_sum(zy, -o.m, dl);          // z_y - m' = dh + dl exactly
     const float ls = logf(o.s);
     const float u = two_sum(dh, -ls, ue);            // dh - ls = u + ue exactly
+    if (exact_log)
+        ue -= log_residual(o.s, ls);
     const float d = u + (ue + dl);                   // logit p
     float lse_m;                                     // lse - m'
     // 1 - p = sigmoid(-d): e^{-d} / (1 + e^{-d}) for d > 0, 1 / (1 + e^d)

@@ -4,14 +4,27 @@
 // Per batch of vectors a thread takes one maximum (bf16 entries compared in
 // pairs), moves its offset at most once, and then spends per entry an unpack,
 // half a packed FMA, an exponential and half a packed add:
-//   S = sum 2^{z log2e - c},  c = fl(m log2e),
-// the rounding residual of c being taken out once at the end.
+//   S = sum 2^{z log2e - c},  c = ceil(m log2e),
+// with whole c, so that sums move between offsets by exact powers of two: the
+// exponential instruction's error is one-sided (-4.9e-8 on average, measured), and a
+// term that is rescaled on its way through threads and warps by it picks that up
+// several times, the same way in every row.
 #pragma once
 
 #include "cis_common.cuh"
 
 namespace cis {
 namespace {
+
+// 2^x for 0 <= x < 1, to fp32 rounding.
+__device__ __forceinline__ float exp2_accurate(float x)
+{
+    constexpr float ln2_lo = (float)(0.693147180559945309417 - (double)kLn2);
+    const float y = x - 1.0f, h = y * kLn2;  // exact, then 2^x = 2 e^{y ln 2}
+    float lo;
+    const float hi = exp_pair(h, fmaf(y, kLn2, -h) + y * ln2_lo, lo);
+    return 2.0f * (hi + lo);
+}
 
 // Running (m, S[, U]) of one thread in the exponent form above; U = sum e x with
 // x = z log2e - c.  With |m| >= kHugeLogit x = (z - m) log2e and c is not used.
@@ -23,7 +36,7 @@ template <bool kEnt> struct ExpAcc {
     __device__ __forceinline__ void raise(float mx)
     {
         if (mx > m || mx != mx) {
-            const float c1 = mx * kLog2e;
+            const float c1 = ceilf(mx * kLog2e);
             const float d = fast() && fabsf(mx) < kHugeLogit ? c - c1 : (m - mx) * kLog2e;
             const float f = ex2_ftz(d);
             if (kEnt)
@@ -58,15 +71,79 @@ template <bool kEnt> struct ExpAcc {
         if (kEnt)
             U = fmaf(e, fmaxf(x, -1024.0f), U);
     }
-    // As sums of e^{z - m}: the residual of c is exact (an FMA).
+    // As sums of e^{z - m}: m log2e - c is exact (an FMA), between -1 and 0 but
+    // for its rounding.
     __device__ __forceinline__ MaxSumU result() const
     {
         if (m == -INFINITY)
             return {m, 0.0f, 0.0f};
-        const float err = fast() ? fmaf(m, kLog2e, -c) : 0.0f, f = ex2_ftz(-err);
+        const float err = fast() ? fminf(fmaf(m, kLog2e, -c), 0.0f) : 0.0f;
+        const float f = fast() ? exp2_accurate(-err) : 1.0f;
         return {m, S * f, kEnt ? f * kLn2 * fmaf(-err, S, U) : 0.0f};
     }
 };
+
+// The CTA's threads' sums together, as sums of e^{z - m}; every thread gets them.
+// red: NT / 32 slots.
+template <int NT, bool kEnt>
+__device__ __forceinline__ MaxSumU block_exp(const ExpAcc<kEnt> &acc, MaxSumU *red)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    float M = acc.m;  // (a NaN is kept by its thread's sum)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    if (lane == 0)
+        red[wid].m = M;
+    __syncthreads();
+    M = red[0].m;
+#pragma unroll
+    for (int w = 1; w < NT / 32; ++w)
+        M = fmaxf(M, red[w].m);
+    ExpAcc<kEnt> all;
+    all.m = M;
+    all.c = ceilf(M * kLog2e);
+    if (M == -INFINITY)
+        all.c = 0.0f;  // no entry: every sum is 0, or NaN
+    // This thread's sums at the common offset: an exact power of two where both are
+    // fast; a thread whose entries are all masked ones counts as 0.
+    MaxSumU t = acc.result();
+    float d, f;
+    if (all.fast()) {
+        d = acc.fast() ? acc.c - all.c : (acc.m - M) * kLog2e;
+        t.s = acc.S;
+        t.u = acc.U;
+    } else {
+        d = acc.m == -INFINITY ? -INFINITY : (acc.m - M) * kLog2e;
+        t.u *= kLog2e;
+    }
+    f = ex2_ftz(d);
+    float s = t.s * f, u = kEnt ? fmaf(fmaxf(d, -1e30f), t.s, t.u) * f : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (kEnt)
+            u += __shfl_xor_sync(0xffffffffu, u, o);
+    }
+    if (lane == 0) {
+        red[wid].s = s;
+        red[wid].u = u;
+    }
+    __syncthreads();
+    all.S = red[0].s;
+    all.U = red[0].u;
+#pragma unroll
+    for (int w = 1; w < NT / 32; ++w) {
+        all.S += red[w].s;
+        all.U += red[w].u;
+    }
+    if (M == -INFINITY)
+        return {M, all.S, all.U};
+    MaxSumU o = all.result();
+    if (!all.fast() && kEnt)
+        o.u = all.U * kLn2;
+    return o;
+}
 
 // One 16-byte vector: 8 bf16 or 4 fp32 entries.
 template <typename InT> struct Vec;

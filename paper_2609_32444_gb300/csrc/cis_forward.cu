@@ -27,8 +27,7 @@ constexpr int kBatch = 4;  // 16-byte loads in flight per thread
 
 template <bool kEnt, int NT> struct FwdShared {
     MaxSumU part[kMaxCluster];  // the cluster's CTAs, in its first CTA
-    MaxSumU redu[kEnt ? NT / 32 : 1];
-    MaxSum red[kEnt ? 1 : NT / 32];
+    MaxSumU red[NT / 32];
 };
 
 // A cluster of `cs` CTAs per row.
@@ -109,13 +108,7 @@ __global__ void __launch_bounds__(NT) cis_logprob_kernel(const PassArgs a, unsig
                 acc.add_entry(z);
         }
     }
-    MaxSumU o = acc.result();
-    if constexpr (kEnt) {
-        o = block_msu<NT, false>(o, sh.redu);
-    } else {
-        const MaxSum ms = block_ms<NT, false>(MaxSum{o.m, o.s}, sh.red);
-        o = MaxSumU{ms.m, ms.s, 0.0f};
-    }
+    MaxSumU o = block_exp<NT>(acc, sh.red);
     if (cs > 1) {
         cluster_wait();  // every CTA of the row has started
         if (tid == 0) {
@@ -129,20 +122,20 @@ __global__ void __launch_bounds__(NT) cis_logprob_kernel(const PassArgs a, unsig
         if (rank != 0)
             return;
         if (tid == 0) {  // in rank order
-            o = sh.part[0];
-            for (unsigned r = 1; r < cs; ++r) {
-                if constexpr (kEnt) {
-                    o = msu_combine(o, sh.part[r]);
-                } else {
-                    const MaxSum ms = ms_combine(MaxSum{o.m, o.s},
-                                                 MaxSum{sh.part[r].m, sh.part[r].s});
-                    o = MaxSumU{ms.m, ms.s, 0.0f};
-                }
+            float M = sh.part[0].m;
+            for (unsigned r = 1; r < cs; ++r)
+                M = fmaxf(M, sh.part[r].m);
+            o = MaxSumU{M, 0.0f, 0.0f};
+            for (unsigned r = 0; r < cs; ++r) {
+                const MaxSumU q = sh.part[r];
+                const float d = q.m == -INFINITY ? -INFINITY : q.m - M, f = expf(d);
+                o.s += q.s * f;
+                o.u += fmaf(fmaxf(d, -1e30f), q.s, q.u) * f;
             }
         }
     }
     if (tid == 0) {
-        const RowScalars rs = row_scalars(MaxSum{o.m, o.s}, zy);
+        const RowScalars rs = row_scalars(MaxSum{o.m, o.s}, zy, a.lp64_out != nullptr);
         if (kEnt) a.entropy_out[t] = row_entropy(o, zy, rs.lp);
         if (a.lp_out) a.lp_out[t] = rs.lp;
         if (a.lse_out) a.lse_out[t] = rs.lse;
