@@ -217,10 +217,12 @@ __device__ __forceinline__ KpopSide kpop_side(float linf)
 // w = min{k, 1 + lambda*phi}; Table 8 for the other modes.  omp is 1 - p
 // where the caller already has it (row_scalars), else negative.  kAll false: the
 // band, IcePop and KPop are left out (the caller has none of them).
-template <bool kAll = true>
+// kMode: the operator where it is known at compile time (-1: P.mode's).
+template <bool kAll = true, int kMode = -1>
 __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float linf,
                                                     const DevParams &P, float omp = -1.0f)
 {
+    const int mode = kMode >= 0 ? kMode : P.mode;
     TokenWeight r;
     float ke;
     const float kh = two_sum(lw, -linf, ke);    // lw - linf = kh + ke exactly
@@ -231,7 +233,7 @@ __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float
     r.logk = logk;
     r.trunc = 0;
     r.w = 1.0f;
-    switch (P.mode) {
+    switch (mode) {
     case CIS_MODE_CIS: {
         // k > cap compared directly: near the cap, k and cap lie in
         // [1, 1 + lambda], where k's relative error is 2^-24 |log k| (the
@@ -278,7 +280,7 @@ __device__ __forceinline__ TokenWeight token_weight(float lw, float lw_lo, float
         break;
     }
     if constexpr (kAll) {
-        switch (P.mode) {
+        switch (mode) {
         case CIS_MODE_BAND: {
             // Sec. 4.3: the CIS weight, lifted from below to (1 + p)/2 (the image
             // of e^eps = 1/2).  Both comparisons as for CIS; k near (1 + p)/2 lies
