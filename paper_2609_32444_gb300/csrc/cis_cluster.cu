@@ -84,11 +84,22 @@ int cluster_threads()
     return v;
 }
 
+// CTA width where make_plan leaves it open.  Short slices give 256 threads too
+// little: with 128, more rows are on an SM at once (bf16, T=16384: V=1000 takes 57.6
+// us against 84.8, V=4000 79 against 105; T=8192: V=16000 86 against 88, but V=20000
+// 105.7 against 104.7, and V=151936 is 7% slower).  fp32 rows have half the entries
+// a byte: 128 threads throughout (T=4096, V=151936: 884 us against 927; T=8192,
+// V=1000: 30 against 41).
+int plan_threads(const ClusterPlan &p, int in_bytes)
+{
+    return in_bytes == 4 || (p.cs == 1 && p.slice <= 16384) ? 128 : 256;
+}
+
 template <typename InT, typename OutT> struct Aligned {
     static cudaError_t run(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
     {
-        if (a.entropy_out)  // the entropy variant is built for 256 threads only
-            return launch_cluster_nt<InT, OutT, 256, true, false, Ops::kPlain>(a, p, s);
+        if (a.entropy_out)
+            return launch_cluster_ent<InT, OutT, false, Ops::kPlain>(a, p, s);
         switch (p.nt) {
         case 512: return launch_cluster_nt<InT, OutT, 512, false, false, Ops::kPlain>(a, p, s);
         case 384: return launch_cluster_nt<InT, OutT, 384, false, false, Ops::kPlain>(a, p, s);
@@ -125,7 +136,7 @@ cudaError_t launch_cluster_fwd_bwd(const PassArgs &a, int dtype, int out_dtype, 
     make_plan(a.V, dtype == CIS_BF16 ? 2 : 4, &p);
     static const bool width_set = getenv("CIS_CLUSTER_THREADS") != nullptr;
     if (p.nt == 0 || width_set)
-        p.nt = cluster_threads();
+        p.nt = width_set ? cluster_threads() : plan_threads(p, dtype == CIS_BF16 ? 2 : 4);
     const bool aligned = aligned_rows(a, dtype == CIS_BF16 ? 2 : 4, out_dtype == CIS_BF16 ? 2 : 4);
     const int m = a.P.mode;
     // the smallest variant that can do the call

@@ -584,6 +584,16 @@ cudaError_t launch_cluster_nt(const PassArgs &a, const ClusterPlan &p, cudaStrea
     return cudaLaunchKernelEx(&cfg, kern, a, p.slice);
 }
 
+// The entropy variant: 128 threads, or for bf16 rows 256 too.
+template <typename InT, typename OutT, bool kRagged, Ops kOps>
+cudaError_t launch_cluster_ent(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
+{
+    if constexpr (sizeof(InT) == 2)
+        if (p.nt != 128)
+            return launch_cluster_nt<InT, OutT, 256, true, kRagged, kOps>(a, p, s);
+    return launch_cluster_nt<InT, OutT, 128, true, kRagged, kOps>(a, p, s);
+}
+
 // f(InT, OutT) for the two element types.
 template <template <typename, typename> class F>
 cudaError_t by_type(int dtype, int out_dtype, const PassArgs &a, const ClusterPlan &p,

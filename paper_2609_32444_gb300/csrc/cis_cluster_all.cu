@@ -9,7 +9,7 @@ template <typename InT, typename OutT> struct AllAligned {
     static cudaError_t run(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
     {
         if (a.entropy_out)
-            return launch_cluster_nt<InT, OutT, 256, true, false, Ops::kAll>(a, p, s);
+            return launch_cluster_ent<InT, OutT, false, Ops::kAll>(a, p, s);
         return p.nt == 128 ? launch_cluster_nt<InT, OutT, 128, false, false, Ops::kAll>(a, p, s)
                            : launch_cluster_nt<InT, OutT, 256, false, false, Ops::kAll>(a, p, s);
     }
@@ -19,7 +19,7 @@ template <typename InT, typename OutT> struct AllRagged {
     static cudaError_t run(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
     {
         if (a.entropy_out)
-            return launch_cluster_nt<InT, OutT, 256, true, true, Ops::kAll>(a, p, s);
+            return launch_cluster_ent<InT, OutT, true, Ops::kAll>(a, p, s);
         return p.nt == 128 ? launch_cluster_nt<InT, OutT, 128, false, true, Ops::kAll>(a, p, s)
                            : launch_cluster_nt<InT, OutT, 256, false, true, Ops::kAll>(a, p, s);
     }

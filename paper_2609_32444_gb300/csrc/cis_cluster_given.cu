@@ -10,7 +10,7 @@ template <typename InT, typename OutT> struct GivenAligned {
     static cudaError_t run(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
     {
         if (a.entropy_out)
-            return launch_cluster_nt<InT, OutT, 256, true, false, Ops::kGiven>(a, p, s);
+            return launch_cluster_ent<InT, OutT, false, Ops::kGiven>(a, p, s);
         return p.nt == 128 ? launch_cluster_nt<InT, OutT, 128, false, false, Ops::kGiven>(a, p, s)
                            : launch_cluster_nt<InT, OutT, 256, false, false, Ops::kGiven>(a, p, s);
     }
@@ -20,7 +20,7 @@ template <typename InT, typename OutT> struct GivenRagged {
     static cudaError_t run(const PassArgs &a, const ClusterPlan &p, cudaStream_t s)
     {
         if (a.entropy_out)
-            return launch_cluster_nt<InT, OutT, 256, true, true, Ops::kGiven>(a, p, s);
+            return launch_cluster_ent<InT, OutT, true, Ops::kGiven>(a, p, s);
         return p.nt == 128 ? launch_cluster_nt<InT, OutT, 128, false, true, Ops::kGiven>(a, p, s)
                            : launch_cluster_nt<InT, OutT, 256, false, true, Ops::kGiven>(a, p, s);
     }
