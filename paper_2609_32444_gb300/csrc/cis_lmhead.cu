@@ -66,6 +66,8 @@ constexpr int kThreads = 64 + kEpiThreads;
 constexpr int kHalf = kBN / 2;          // columns per epilogue half
 constexpr uint32_t kTmemCols = 2 * kBN;  // two accumulators
 constexpr size_t kSmemBytes = (size_t)kStages * kStageBytes + 1024;
+constexpr int kStageOut = 32 * 128;      // an epilogue warp's staging of dW: 32 rows of 128 bytes
+constexpr size_t kDualSmem = kSmemBytes + (size_t)kEpiWarps * kStageOut;
 constexpr int kMnBox = 64 * kBK * 2;     // one MN-major box: 64 MN entries x 64 K rows, 8 KB
 // dz of one chunk takes 2 Tp bytes per vocabulary column; the default chunk
 // keeps it within this many bytes.
@@ -148,8 +150,9 @@ struct GemmArgs {
     float *zy;        // kStats: z at the sampled token
     uint16_t *dz;     // kDz: bf16 [Tp, ld_dz], column = chunk-local vocabulary index
     int64_t ld_dz;
-    // kStore, kAccum: rows m 128 + r < rows_valid of out [., ld_out]; out_v8:
-    // out is 32-byte aligned (32-byte accesses), else 16-byte ones
+    // kStore, kAccum: rows m 128 + r < rows_valid of out [., ld_out] (fp32; dW, which
+    // may be bf16, goes through its tensor map); out_v8: out is 32-byte aligned
+    // (32-byte accesses), else 16-byte ones
     void *out;
     int out_bf16, rows_valid, out_v8;
     int64_t ld_out;
@@ -474,23 +477,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, uint32_t taddr,
             tc::tmem_ld32(taddr + c0, v);
             if (!live)
                 continue;
-            if (g.out_bf16) {
-                uint32_t w[16];
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    w[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
-                uint16_t *dst = reinterpret_cast<uint16_t *>(g.out) + o + c0;
-                if (g.out_v8) {  // streaming: outputs are not re-read here
-                    st_v8_cs(dst, w);
-                    st_v8_cs(dst + 16, w + 8);
-                } else {
-                    uint4 *d4 = reinterpret_cast<uint4 *>(dst);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        __stcs(d4 + q, make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2],
-                                                  w[4 * q + 3]));
-                }
-            } else if (g.out_v8) {
+            if (g.out_v8) {
                 float *dst = reinterpret_cast<float *>(g.out) + o + c0;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -525,6 +512,52 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, uint32_t taddr,
                 }
             }
         }
+    }
+}
+
+// dW's epilogue for one warp: its 32 rows and 128 columns of the tile go through
+// `stage` (128-byte rows, the tensor map's swizzle) to the copy engine, which
+// writes whole lines.  A tile of few K blocks is bound by its 128 KB of output, which
+// stores of 32 bytes to 32 rows a warp wrote at half the rate: T=512,
+// H=2048, V=151936: dH and dW take 527 us against 552, T=1024 with a quarter masked 681
+// against 729.
+template <bool kBf16>
+__device__ __forceinline__ void epilogue_staged(const GemmArgs &g, const CUtensorMap &tm,
+                                                uint32_t taddr, int m, int n, int lg, int lane,
+                                                int half, uint8_t *stage)
+{
+    constexpr int kCols = kBf16 ? 64 : 32;  // of a 128-byte row
+    const int y = m * kBM + lg * 32;
+    uint8_t *row = stage + lane * 128;
+#pragma unroll
+    for (int c0 = half * kHalf; c0 < (half + 1) * kHalf; c0 += kCols) {
+        uint32_t w[32];
+        float v[32];
+        tc::tmem_ld32(taddr + c0, v);
+        if (kBf16) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+                w[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
+            tc::tmem_ld32(taddr + c0 + 32, v);
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+                w[16 + q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 32; ++q)
+                w[q] = __float_as_uint(v[q]);
+        }
+        if (lane == 0)
+            tc::tma_store_wait_read();  // the last box has left the staging rows
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<uint4 *>(row + ((q ^ (lane & 7)) << 4)) =
+                make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+        tc::fence_async_shared();
+        __syncwarp();
+        if (lane == 0 && y < g.rows_valid)
+            tc::tma_store_2d(&tm, n * kBN + c0, y, stage);
     }
 }
 
@@ -620,6 +653,29 @@ __device__ __forceinline__ void epilogue_unit(const GemmArgs &g, const Unit &w, 
     if (!(MC && w.m >= g.nMt))
         epilogue_tile<EPI>(g, tmem + lane_off + acc * kBN, w.m, w.n, w.split, lg * 32 + lane,
                            half);
+    tc::fence_before_sync();
+    tc::bar_arrive(&bars.accempty[acc]);
+}
+
+// The same for a tile of dW, staged.
+template <bool MC>
+__device__ __forceinline__ void epilogue_dw(const GemmArgs &g, const CUtensorMap &tm,
+                                            const Unit &w, int i, uint32_t tmem, int warp,
+                                            int lane, Barriers &bars, const Abort &ab,
+                                            uint8_t *stage)
+{
+    const int lg = warp & 3;
+    const int half = (warp - 2) >> 2;
+    const int acc = i & 1;
+    ab.wait(&bars.accfull[acc], (i >> 1) & 1);
+    tc::fence_after_sync();
+    if (!(MC && w.m >= g.nMt)) {
+        const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + acc * kBN;
+        if (g.out_bf16)
+            epilogue_staged<true>(g, tm, taddr, w.m, w.n, lg, lane, half, stage);
+        else
+            epilogue_staged<false>(g, tm, taddr, w.m, w.n, lg, lane, half, stage);
+    }
     tc::fence_before_sync();
     tc::bar_arrive(&bars.accempty[acc]);
 }
@@ -744,7 +800,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     cis_lmhead_dual_kernel(const __grid_constant__ CUtensorMap tmA0,
                            const __grid_constant__ CUtensorMap tmB0,
                            const __grid_constant__ CUtensorMap tmA1,
-                           const __grid_constant__ CUtensorMap tmB1, const GemmArgs args0,
+                           const __grid_constant__ CUtensorMap tmB1,
+                           const __grid_constant__ CUtensorMap tmC1, const GemmArgs args0,
                            const GemmArgs args1)
 {
     extern __shared__ __align__(1024) uint8_t dsm[];
@@ -799,9 +856,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 epilogue_unit<EPI0, MC>(g0, unit_at<MC>(g0, u, rank), i, tmem, warp, lane,
                                         sh.bars, ab);
             else
-                epilogue_unit<kStore, MC>(g1, unit_at<MC>(g1, u, rank), i, tmem, warp, lane,
-                                          sh.bars, ab);
+                epilogue_dw<MC>(g1, tmC1, unit_at<MC>(g1, u, rank), i, tmem, warp, lane, sh.bars,
+                                ab, ring + kStages * kStageBytes + (warp - 2) * kStageOut);
         }
+        if (lane == 0)
+            tc::tma_store_wait();
     }
     gemm_teardown<MC>(sh, warp);
 }
@@ -1082,11 +1141,30 @@ bool make_map(CUtensorMap *m, const void *ptr, int64_t inner, int64_t outer, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// dW [rows, inner] as a store's target: boxes of 128 bytes x 32 rows, 128-byte
+// swizzle in shared memory.
+bool make_out_map(CUtensorMap *m, void *ptr, int64_t inner, int64_t rows, bool bf16)
+{
+    auto enc = encoder();
+    if (!enc)
+        return false;
+    const cuuint64_t es = bf16 ? 2 : 4;
+    cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)inner * es};
+    cuuint32_t box[2] = {(cuuint32_t)(128 / es), 32};
+    cuuint32_t one[2] = {1, 1};
+    return enc(m, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+               ptr, dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // The groups that run at once: co-resident 2-CTA clusters (MC), else SMs.
-template <typename K> cudaError_t resident_groups(K kern, bool mc, int *groups)
+template <typename K>
+cudaError_t resident_groups(K kern, bool mc, size_t smem, int *groups)
 {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBytes);
+                                         (int)smem);
     if (e != cudaSuccess)
         return e;
     if (!mc) {
@@ -1103,7 +1181,7 @@ template <typename K> cudaError_t resident_groups(K kern, bool mc, int *groups)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.dynamicSmemBytes = smem;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if ((e = cudaOccupancyMaxActiveClusters(groups, kern, &cfg)) != cudaSuccess)
@@ -1114,10 +1192,11 @@ template <typename K> cudaError_t resident_groups(K kern, bool mc, int *groups)
 // A persistent launch: one group (a cluster, or a CTA) per resident place, or
 // per unit where there are fewer.
 template <bool MC, typename K, typename... Args>
-cudaError_t launch_groups(K kern, int64_t units, cudaStream_t s, const Args &...args)
+cudaError_t launch_groups(K kern, int64_t units, size_t smem, cudaStream_t s,
+                          const Args &...args)
 {
     int groups = 0;
-    cudaError_t e = resident_groups(kern, MC, &groups);
+    cudaError_t e = resident_groups(kern, MC, smem, &groups);
     if (e != cudaSuccess)
         return e;
     if (units <= 0)
@@ -1130,7 +1209,7 @@ cudaError_t launch_groups(K kern, int64_t units, cudaStream_t s, const Args &...
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((units < groups ? units : groups) * (MC ? 2 : 1)));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = MC ? 1 : 0;
@@ -1150,25 +1229,23 @@ template <int EPI, bool MC>
 cudaError_t launch_gemm(const CUtensorMap &a, const CUtensorMap &b, const GemmArgs &g,
                         cudaStream_t s)
 {
-    return launch_groups<MC>(cis_lmhead_gemm_kernel<EPI, MC>, host_units<MC>(g), s, a, b, g);
+    return launch_groups<MC>(cis_lmhead_gemm_kernel<EPI, MC>, host_units<MC>(g), kSmemBytes, s, a,
+                             b, g);
 }
 
-// dH and dW of a chunk in one launch.
-template <int EPI0, bool MC>
-cudaError_t launch_dual(const CUtensorMap &a0, const CUtensorMap &b0, const GemmArgs &g0,
-                        const CUtensorMap &a1, const CUtensorMap &b1, const GemmArgs &g1,
+// dH and dW of a chunk in one launch: the maps of dz and W, of dz and H, and of dW.
+struct DualMaps {
+    CUtensorMap dz, w, dz_mn, h, dw;
+};
+template <bool MC>
+cudaError_t launch_dual(bool first, const DualMaps &m, const GemmArgs &g0, const GemmArgs &g1,
                         cudaStream_t s)
 {
-    return launch_groups<MC>(cis_lmhead_dual_kernel<EPI0, MC>,
-                             host_units<MC>(g0) + host_units<MC>(g1), s, a0, b0, a1, b1, g0, g1);
-}
-template <bool MC>
-cudaError_t launch_dual(bool first, const CUtensorMap &a0, const CUtensorMap &b0,
-                        const GemmArgs &g0, const CUtensorMap &a1, const CUtensorMap &b1,
-                        const GemmArgs &g1, cudaStream_t s)
-{
-    return first ? launch_dual<kStore, MC>(a0, b0, g0, a1, b1, g1, s)
-                 : launch_dual<kAccum, MC>(a0, b0, g0, a1, b1, g1, s);
+    const int64_t units = host_units<MC>(g0) + host_units<MC>(g1);
+    return first ? launch_groups<MC>(cis_lmhead_dual_kernel<kStore, MC>, units, kDualSmem, s, m.dz,
+                                     m.w, m.dz_mn, m.h, m.dw, g0, g1)
+                 : launch_groups<MC>(cis_lmhead_dual_kernel<kAccum, MC>, units, kDualSmem, s, m.dz,
+                                     m.w, m.dz_mn, m.h, m.dw, g0, g1);
 }
 
 // Whether a chunk's dH and dW run as one launch (CIS_LMHEAD_DUAL=0: one after
@@ -1264,7 +1341,7 @@ static int64_t chunk_for_bytes(int64_t T, int64_t V, int64_t Hd, size_t bytes)
 // the end in order.  The products take the room of a narrower chunk's dz, or
 // what the caller's workspace has beyond the layout.  T=512, H=2048, V=151936:
 // dH and dW take 552 us (two chunks) against 1123 one after the other, the call
-// 1096 against 1600; ranges of a share took 578, of a third 626, of a sixth
+// 1096 against 1600 (then); ranges of a share took 578, of a third 626, of a sixth
 // 577.  T=300, H=1024, V=32003: 68 against 212.
 // Leaving masked tokens out costs a call about 20 us (a scan, a copy, the zeroed
 // rows), whether or not many are masked: T=1244, V=1040, H=3072 with 40% masked took
@@ -1548,7 +1625,6 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
             gdh.b_k0 = (int)v0;
             gdh.rowmap = direct ? rowmap : nullptr;
             gdh.out = dh_rows;
-            gdh.out_bf16 = 0;
             gdh.out_v8 = (reinterpret_cast<uintptr_t>(dh_rows) & 31) == 0;
             gdh.ld_out = H;
             // DW[chunk] = dz^T H: A = dz MN-major (M along the chunk's columns,
@@ -1564,27 +1640,25 @@ CIS_API cis_status_t cis_lmhead_fused(const void *hidden, const void *weight, in
             gdw.b_row0 = 0;
             gdw.out = static_cast<uint8_t *>(dweight) + (size_t)v0 * (size_t)H * (bf16 ? 2 : 4);
             gdw.out_bf16 = bf16;
-            gdw.out_v8 = (reinterpret_cast<uintptr_t>(gdw.out) & 31) == 0;
             gdw.rows_valid = (int)w;
             gdw.ld_out = H;
             // both in one launch if both take the same CTA grouping, else each
             // in one that leaves the other out
+            lm::DualMaps maps{mDz, mWmn, mDzmn, mHmn, {}};
+            if (!lm::make_out_map(&maps.dw, gdw.out, H, w, bf16))
+                return CIS_ERR_UNSUPPORTED;
+            const bool first = v0 == 0;
             if (lm::dual_on() && ((mc & 12) == 12 || (mc & 12) == 0)) {
-                e = (mc & 12) ? lm::launch_dual<true>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, gdw, s)
-                              : lm::launch_dual<false>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, gdw,
-                                                       s);
+                e = (mc & 12) ? lm::launch_dual<true>(first, maps, gdh, gdw, s)
+                              : lm::launch_dual<false>(first, maps, gdh, gdw, s);
             } else {
                 lm::GemmArgs no_dh = gdh, no_dw = gdw;
                 no_dh.nNt = no_dw.nNt = 0;
-                e = (mc & 4) ? lm::launch_dual<true>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, no_dw,
-                                                     s)
-                             : lm::launch_dual<false>(v0 == 0, mDz, mWmn, gdh, mDzmn, mHmn, no_dw,
-                                                      s);
+                e = (mc & 4) ? lm::launch_dual<true>(first, maps, gdh, no_dw, s)
+                             : lm::launch_dual<false>(first, maps, gdh, no_dw, s);
                 if (e == cudaSuccess)
-                    e = (mc & 8) ? lm::launch_dual<true>(true, mDz, mWmn, no_dh, mDzmn, mHmn, gdw,
-                                                         s)
-                                 : lm::launch_dual<false>(true, mDz, mWmn, no_dh, mDzmn, mHmn, gdw,
-                                                          s);
+                    e = (mc & 8) ? lm::launch_dual<true>(true, maps, no_dh, gdw, s)
+                                 : lm::launch_dual<false>(true, maps, no_dh, gdw, s);
             }
             if (e != cudaSuccess)
                 return CIS_ERR_CUDA;
