@@ -353,14 +353,26 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         const bool far = !kRagged && m < kFarLogit;
         const float cm = far ? 0.0f : m * kLog2e;
         const float cm_err = far ? 0.0f : fmaf(m, kLog2e, -cm);  // m log2e - cm, exactly
-#pragma unroll 2
-        for (int g = threadIdx.x; g < ng; g += kThreads) {
+        auto add = [&](int g) {
             float z[8];
             load8<InT>(slab, g, z);
-            if (kEnt)
-                s += sum8_exp2_off_u(z, cm, u);
-            else
-                s += sum8_exp2_off(z, cm);
+            return kEnt ? sum8_exp2_off_u(z, cm, u) : sum8_exp2_off(z, cm);
+        };
+        if constexpr (kThreads == 128) {
+            // twice as many groups a thread as with 256: two at a time, added to
+            // each other first, so that the growing sum is added to as often
+            int g = threadIdx.x;
+#pragma unroll 1
+            for (; g + kThreads < ng; g += 2 * kThreads) {
+                const float a = add(g);
+                s += a + add(g + kThreads);
+            }
+            if (g < ng)
+                s += add(g);
+        } else {
+#pragma unroll 2
+            for (int g = threadIdx.x; g < ng; g += kThreads)
+                s += add(g);
         }
         const float f = ex2_ftz(-cm_err);
         if (kEnt)  // sum e (z - m) = f ln2 (sum e x - cm_err sum e)
