@@ -434,8 +434,11 @@ def run_lmhead(args, rank, world, local):
     tp = -(-T // 128) * 128
     chunk = min(-(-V // 256) * 256, max(256, (1 << 30) // (2 * tp) // 256 * 256))
     n_chunks = -(-V // chunk)
-    # scales, FWD, token, (DZ, then DH and DW in one launch) per chunk, reduce
+    # scales, FWD, token, (DZ, then DH and DW in one launch) per chunk, reduce; with a mask and
+    # T V H >= 8e10 also the valid tokens' numbering and gathering, and the zeroed rows
     launches_per_call = 3 + 2 * n_chunks + 1
+    if b.mask is not None and T > 128 and T * V * H >= 8e10:
+        launches_per_call += 3
 
     def step():
         return binding.cis_lmhead_fused(b.hidden, b.weight, b.ids, b.lp_infer, b.adv, P,

@@ -98,8 +98,8 @@ typedef enum {
     CIS_MODE_BAND = 4,    /* w = max{min{k, 1 + lambda*phi}, (1 + p)/2}        */
     CIS_MODE_ICEPOP = 5,  /* w = k if k in [icepop_lo, icepop_hi], else 0      */
     CIS_MODE_KPOP = 6,    /* w = k if max(KL_B(p||q), KL_B(q||p)) <= kpop_phi,
-                           *     else 0; fp64, p and q clamped to
-                           *     [1e-8, 1 - 1e-8] (App. D.5)                   */
+                           *     else 0, as fp64 decides; p and q clamped
+                           *     to [1e-8, 1 - 1e-8] (App. D.5)                */
     CIS_MODE_SEQ_TIS = 7, /* w = min(K, seq_cap)                               */
     CIS_MODE_SEQ_MIS = 8  /* w = K if K in [seq_lo, seq_hi], else 0           */
 } cis_mode_t;
@@ -220,10 +220,10 @@ CIS_API cis_status_t cis_token_logprobs(const void *logits, int32_t dtype, int64
  *             eps = logit p - logit q (Lemma 3.1); +-inf or NaN where p or q
  *             rounds to 1 (the weight itself stays finite).
  * Decisions are taken on log k = lp_train - lp_infer, evaluated exactly.  CIS
- * compares k with the cap, and TIS and EXACT compare log k with the log of the
- * bound.  Each is settled in fp32 where its error bound proves the answer, else
- * in fp64.  The band, IcePop, KPop and the sequence operators (log K summed in
- * fp64) decide in fp64.  Errors:
+ * and the band compare k with their bounds, TIS, EXACT and IcePop log k with
+ * the log of theirs, KPop the binary KL with phi.  Each is settled in fp32 where
+ * its error bound proves the answer, else in fp64.  The sequence operators (log K
+ * summed in fp64) decide in fp64.  Errors:
  * CIS_ERR_INVALID_ARG for NULL required pointers, T < 0, parameters outside
  * the ranges of cis_params_t, or a sequence operator without cu_seqlens.
  */
@@ -360,7 +360,7 @@ CIS_API cis_status_t cis_lmhead_workspace_size_chunk(int64_t T, int64_t V, int64
  *   ids, lp_infer, lp_old, adv, mask, cu_seqlens, B, params: as for
  *               cis_loss_fwd_bwd.
  *   dhidden     device [T, H] of grad_dtype (CIS_F32 or CIS_BF16), written;
- *               16-byte aligned (32-byte aligned buffers take the wider stores).
+ *               16-byte aligned (32-byte aligned fp32 buffers take wider stores).
  *   dweight     device [V, H] of grad_dtype, written (rows of tokens that are
  *               masked contribute nothing); alignment as for dhidden.
  *   lp_out, w_out, trunc_out, entropy_out, stats_out, loss_out: as for

@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
 
 // Groups per slot (CIS_DIAG_SLOT_GROUPS, read at each call: small values
 // make short rows span several slots in tests), and whether the streaming
-// kernel applies at all (CIS_DIAG_KERNEL=row selects the one-CTA kernel).
+// kernel applies at all (CIS_DIAG_KERNEL=row selects the split kernel).
 int diag_slot_groups(int max_groups)
 {
     const char *e = getenv("CIS_DIAG_SLOT_GROUPS");

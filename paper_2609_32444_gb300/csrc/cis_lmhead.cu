@@ -783,7 +783,7 @@ __device__ __forceinline__ DualList dual_list(const GemmArgs &g0, const GemmArgs
     d.L = r ? G - r : 0;
     d.pos = c >= r ? c - r : c - r + G;
     d.n_dh = q + (c < r);
-        const int cost1 = g1.ksplit > kDwBlocks ? g1.ksplit : kDwBlocks;
+    const int cost1 = g1.ksplit > kDwBlocks ? g1.ksplit : kDwBlocks;
     const int x = d.L ? g0.ksplit / cost1 : 0;
     d.A = d.L * x < n1 ? d.L * x : n1;
     d.n_a = d.pos < d.L && d.A > d.pos ? (d.A - d.pos + d.L - 1) / d.L : 0;
@@ -1340,9 +1340,9 @@ static int64_t chunk_for_bytes(int64_t T, int64_t V, int64_t Hd, size_t bytes)
 // cluster's share of the launch, each with fp32 products of its own, added at
 // the end in order.  The products take the room of a narrower chunk's dz, or
 // what the caller's workspace has beyond the layout.  T=512, H=2048, V=151936:
-// dH and dW take 552 us (two chunks) against 1123 one after the other, the call
-// 1096 against 1600 (then); ranges of a share took 578, of a third 626, of a sixth
-// 577.  T=300, H=1024, V=32003: 68 against 212.
+// dH and dW take 527 us (two chunks) against 1123 one after the other, the call
+// 1054 against 1600; ranges of a share took 5% longer, of a third 13%, of a sixth
+// 5%.  T=300, H=1024, V=32003: 68 against 212.
 // Leaving masked tokens out costs a call about 20 us (a scan, a copy, the zeroed
 // rows), whether or not many are masked: T=1244, V=1040, H=3072 with 40% masked took
 // 107 us against 93.  It is done from here on, where the products take 400 us.

@@ -4,7 +4,8 @@
 //
 // Bound: the host.  A fused pass of T=256, V=1024 keeps the GPU busy for 13 us,
 // and its call took 45 us of Python (checks of five tensors, seven outputs,
-// twenty-six converted arguments); from here it takes 21 us, most of it in the three launches.
+// twenty-six converted arguments); from here it takes 17 us, 7.5 of them the
+// library's (three launches).
 //
 // Every function takes its Python counterpart's arguments by position, and
 // answers with that function's result; with an int, the library's error; or with
