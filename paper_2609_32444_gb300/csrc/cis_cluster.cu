@@ -88,8 +88,8 @@ int cluster_threads()
 // little: with 128, more rows are on an SM at once (bf16, T=16384: V=1000 takes 57.6
 // us against 84.8, V=4000 79 against 105; T=8192: V=16000 86 against 88, but V=20000
 // 105.7 against 104.7, and V=151936 is 7% slower).  fp32 rows have half the entries
-// a byte: 128 threads throughout (T=4096, V=151936: 884 us against 927; T=8192,
-// V=1000: 30 against 41).
+// a byte: 128 threads throughout (T=4096, V=151936: 718 us against 736; T=8192,
+// V=1000: 28.6 against 43).
 int plan_threads(const ClusterPlan &p, int in_bytes)
 {
     return in_bytes == 4 || (p.cs == 1 && p.slice <= 16384) ? 128 : 256;

@@ -73,10 +73,8 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
     return __float2bfloat16_rn(v);
 }
 
-// 8 results to global memory with streaming (evict-first) 16-byte stores.
-template <typename OutT> __device__ __forceinline__ void store8(OutT *dst, const float (&v)[8]);
-template <>
-__device__ __forceinline__ void store8<__nv_bfloat16>(__nv_bfloat16 *dst, const float (&v)[8])
+// 8 or 4 results to global memory with a streaming (evict-first) store.
+__device__ __forceinline__ void store_group(__nv_bfloat16 *dst, const float (&v)[8])
 {
     uint4 q;
     __nv_bfloat162 h;
@@ -86,13 +84,36 @@ __device__ __forceinline__ void store8<__nv_bfloat16>(__nv_bfloat16 *dst, const 
     h = __floats2bfloat162_rn(v[6], v[7]); q.w = *reinterpret_cast<uint32_t *>(&h);
     __stcs(reinterpret_cast<uint4 *>(dst), q);
 }
-template <>
-__device__ __forceinline__ void store8<float>(float *dst, const float (&v)[8])
+__device__ __forceinline__ void store_group(float *dst, const float (&v)[4])
 {
     __stcs(reinterpret_cast<float4 *>(dst), make_float4(v[0], v[1], v[2], v[3]));
-    __stcs(reinterpret_cast<float4 *>(dst) + 1, make_float4(v[4], v[5], v[6], v[7]));
 }
-
+__device__ __forceinline__ void store_group(__nv_bfloat16 *dst, const float (&v)[4])
+{
+    uint2 q;
+    __nv_bfloat162 h;
+    h = __floats2bfloat162_rn(v[0], v[1]); q.x = *reinterpret_cast<uint32_t *>(&h);
+    h = __floats2bfloat162_rn(v[2], v[3]); q.y = *reinterpret_cast<uint32_t *>(&h);
+    __stcs(reinterpret_cast<uint2 *>(dst), q);
+}
+// Group g of a slab, of 8 entries or 4.
+template <typename InT>
+__device__ __forceinline__ void load_group(const uint8_t *slab, int g, float (&z)[8])
+{
+    load8<InT>(slab, g, z);
+}
+template <typename InT>
+__device__ __forceinline__ void load_group(const uint8_t *slab, int g, float (&z)[4])
+{
+    if constexpr (sizeof(InT) == 4) {
+        const float4 q = reinterpret_cast<const float4 *>(slab)[g];
+        z[0] = q.x; z[1] = q.y; z[2] = q.z; z[3] = q.w;
+    } else {
+        const uint2 q = reinterpret_cast<const uint2 *>(slab)[g];
+        z[0] = bf16_lo(q.x); z[1] = bf16_hi(q.x);
+        z[2] = bf16_lo(q.y); z[3] = bf16_hi(q.y);
+    }
+}
 
 // Zero the n entries at dst (any alignment), 16 bytes a store between the ends.
 template <typename OutT, int kThreads> __device__ __forceinline__ void zero_run(OutT *dst, int n)
@@ -188,6 +209,7 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     const int pad = kRagged ? (int)(reinterpret_cast<uintptr_t>(irow) / sizeof(InT) & 7) : 0;
     const int ng = kRagged ? (n > 0 ? (int)((pad + n + 7) / 8) : 0) : (int)(n / 8);
     constexpr int kGroupBytes = 8 * sizeof(InT);
+    constexpr bool kExact = kRagged && sizeof(OutT) == 4;  // pass 2's exponents, below
     OutT *orow = reinterpret_cast<OutT *>(a.dz) + t * a.ld_out + v0;
 
     const bool valid = a.mask == nullptr || a.mask[t] != 0;
@@ -199,9 +221,13 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         if constexpr (kRagged) {
             zero_run<OutT, kThreads>(orow, (int)n);
         } else {
-            const float zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            for (int g = threadIdx.x; g < ng; g += kThreads)
-                store8<OutT>(orow + 8 * g, zero);
+            constexpr int ZV = 16 / sizeof(OutT);
+            float zero[ZV];
+#pragma unroll
+            for (int i = 0; i < ZV; ++i)
+                zero[i] = 0.0f;
+            for (int g = threadIdx.x; g < ng * (8 / ZV); g += kThreads)
+                store_group(orow + ZV * g, zero);
         }
         if (threadIdx.x == 0)
             grid_wait();  // in every CTA, so that this grid ends after the one before
@@ -319,8 +345,8 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     __syncthreads();  // barriers initialised before anyone polls them
 
     // The sampled entry takes no part in the sums over j != y: the thread that
-    // owns its 8-entry group (the only thread that reads that group in either
-    // pass) overwrites it with -inf in shared memory once its chunk has landed.
+    // owns its 8-entry group (the only thread that reads that group in pass
+    // 1) overwrites it with -inf in shared memory once its chunk has landed.
     const int64_t yl = y - v0;
     const int gy = (yl >= 0 && yl < n) ? (int)((yl + pad) >> 3) : -1;
     const int iy = (int)((yl + pad) & 7);
@@ -353,16 +379,20 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         const bool far = !kRagged && m < kFarLogit;
         const float cm = far ? 0.0f : m * kLog2e;
         const float cm_err = far ? 0.0f : fmaf(m, kLog2e, -cm);  // m log2e - cm, exactly
+        const auto sum8_u = [](const float (&z)[8], float off, float &u) {
+            return sizeof(InT) == 4 ? sum8_exp2_off_u2(z, off, u) : sum8_exp2_off_u(z, off, u);
+        };
         auto add = [&](int g) {
             float z[8];
-            load8<InT>(slab, g, z);
-            return kEnt ? sum8_exp2_off_u(z, cm, u) : sum8_exp2_off(z, cm);
+            load8_any<InT>(slab, g, z);
+            return kEnt ? sum8_u(z, cm, u) : sum8_exp2_off(z, cm);
         };
         if constexpr (kThreads == 128) {
             // twice as many groups a thread as with 256: two at a time, added to
             // each other first, so that the growing sum is added to as often
+            // (fp32 slices are long and the warps few: two such pairs in flight)
             int g = threadIdx.x;
-#pragma unroll 1
+#pragma unroll sizeof(InT) == 4 ? 2 : 1
             for (; g + kThreads < ng; g += 2 * kThreads) {
                 const float a = add(g);
                 s += a + add(g + kThreads);
@@ -483,7 +513,7 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
             cs *= ex2_ftz(-(se + pe + qe));
         }
         sh.row = make_float4(cs * scale, B, c * (0.0f - omp), 0.0f);  // c (p - 1): +0 if p = 1
-        if (kRagged && !(fabsf(m) < kHugeLogit)) {
+        if (kExact || (kRagged && !(fabsf(m) < kHugeLogit))) {
             sh.row.x = c * scale;
             sh.row.w = 1.0f;
             sh.slow = make_float2(m, bias_log2);
@@ -513,24 +543,41 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
     // 2^(x_j + K) would be subnormal, |c softmax_j| < 2^-150 rounds to zero in
     // fp32 and bf16 anyway; c 2^-K stays normal and 2^(x_j + K) finite.  The
     // final multiply keeps subnormal products.
+    // With an fp32 side a thread takes W = 4 entries at a time, so that a warp's
+    // accesses are to neighbouring bytes (8 fp32 entries a thread left gaps between
+    // its vectors: two-way bank conflicts, and every sector written in halves).
+    // T=1024, V=151936 fp32 with the entropy and KPop: the pass takes 217 us against
+    // 264 (pass 1's loads likewise, load8_any); T=4096, V=32000: fp32 to bf16 133
+    // against 155, bf16 to fp32 120 against 128.
+    // kExact: exponents from the exact z - m, without the power of two, whose
+    // place in the exponent's argument costs it up to 4 bits (fp32 gradients of a row
+    // are within 1.1e-7, else 1.6e-7; the aligned form has no issue slots to spare).
     const float4 row = sh.row;
+    const float2 exact = kExact ? sh.slow : make_float2(0.0f, 0.0f);
+    const auto grad = [&](float z, float c2, float b) {
+        return kExact ? c2 * ex2_full(fmaf(z - exact.x, kLog2e, -exact.y))
+                      : c2 * ex2_ftz(fmaf(z, kLog2e, -b));
+    };
     const float cs2 = row.x, B = row.y, dzy = row.z;
-    if (kRagged && row.w != 0.0f) {
+    constexpr int W = sizeof(InT) == 4 || sizeof(OutT) == 4 ? 4 : 8;
+    constexpr int kUnroll = 16 / W;
+    const int gw = W == 8 ? gy : 2 * gy + (iy >> 2), iw = iy & (W - 1);  // (gy < 0: gw < 0)
+    if (kRagged && !kExact && row.w != 0.0f) {
         slow_gradient<InT, OutT, kThreads>(slab, pad, (int)n, (int)yl, orow, cs2, dzy, sh.slow);
     } else if constexpr (!kRagged) {
-#pragma unroll 2
-        for (int g = threadIdx.x; g < ng; g += kThreads) {
-            float z[8], v[8];
-            load8<InT>(slab, g, z);
+#pragma unroll kUnroll
+        for (int g = threadIdx.x; g < ng * (8 / W); g += kThreads) {
+            float z[W], v[W];
+            load_group<InT>(slab, g, z);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < W; ++i)
                 v[i] = cs2 * ex2_ftz(fmaf(z[i], kLog2e, -B));
-            if (g == gy) {  // the sampled entry: c (p - 1)
+            if (g == gw) {  // the sampled entry: c (p - 1)
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    v[i] = i == iy ? dzy : v[i];
+                for (int i = 0; i < W; ++i)
+                    v[i] = i == iw ? dzy : v[i];
             }
-            store8<OutT>(orow + 8 * g, v);
+            store_group(orow + W * g, v);
         }
     } else {
         // Groups whose entries all exist go out whole where the output has the
@@ -540,30 +587,29 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         const InT *sl = reinterpret_cast<const InT *>(slab);
         const int phase = (int)(reinterpret_cast<uintptr_t>(orow) / sizeof(OutT)) - pad;
         const bool whole = (phase & (EV - 1)) == 0;
-        const int g0 = whole ? (pad > 0) : 0;
-        const int g1 = whole ? (int)((pad + n) / 8) : 0;
-#pragma unroll 2
+        const int g0 = whole ? (pad + W - 1) / W : 0;
+        const int g1 = whole ? (int)((pad + n) / W) : 0;
+#pragma unroll kUnroll
         for (int g = g0 + threadIdx.x; g < g1; g += kThreads) {
-            float z[8], v[8];
-            load8<InT>(slab, g, z);
+            float z[W], v[W];
+            load_group<InT>(slab, g, z);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                v[i] = cs2 * ex2_ftz(fmaf(z[i], kLog2e, -B));
-            if (g == gy) {
+            for (int i = 0; i < W; ++i)
+                v[i] = grad(z[i], cs2, B);
+            if (g == gw) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    v[i] = i == iy ? dzy : v[i];
+                for (int i = 0; i < W; ++i)
+                    v[i] = i == iw ? dzy : v[i];
             }
-            store8<OutT>(orow + (8 * g - pad), v);
+            store_group(orow + (W * g - pad), v);
         }
         // entries [0, e0) and [e1, n) of the slice
-        const int e0 = whole ? min((int)n, 8 * g0 - (g0 ? pad : 0)) : 0;
-        const int e1 = whole ? max(e0, 8 * g1 - pad) : 0;
+        const int e0 = whole ? min((int)n, W * g0 - (g0 ? pad : 0)) : 0;
+        const int e1 = whole ? max(e0, W * g1 - pad) : 0;
         for (int k = threadIdx.x; k < e0 + ((int)n - e1); k += kThreads) {
             const int e = k < e0 ? k : e1 + (k - e0);
             orow[e] = from_f32<OutT>(e == (int)yl ? dzy
-                                                  : cs2 * ex2_ftz(fmaf(to_f32(sl[pad + e]),
-                                                                       kLog2e, -B)));
+                                                 : grad(to_f32(sl[pad + e]), cs2, B));
         }
     }
     cluster_wait();

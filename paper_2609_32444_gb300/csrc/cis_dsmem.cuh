@@ -111,6 +111,23 @@ __device__ __forceinline__ void load8<float>(const uint8_t *sm, int g, float (&z
     z[6] = __uint_as_float(q1.z); z[7] = __uint_as_float(q1.w);
 }
 
+// The same 8 entries where the halves' order does not matter (a maximum, a sum
+// that adds the halves last).  In fp32 every other four threads take the second
+// half first: eight threads then read all banks once instead of half of them twice.
+template <typename InT> __device__ __forceinline__ void load8_any(const uint8_t *sm, int g,
+                                                                  float (&z)[8])
+{
+    if constexpr (sizeof(InT) == 4) {
+        const int h = (int)(threadIdx.x >> 2) & 1;
+        const float4 q0 = reinterpret_cast<const float4 *>(sm)[2 * g + h];
+        const float4 q1 = reinterpret_cast<const float4 *>(sm)[2 * g + (h ^ 1)];
+        z[0] = q0.x; z[1] = q0.y; z[2] = q0.z; z[3] = q0.w;
+        z[4] = q1.x; z[5] = q1.y; z[6] = q1.z; z[7] = q1.w;
+    } else {
+        load8<InT>(sm, g, z);
+    }
+}
+
 // Overwrite entry j of the slab with -inf.
 template <typename InT> __device__ __forceinline__ void poke_neg_inf(uint8_t *sm, int j);
 template <> __device__ __forceinline__ void poke_neg_inf<__nv_bfloat16>(uint8_t *sm, int j)
@@ -149,18 +166,22 @@ template <> struct MaxAcc<__nv_bfloat16> {
     }
 };
 template <> struct MaxAcc<float> {
-    float m = -INFINITY;
+    float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
     __device__ __forceinline__ void consume(const uint8_t *sm, int g0, int g1, int step)
     {
+#pragma unroll 1
         for (int g = g0; g < g1; g += step) {
             float z[8];
-            load8<float>(sm, g, z);
+            load8_any<float>(sm, g, z);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                m = max_nan(m, z[i]);
+            for (int i = 0; i < 4; ++i)
+                m[i] = max_nan(m[i], max_nan(z[i], z[i + 4]));
         }
     }
-    __device__ __forceinline__ float result() const { return m; }
+    __device__ __forceinline__ float result() const
+    {
+        return max_nan(max_nan(m[0], m[1]), max_nan(m[2], m[3]));
+    }
 };
 
 // Sum of 2^{z_i log2e - off} over 8 values, added pairwise.
@@ -186,6 +207,22 @@ __device__ __forceinline__ float sum8_exp2_off_u(const float (&z)[8], float off,
         e[i] = ex2_ftz(x);
         u = fmaf(e[i], fmaxf(x, -1024.0f), u);
     }
+    return ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
+}
+
+// The same with the second half's u terms added on their own: half the chain, for
+// fp32 slices, which leave few warps a SM to hide it.
+__device__ __forceinline__ float sum8_exp2_off_u2(const float (&z)[8], float off, float &u)
+{
+    float e[8], uh = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const float x = fmaf(z[i], kLog2e, -off);
+        e[i] = ex2_ftz(x);
+        float &v = i < 4 ? u : uh;
+        v = fmaf(e[i], fmaxf(x, -1024.0f), v);
+    }
+    u += uh;
     return ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
 }
 

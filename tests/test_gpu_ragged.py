@@ -58,7 +58,8 @@ def _check(z, ids, dz, T, V, entropy=False):
 @pytest.mark.parametrize("din,dout", [(BF16, BF16), (BF16, F32), (F32, F32), (F32, BF16)])
 @pytest.mark.parametrize("T,V", [(5, 1), (9, 2), (9, 7), (9, 8), (9, 9), (17, 15), (17, 17),
                                  (9, 31), (5, 1001), (9, 2047), (9, 2056), (3, 20483),
-                                 (3, 32003), (2, 90005)])
+                                 (3, 32003), (2, 90005),
+                                 (2, 409601), (2, 819201)])  # too long for a cluster: row kernel
 def test_any_alignment(din, dout, T, V):
     """Rows that start at every phase of a 16-byte boundary: contiguous odd rows
     in both tensors (whole groups are stored), rows whose strides or first
