@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         if (has_old) {
             lold = a.lp_old[t];
             tw = token_weight<kAll>(lold, 0.0f, linf, a.P);
-        } else if (kAll) {
+        } else if (kAll || kRagged) {
             // 1 / q as a pair: q as one, its reciprocal's residual from FMAs
             float ql;
             const float qh = exp_pair(linf, 0.0f, ql);
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
                 qinv = 1.0f / qh;
                 qinv_lo = -qinv * fmaf(ql, qinv, fmaf(qh, qinv, -1.0f));
             }
-            if (a.P.mode == CIS_MODE_KPOP)
+            if (kAll && a.P.mode == CIS_MODE_KPOP)
                 kq = kpop_side(linf);
         }
         // the workspace is the kernel before's until it has ended; with the
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         DirectRow dw;
         direct = !has_old && row_direct(o, zy, dw);
         if (direct && !given)
-            direct = weight_direct<kAll>(dw, linf, qinv, qinv_lo, kq, a.P, tw.w, tw.trunc);
+            direct = weight_direct<kAll, kAll || kRagged>(dw, linf, qinv, qinv_lo, kq, a.P, tw.w, tw.trunc);
         if (direct) {
             omp = dw.omp;
             tdir = dw.t;

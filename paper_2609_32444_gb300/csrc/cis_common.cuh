@@ -606,19 +606,19 @@ __device__ __forceinline__ bool row_direct(MaxSum o, float zy, DirectRow &r)
 }
 
 // The weight with the current log p as l_w (no l_old, no sequence weight); qinv
-// (+ qinv_lo with kAll) is e^{-l_inf}.  kAll as in token_weight.  False where a decision is too close
+// (+ qinv_lo with kPair) is e^{-l_inf}.  kAll as in token_weight.  False where a decision is too close
 // to call, l_inf < -70, or the band's bounds are taken (they are rounded once,
 // from pairs, by token_weight).
-template <bool kAll>
+template <bool kAll, bool kPair>
 __device__ __forceinline__ bool weight_direct(const DirectRow &d, float linf, float qinv,
                                               float qinv_lo, const KpopSide &kq,
                                               const DevParams &P, float &w, uint8_t &trunc)
 {
     if (!(linf >= -70.0f))
         return false;
-    // the other operators' weights come from log k, rounded less often than
-    // p / q: 1 / q as a pair makes up for it
-    const float k = kAll ? fmaf(d.p, qinv, d.p * qinv_lo) : d.p * qinv;
+    // log k, which token_weight takes them from, is rounded less often than p / q:
+    // 1 / q as a pair makes up for it (not in the plain aligned form)
+    const float k = kPair ? fmaf(d.p, qinv, d.p * qinv_lo) : d.p * qinv;
     trunc = 0;
     w = k;
     switch (P.mode) {
