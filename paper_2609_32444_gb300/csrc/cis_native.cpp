@@ -12,6 +12,9 @@
 // None where an argument is not what the plain case expects (a tensor of another
 // kind, type, shape or device): then nothing was done, and the counterpart goes
 // on in Python, where the checks raise.
+//
+// Data pointers are taken before the GIL is released: a tensor without storage (a
+// functorch wrapper, which passes for a plain tensor) raises there.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <dlfcn.h>
@@ -110,7 +113,10 @@ template <typename T = void> T *ptr(const Tensor *t)
 {
     return t ? static_cast<T *>(t->data_ptr()) : nullptr;
 }
-template <typename T = void> T *ptr(const Tensor &t) { return ptr<T>(&t); }
+template <typename T = void> T *ptr(const Tensor &t)
+{
+    return t.defined() ? ptr<T>(&t) : nullptr;
+}
 Tensor fresh(at::IntArrayRef shape, at::ScalarType dt, const at::Device &dev)
 {
     return at::empty(shape, at::TensorOptions().dtype(dt).device(dev));
@@ -189,15 +195,22 @@ PyObject *loss_fwd_bwd(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Tensor loss = fresh({1}, at::kDouble, dev);
     const Tensor ws = ws_in && ws_in->numel() >= (int64_t)need ? *ws_in
                                                                : fresh({(int64_t)need}, at::kByte, dev);
+    const void *pz = ptr(z);
+    const int32_t *pids = ptr<int32_t>(ids), *pcu = ptr<int32_t>(cu);
+    const float *plpi = ptr<float>(lpi), *pold = ptr<float>(old), *padv = ptr<float>(adv);
+    const uint8_t *pmask = ptr<uint8_t>(mask);
+    const int64_t nseq = cu ? cu->size(0) - 1 : 0;
+    void *pdz = ptr(dz), *pws = ptr(ws);
+    float *plp = ptr<float>(lp), *pw = ptr<float>(w), *pent = ptr<float>(ent);
+    uint8_t *ptrunc = ptr<uint8_t>(tr);
+    cis_stats_t *pstats = ptr<cis_stats_t>(stats);
+    double *ploss = ptr<double>(loss);
+    const size_t nws = (size_t)ws.numel();
     int rc;
     void *s = stream();
     Py_BEGIN_ALLOW_THREADS
-    rc = lib.loss(ptr(z), code, T, V, ld, ptr<int32_t>(ids), ptr<float>(lpi), ptr<float>(old),
-                  ptr<float>(adv), ptr<uint8_t>(mask), ptr<int32_t>(cu), cu ? cu->size(0) - 1 : 0,
-                  &P, ptr(dz), code_out, ldo, lp.defined() ? ptr<float>(lp) : nullptr,
-                  w.defined() ? ptr<float>(w) : nullptr, tr.defined() ? ptr<uint8_t>(tr) : nullptr,
-                  ent.defined() ? ptr<float>(ent) : nullptr, ptr<cis_stats_t>(stats),
-                  ptr<double>(loss), ptr(ws), (size_t)ws.numel(), s);
+    rc = lib.loss(pz, code, T, V, ld, pids, plpi, pold, padv, pmask, pcu, nseq, &P, pdz, code_out,
+                  ldo, plp, pw, ptrunc, pent, pstats, ploss, pws, nws, s);
     Py_END_ALLOW_THREADS
     if (rc != CIS_OK)
         return PyLong_FromLong(rc);
@@ -227,12 +240,15 @@ PyObject *token_logprobs(PyObject *, PyObject *const *a, Py_ssize_t n)
     const at::Device dev = z->device();
     const Tensor lp = fresh({T}, at::kFloat, dev), lse = fresh_if(want_lse, T, at::kFloat, dev);
     const Tensor ent = fresh_if(want_ent, T, at::kFloat, dev);
+    const void *pz = ptr(z);
+    const int32_t *pids = ptr<int32_t>(ids);
+    const uint8_t *pmask = ptr<uint8_t>(mask);
+    float *plp = ptr<float>(lp), *plse = ptr<float>(lse), *pent = ptr<float>(ent);
+    int32_t *pst = ptr<int32_t>(st);
     int rc;
     void *s = stream();
     Py_BEGIN_ALLOW_THREADS
-    rc = lib.logprobs(ptr(z), code, T, V, ld, ptr<int32_t>(ids), ptr<uint8_t>(mask),
-                      ptr<float>(lp), lse.defined() ? ptr<float>(lse) : nullptr,
-                      ent.defined() ? ptr<float>(ent) : nullptr, ptr<int32_t>(st), s);
+    rc = lib.logprobs(pz, code, T, V, ld, pids, pmask, plp, plse, pent, pst, s);
     Py_END_ALLOW_THREADS
     if (rc != CIS_OK)
         return PyLong_FromLong(rc);
@@ -263,13 +279,16 @@ PyObject *weights(PyObject *, PyObject *const *a, Py_ssize_t n)
     const at::Device dev = lt->device();
     const Tensor w = fresh({T}, at::kFloat, dev), tr = fresh_if(want_tr, T, at::kByte, dev);
     const Tensor eps = fresh_if(want_eps, T, at::kFloat, dev);
+    const float *plt = ptr<float>(lt), *pli = ptr<float>(li);
+    const uint8_t *pmask = ptr<uint8_t>(mask);
+    const int32_t *pcu = ptr<int32_t>(cu);
+    const int64_t nseq = cu ? cu->size(0) - 1 : 0;
+    float *pw = ptr<float>(w), *peps = ptr<float>(eps);
+    uint8_t *ptrunc = ptr<uint8_t>(tr);
     int rc;
     void *s = stream();
     Py_BEGIN_ALLOW_THREADS
-    rc = lib.weights(ptr<float>(lt), ptr<float>(li), ptr<uint8_t>(mask), T, ptr<int32_t>(cu),
-                     cu ? cu->size(0) - 1 : 0, &P, ptr<float>(w),
-                     tr.defined() ? ptr<uint8_t>(tr) : nullptr,
-                     eps.defined() ? ptr<float>(eps) : nullptr, s);
+    rc = lib.weights(plt, pli, pmask, T, pcu, nseq, &P, pw, ptrunc, peps, s);
     Py_END_ALLOW_THREADS
     if (rc != CIS_OK)
         return PyLong_FromLong(rc);
@@ -315,11 +334,15 @@ PyObject *binned_sums(PyObject *, PyObject *const *a, Py_ssize_t n)
     const Tensor sums = fresh({(int64_t)nv, (int64_t)nb}, at::kDouble, dev);
     uint8_t *w = ptr<uint8_t>(ws);
     w += (256 - (reinterpret_cast<uintptr_t>(w) & 255)) & 255;
+    const float *pkey = ptr<float>(key);
+    const uint8_t *pmask = ptr<uint8_t>(mask);
+    int64_t *pcounts = ptr<int64_t>(counts);
+    double *psums = nv ? ptr<double>(sums) : nullptr;
     int rc;
     void *s = stream();
     Py_BEGIN_ALLOW_THREADS
-    rc = lib.bins(ptr<float>(key), ptr<uint8_t>(mask), T, edges, nb, nv ? vals : nullptr,
-                  (int32_t)nv, ptr<int64_t>(counts), nv ? ptr<double>(sums) : nullptr, w, need, s);
+    rc = lib.bins(pkey, pmask, T, edges, nb, nv ? vals : nullptr, (int32_t)nv, pcounts, psums, w,
+                  need, s);
     Py_END_ALLOW_THREADS
     if (rc != CIS_OK)
         return PyLong_FromLong(rc);
@@ -351,12 +374,18 @@ PyObject *mismatch_diagnostics(PyObject *, PyObject *const *a, Py_ssize_t n)
     Tensor o[5];
     for (Tensor &t : o)
         t = fresh({T}, at::kFloat, dev);
+    const void *pzt = ptr(zt), *pzi = ptr(zi);
+    const int32_t *pids = ptr<int32_t>(ids);
+    const uint8_t *pmask = ptr<uint8_t>(mask);
+    float *po[5];
+    for (int i = 0; i < 5; ++i)
+        po[i] = ptr<float>(o[i]);
+    int32_t *pst = ptr<int32_t>(st);
     int rc;
     void *s = stream();
     Py_BEGIN_ALLOW_THREADS
-    rc = lib.diagnostics(ptr(zt), ptr(zi), code, T, V, ldt, ldi, ptr<int32_t>(ids),
-                         ptr<uint8_t>(mask), &P, ptr<float>(o[0]), ptr<float>(o[1]),
-                         ptr<float>(o[2]), ptr<float>(o[3]), ptr<float>(o[4]), ptr<int32_t>(st), s);
+    rc = lib.diagnostics(pzt, pzi, code, T, V, ldt, ldi, pids, pmask, &P, po[0], po[1], po[2],
+                         po[3], po[4], pst, s);
     Py_END_ALLOW_THREADS
     if (rc != CIS_OK)
         return PyLong_FromLong(rc);

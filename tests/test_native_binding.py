@@ -131,6 +131,27 @@ class TestOnGpu:
                     errors.append((type(e.value), str(e.value)))
             assert errors[0] == errors[1], (i, errors)
 
+    @pytest.mark.parametrize("call", ["loss", "logprobs", "weights", "bins", "diagnostics"])
+    @pytest.mark.parametrize("transform", ["vmap", "grad"])
+    def test_tensors_without_storage(self, call, transform):
+        """A functorch wrapper passes for a plain tensor and has no data pointer: the
+        calls raise what the Python code raises."""
+        P = binding.cis_default_params("cis")
+        z = torch.randn(3, 4, 8, device=DEV)
+        ids, v = torch.zeros(4, dtype=torch.int32, device=DEV), torch.zeros(4, device=DEV)
+        f = {"loss": lambda x: binding.cis_loss_fwd_bwd(x, ids, v, v, P)["loss"],
+             "logprobs": lambda x: binding.cis_token_logprobs(x, ids),
+             "weights": lambda x: binding.cis_weights(x[:, 0].contiguous(), v, P)[0],
+             "bins": lambda x: binding.cis_binned_sums(x[:, 0].contiguous(), [0.0, 1.0])[1],
+             "diagnostics": lambda x: binding.cis_mismatch_diagnostics(x, x, ids, P)["p"]}[call]
+        for python in (False, True):
+            with _python_only() if python else contextlib.nullcontext():
+                with pytest.raises(RuntimeError, match="doesn't have storage"):
+                    if transform == "vmap":
+                        torch.vmap(f)(z)
+                    else:
+                        torch.func.grad(lambda x: f(x).sum())(z[0])
+
 
 def test_host_tensors_are_refused_as_before():
     z, ids, v = torch.zeros(4, 8), torch.zeros(4, dtype=torch.int32), torch.zeros(4)
