@@ -1371,6 +1371,8 @@ static int split_count(int64_t T, int64_t w, int64_t Hd)
     const int64_t n0 = (pairs ? (nM + 1) / 2 : nM) * nH, c0 = (w + lm::kBK - 1) / lm::kBK;
     const int64_t n1 = (pairs ? (nV + 1) / 2 : nV) * nH, c1 = std::max<int64_t>((T + lm::kBK - 1) / lm::kBK, lm::kDwBlocks);
     const int64_t share = (n0 * c0 + n1 * c1) / G;
+    if (share < 1)  // less than a K block a group: nothing to share out
+        return 1;
     int64_t S = (2 * c0 + share - 1) / share;
     S = S < c0 / 16 ? S : c0 / 16;
     S = S < kMaxSplits ? S : kMaxSplits;

@@ -7,6 +7,7 @@ import os
 import re
 import shutil
 import subprocess
+import sys
 
 import pytest
 
@@ -219,3 +220,29 @@ def test_binned_sums_workspace_size(binding):
     assert n.value == (1024 * 64 * 5 * 8 + 255) // 256 * 256 + 256
     for bad in ((-1, 1, 0), (10, 0, 0), (10, 65, 0), (10, 4, 5)):
         assert L.cis_binned_sums_workspace_size(*bad, ctypes.byref(n)) == 1
+
+
+_LMHEAD_PLAN = """
+import ctypes, itertools
+from paper_2609_32444_gb300 import binding as b
+L, p = b.lib(), b.cis_default_params()
+fake, mib = ctypes.c_void_p(0x10000), 1 << 20
+for T, V, H in itertools.product((1, 64, 128, 129, 200, 300, 512, 2000), (1, 256, 1000, 1024, 4096),
+                                 (256, 512, 1024)):
+    sizes = [b.cis_lmhead_workspace_size(T, V, H),
+             b.cis_lmhead_workspace_size_chunk(T, V, H, 256)]
+    for n in sizes + [sizes[0] + 64 * mib]:
+        rc = L.cis_lmhead_fused(fake, fake, T, H, V, fake, fake, None, fake, None, None, 0,
+                                ctypes.byref(p), fake, fake, 0, None, None, None, None, None, None,
+                                ctypes.c_void_p(0x100000), n, None)
+        assert rc == 3, (T, V, H, n, rc)  # planned, then stopped at the first launch
+print("planned")
+"""
+
+
+def test_lmhead_plans_small_calls(binding):
+    """The split of dH's contraction for calls of less than one K block a group of
+    CTAs (a division by their share), in a process that sees no GPU."""
+    r = subprocess.run([sys.executable, "-c", _LMHEAD_PLAN], cwd=ROOT, capture_output=True,
+                       text=True, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""))
+    assert (r.returncode, r.stdout.strip()) == (0, "planned"), r.stderr[-2000:]
