@@ -11,6 +11,7 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import threading
 
 import torch
 
@@ -68,6 +69,7 @@ class CisError(RuntimeError):
 
 _lib = None
 _native = None
+_load_lock = threading.Lock()
 
 
 def library_path() -> str:
@@ -77,8 +79,14 @@ def library_path() -> str:
 def lib():
     """The loaded libcis.so.  Raises if it has not been built."""
     global _lib
-    if _lib is not None:
-        return _lib
+    if _lib is None:
+        with _load_lock:
+            if _lib is None:
+                _lib = _load()  # last: whoever sees it has the native part too
+    return _lib
+
+
+def _load():
     path = _build.LIB_PATH
     if not os.path.exists(path):
         raise ImportError(f"libcis.so is not built ({path}); run __graft_entry__.build()")
@@ -129,7 +137,6 @@ def lib():
                                   ctypes.POINTER(ctypes.c_void_p), i32, P, P, P, ctypes.c_size_t,
                                   P]
     L.cis_binned_sums.restype = ctypes.c_int
-    _lib = L
     _load_native(path)
     return L
 

@@ -3,6 +3,8 @@ both make the call, and the same refusals (what the native part does not take
 goes on to the Python code, whose checks raise).
 """
 import contextlib
+import threading
+import time
 
 import pytest
 import torch
@@ -162,3 +164,42 @@ def test_host_tensors_are_refused_as_before():
               lambda: binding.cis_binned_sums(v, [0.0, 1.0])):
         with pytest.raises(ValueError, match="libcis takes CUDA tensors"):
             f()
+
+
+def test_threads_meet_a_whole_library(monkeypatch):
+    """Calls from several threads while the library loads: none sees it without its
+    native part; after a failed load every call raises the load's error."""
+    z, ids = torch.zeros(4, 8), torch.zeros(4, dtype=torch.int32)
+    load = binding._load_native
+
+    def slow(path):
+        time.sleep(0.2)
+        load(path)
+
+    monkeypatch.setattr(binding, "_load_native", slow)
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_native", None)
+    errors = []
+
+    def call():
+        try:
+            binding.cis_token_logprobs(z, ids)
+        except Exception as e:
+            errors.append((type(e), str(e)))
+
+    threads = [threading.Thread(target=call) for _ in range(3)]
+    for t in threads:
+        t.start()
+        time.sleep(0.02)
+    for t in threads:
+        t.join()
+    assert errors == [(ValueError, "libcis takes CUDA tensors")] * 3
+
+    def fail(path):
+        raise ImportError("no native part")
+
+    monkeypatch.setattr(binding, "_load_native", fail)
+    monkeypatch.setattr(binding, "_lib", None)
+    for _ in range(2):
+        with pytest.raises(ImportError, match="no native part"):
+            binding.cis_token_logprobs(z, ids)
