@@ -12,6 +12,7 @@ import ctypes
 import importlib.util
 import os
 import threading
+import warnings
 
 import torch
 
@@ -141,14 +142,25 @@ def _load():
     return L
 
 
+class _PythonCalls:
+    """In place of the native part: every call is made by the Python code."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _load_native(path):
     """The calls' native part (csrc/cis_native.cpp).  Each of its functions returns
     the call's result, an int (the library's error), or None where its plain case
-    does not apply; the Python code below then makes the call."""
+    does not apply; the Python code below then makes the call.  It is built for one
+    version of Python and PyTorch; under another the Python code makes every call."""
     global _native
     so = _build.native_path()
     if not os.path.exists(so):
-        raise ImportError(f"{so} is not built; run __graft_entry__.build()")
+        warnings.warn(f"{so} is not built (run __graft_entry__.build()): calls go through "
+                      "ctypes, 10 to 30 us slower each", RuntimeWarning, stacklevel=4)
+        _native = _PythonCalls()
+        return
     spec = importlib.util.spec_from_file_location("_cis_native", so)
     m = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(m)

@@ -203,3 +203,14 @@ def test_threads_meet_a_whole_library(monkeypatch):
     for _ in range(2):
         with pytest.raises(ImportError, match="no native part"):
             binding.cis_token_logprobs(z, ids)
+
+
+def test_without_the_native_part(monkeypatch):
+    """A tree built for another PyTorch: a warning, and the Python code's calls."""
+    monkeypatch.setattr(binding._build, "native_path", lambda: "/nonexistent/_cis_native.so")
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_native", None)
+    with pytest.warns(RuntimeWarning, match="is not built"):
+        assert binding.lib() is not None
+    test_host_tensors_are_refused_as_before()
+    assert binding.cis_default_params("tis").mode == binding.CIS_MODE_TIS
