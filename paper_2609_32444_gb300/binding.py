@@ -164,7 +164,7 @@ def _load_native(path):
     spec = importlib.util.spec_from_file_location("_cis_native", so)
     m = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(m)
-    m.init(path)
+    m.init(path, cis_params_t)
     _native = m
 
 

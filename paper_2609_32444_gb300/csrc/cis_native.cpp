@@ -94,11 +94,13 @@ bool flag(PyObject *o, bool &v)
     v = o == Py_True;
     return PyBool_Check(o);
 }
-// The parameter struct behind a ctypes object, copied.
+// The parameter struct behind a ctypes object of the binding's own type, copied.
+PyObject *params_type = nullptr;
 bool params(PyObject *o, cis_params_t &p)
 {
     Py_buffer b;
-    if (strcmp(Py_TYPE(o)->tp_name, "cis_params_t") != 0 || !PyObject_CheckBuffer(o) || PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) {
+    if (reinterpret_cast<PyObject *>(Py_TYPE(o)) != params_type || !PyObject_CheckBuffer(o) ||
+        PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) {
         PyErr_Clear();
         return false;
     }
@@ -393,11 +395,12 @@ PyObject *mismatch_diagnostics(PyObject *, PyObject *const *a, Py_ssize_t n)
     END_HANDLE_TH_ERRORS
 }
 
-// init(path): the library's entry points.
-PyObject *init(PyObject *, PyObject *arg)
+// init(path, params type): the library's entry points, and the type of `params`.
+PyObject *init(PyObject *, PyObject *args)
 {
-    const char *path = PyUnicode_AsUTF8(arg);
-    if (path == nullptr)
+    const char *path;
+    PyObject *type;
+    if (!PyArg_ParseTuple(args, "sO", &path, &type))
         return nullptr;
     void *h = dlopen(path, RTLD_NOW | RTLD_LOCAL);
     if (h == nullptr)
@@ -416,6 +419,8 @@ PyObject *init(PyObject *, PyObject *arg)
     get(lib.diagnostics, "cis_mismatch_diagnostics");
     if (!ok)
         return PyErr_Format(PyExc_ImportError, "%s lacks an entry point", path);
+    Py_INCREF(type);
+    Py_XSETREF(params_type, type);
     return none();
 }
 
@@ -424,7 +429,7 @@ template <typename F> PyCFunction fast(F f)
     return reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(f));
 }
 PyMethodDef methods[] = {
-    {"init", init, METH_O, nullptr},
+    {"init", init, METH_VARARGS, nullptr},
     {"loss_fwd_bwd", fast(loss_fwd_bwd), METH_FASTCALL, nullptr},
     {"token_logprobs", fast(token_logprobs), METH_FASTCALL, nullptr},
     {"weights", fast(weights), METH_FASTCALL, nullptr},

@@ -3,6 +3,7 @@ both make the call, and the same refusals (what the native part does not take
 goes on to the Python code, whose checks raise).
 """
 import contextlib
+import ctypes
 import threading
 import time
 
@@ -132,6 +133,15 @@ class TestOnGpu:
                         f()
                     errors.append((type(e.value), str(e.value)))
             assert errors[0] == errors[1], (i, errors)
+
+    def test_another_type_of_the_same_name_is_refused(self):
+        x = _args()
+        other = type("cis_params_t", (ctypes.Structure,),
+                     {"_fields_": [("b", ctypes.c_uint8 * ctypes.sizeof(binding.cis_params_t))]})
+        for python in (False, True):
+            with _python_only() if python else contextlib.nullcontext():
+                with pytest.raises(ctypes.ArgumentError):
+                    binding.cis_weights(x["lp_infer"], x["lp_infer"], other())
 
     @pytest.mark.parametrize("call", ["loss", "logprobs", "weights", "bins", "diagnostics"])
     @pytest.mark.parametrize("transform", ["vmap", "grad"])
