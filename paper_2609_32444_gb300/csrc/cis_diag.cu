@@ -34,6 +34,8 @@
 //     position reading both rows from global memory with vector loads, twice.
 #include <stdlib.h>
 
+#include <algorithm>
+
 #include "cis_dsmem.cuh"
 #include "cis_kernels.h"
 #include "cis_expacc.cuh"
@@ -92,8 +94,9 @@ __device__ __forceinline__ float elem_weight(float xp, float xq, float p, float 
 // The operator's weight for two candidates at once (f32x2 where the
 // arithmetic allows it); the same values as elem_weight lane by lane.  Where
 // q = 0 the candidate is never drawn and only r = -p counts: every operator
-// here but IcePop and KPop gives a finite f there, so q (f - 1) = 0 without a
-// test; those two can return k = inf and keep the explicit guard.
+// here but IcePop and KPop gives a finite f there (k may be inf or NaN, the bounds
+// are finite: finite_bounds), so q (f - 1) = 0 without a test; those two can
+// return k = inf and keep the explicit guard.
 template <int MODE>
 __device__ __forceinline__ float2 elem_weight2(float2 xp, float2 xq, float2 p, float2 q, float2 k,
                                                const DevParams &P)
@@ -1058,6 +1061,22 @@ cudaError_t launch_stream(const DiagArgs &a, cudaStream_t s)
 
 }  // namespace
 
+// The bounds the kernels compare k with, as finite numbers: one that is infinite (or
+// is in fp32) bounds nothing, and the type's largest value does not either, since k
+// is finite wherever q is not 0.  With lambda infinite, kappa = 1 keeps p = 1 from
+// taking the bound down to 1.
+DevParams finite_bounds(DevParams P)
+{
+    constexpr float top = 3.0e38f;  // 1 + lambda stays finite too
+    if (P.lam_f > top) {
+        P.lam_f = top;
+        P.kappa_f = 1.0f;
+    }
+    P.tis_cap_f = std::min(P.tis_cap_f, top);
+    P.exact_hi_f = std::min(P.exact_hi_f, top);
+    return P;
+}
+
 cudaError_t launch_mismatch(const void *zt, const void *zi, int dtype, int64_t T, int64_t V,
                             int64_t ld_t, int64_t ld_i, const int32_t *ids, const uint8_t *mask,
                             const DevParams &P, float *eps, float *logk, float *p, float *bias2,
@@ -1093,7 +1112,7 @@ extern "C" CIS_API cis_status_t cis_mismatch_diagnostics(
     if (logits_train == nullptr || logits_infer == nullptr || ids == nullptr ||
         eps_out == nullptr)
         return CIS_ERR_INVALID_ARG;
-    const DevParams P = make_dev_params(*params);
+    const DevParams P = finite_bounds(make_dev_params(*params));
     const cudaError_t e =
         launch_mismatch(logits_train, logits_infer, dtype, T, V, ld_train, ld_infer, ids, mask, P,
                         eps_out, logk_out, p_out, bias2_out, dvar_out, dev_status,

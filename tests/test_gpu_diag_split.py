@@ -110,3 +110,33 @@ def test_streaming_kernel_on_short_rows(monkeypatch, T, V, mode):
         logits_for_oracle(z), logits_for_oracle(zi), ids.numpy(),
         oracle.params(mode=getattr(oracle, "MODE_" + mode.upper())), mask=m.numpy())
     _compare(out, ref, z, zi, mode, n_thread(V), m.numpy())
+
+
+@pytest.mark.parametrize("mode,kw", [("cis", {"lam": math.inf}), ("cis", {"lam": 1e39}),
+                                     ("cis", {"lam": math.inf, "kappa": 0.0}),
+                                     ("band", {"lam": math.inf}), ("tis", {"tis_cap": math.inf}),
+                                     ("exact", {"exact_hi": math.inf})])
+@pytest.mark.parametrize("kernel,dtype,V", [("row", torch.float32, 1001), ("row", torch.bfloat16, 1001),
+                                            ("row", torch.bfloat16, 1024),
+                                            ("stream", torch.bfloat16, 1024)])
+def test_operators_without_an_upper_bound(monkeypatch, mode, kw, kernel, dtype, V):
+    """f = k (the band lifts it to (1 + p) / 2 at least), also where candidates of an
+    odd row are paired with none and where both engines mask entries at -inf; the
+    bounds are those of the large finite ones."""
+    monkeypatch.setenv("CIS_DIAG_KERNEL", kernel)
+    z, zi, ids = (x.to(DEV) for x in _rows(9, 5, V, torch.float32, sd=0.3))
+    z, zi, ids = z.to(dtype), zi.to(dtype), ids % 700
+    zi[0, 700:750] = -1e4  # q flushes to 0, k does not exist
+    for masked in (0, V - 800):
+        if masked:
+            z[:, 800:], zi[:, 800:] = -math.inf, -math.inf
+        out = binding.cis_mismatch_diagnostics(z, zi, ids, binding.cis_default_params(mode, **kw))
+        big = {k: min(v, 1e30) if k != "kappa" else 1.0 for k, v in kw.items()}
+        if "lam" in kw:
+            big["kappa"] = 1.0
+        want = binding.cis_mismatch_diagnostics(z, zi, ids, binding.cis_default_params(mode, **big))
+        for k in ("bias2", "dvar"):
+            assert bool(torch.isfinite(out[k]).all()), (k, masked)
+            assert torch.equal(out[k], want[k]), (k, masked)
+        if mode != "band":  # q f = p: no bias but rounding, each of 1024 entries' squared
+            assert bool((out["bias2"][1:] <= V * (8 * U) ** 2).all())
