@@ -130,9 +130,6 @@ template <typename OutT, int kThreads> __device__ __forceinline__ void zero_run(
         dst[tail + threadIdx.x - head] = from_f32<OutT>(0.0f);
 }
 
-// Below this, fl(m log2e) may be off by more than 2^7.
-constexpr float kFarLogit = -1.4e9f;
-
 // Ragged form, rows with maxima beyond z log2e's range (kHugeLogit), or NaN:
 // exponents from z - m.  Rare, and kept out of the kernel's own code (the same
 // in the aligned form costs 0.5% at T=16384, V=151936, so there only threads

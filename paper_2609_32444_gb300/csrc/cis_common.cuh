@@ -34,6 +34,8 @@ constexpr float kLn2 = 0.6931471805599453f;
 // offset stays below 2^-4, that is, for maxima up to this magnitude, and from
 // z - m beyond it (masked entries at -1e9, -1e30 or the type's lowest value).
 constexpr float kHugeLogit = 1e6f;
+// Below this, fl(m log2e) may be off by more than 2^7.
+constexpr float kFarLogit = -1.4e9f;
 
 // Hyper-parameters as the kernels use them: fp32 copies for the fast path and
 // fp64 values (with logs taken on the host) for the certified fallback.

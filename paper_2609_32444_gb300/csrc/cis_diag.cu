@@ -191,17 +191,21 @@ struct DiagArgs {
     int32_t *status;
 };
 
-// Masked rows give 0; valid ones with a bad id NaN, and the status bit.
-__device__ __forceinline__ void no_row(const DiagArgs &a, int64_t t, bool valid)
+__device__ __forceinline__ void write_all(const DiagArgs &a, int64_t t, float v)
 {
-    const float v = valid ? NAN : 0.0f;
-    if (valid)
-        set_status(a.status, kStatusBadId);
     a.eps[t] = v;
     if (a.logk) a.logk[t] = v;
     if (a.p) a.p[t] = v;
     if (a.bias2) a.bias2[t] = v;
     if (a.dvar) a.dvar[t] = v;
+}
+
+// Masked rows give 0; valid ones with a bad id NaN, and the status bit.
+__device__ __forceinline__ void no_row(const DiagArgs &a, int64_t t, bool valid)
+{
+    if (valid)
+        set_status(a.status, kStatusBadId);
+    write_all(a, t, valid ? NAN : 0.0f);
 }
 
 // bias2 and dvar from the nine sums in diag_pair's signs.
@@ -529,13 +533,16 @@ __device__ __forceinline__ uint4 drop_entry(uint4 w, int i)
 // the group (bf16 pairs compared packed, NaN propagating); when it rises the
 // sum is rescaled; the exponentials are 2^{z log2e - cm} with cm = fl(m log2e),
 // the residual m log2e - cm being taken out once per thread at the end.
+// Rounding cm upwards keeps every exponential within 1: a thread that has seen only
+// masked entries, so low that the residual leaves the exponential's range (kFarLogit),
+// holds no infinity, and its sum is left as it is (next to any other entry it is 0).
 __device__ __forceinline__ void pass1_update(uint4 w, float &m, float &cm, float2 &s)
 {
     const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&w);
     const __nv_bfloat162 a = __hmax2_nan(__hmax2_nan(h[0], h[1]), __hmax2_nan(h[2], h[3]));
     const float lm = max_nan(__low2float(a), __high2float(a));
     if (lm > m || lm != lm) {
-        const float ncm = lm * kLog2e;
+        const float ncm = __fmul_ru(lm, kLog2e);
         // cm - ncm < 0 once m is finite (the maximum only rises); while the
         // sum is still empty (m = -inf, cm = 0) a very negative first maximum
         // would make 2^{0 - ncm} overflow and 0 x inf = NaN: the clamp keeps
@@ -562,7 +569,7 @@ __device__ __forceinline__ void pass1_update4(const uint4 (&w)[4], float &m, flo
     const __nv_bfloat162 a = __hmax2_nan(__hmax2_nan(g[0], g[1]), __hmax2_nan(g[2], g[3]));
     const float lm = max_nan(__low2float(a), __high2float(a));
     if (lm > m || lm != lm) {  // as in pass1_update
-        const float ncm = lm * kLog2e;
+        const float ncm = __fmul_ru(lm, kLog2e);
         const float f = ex2_ftz(fminf(cm - ncm, 0.0f));
         s = __fmul2_rn(s, make_float2(f, f));
         m = lm;
@@ -732,6 +739,10 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
                 if (a.logk) a.logk[t] = (float)(rs.lp64() - lp64_q);
                 if (a.p) a.p[t] = expf(rs.lp);
                 finish_sums(a, t, S);
+                // nothing but entries below kFarLogit: the count is lost
+                if ((zyr < kFarLogit && o.m < kFarLogit && o.m > -INFINITY) ||
+                    (zy_q < kFarLogit && om_q < kFarLogit && om_q > -INFINITY))
+                    write_all(a, t, NAN);
             }
             ++rr;
         }
@@ -800,9 +811,9 @@ __global__ void __launch_bounds__(StreamCfg<NW, CPS>::kThreads, CPS)
                 mbar_arrive(smem_u32(&sh.empty[s]));
         }
         MaxSum rp{m_p, s_p.x + s_p.y}, rq{m_q, s_q.x + s_q.y};
-        if (m_p != -INFINITY)
+        if (m_p > kFarLogit)
             rp.s *= ex2_ftz(-fmaf(m_p, kLog2e, -cm_p));
-        if (m_q != -INFINITY)
+        if (m_q > kFarLogit)
             rq.s *= ex2_ftz(-fmaf(m_q, kLog2e, -cm_q));
         rp = warp_ms(rp);
         rq = warp_ms(rq);

@@ -76,7 +76,8 @@ def test_widths_clusters_and_alignments(dtype, T, V):
             assert np.all(d <= t), (k, pad_t)
 
 
-def test_masked_entries(monkeypatch):
+@pytest.mark.parametrize("kernel", ["row", "stream"])
+def test_masked_entries(monkeypatch, kernel):
     """Entries masked in both engines, at -inf and at large negative values: the
     results of the rows without those columns, on both kernels."""
     V, T = 2048, 6
@@ -85,15 +86,21 @@ def test_masked_entries(monkeypatch):
     P = binding.cis_default_params("cis")
     base = _closed_forms(z[:, :500].to(DEV), zi[:, :500].to(DEV), ids.to(DEV), "cis")
     tol = dict(zip(("bias2", "dvar"), diag_error_bounds(z[:, :500], zi[:, :500], "cis", 328)))
-    for low in (-math.inf, torch.finfo(torch.bfloat16).min, -1e30, -1e9):
+    for low in (-math.inf, torch.finfo(torch.bfloat16).min, -1e30, -1e10, -1e9):
         a, b = z.clone().to(DEV), zi.clone().to(DEV)
         a[:, 500:], b[:, 500:] = low, low
-        monkeypatch.setenv("CIS_DIAG_KERNEL", "row")
+        monkeypatch.setenv("CIS_DIAG_KERNEL", kernel)
         out = binding.cis_mismatch_diagnostics(a, b, ids.to(DEV), P)
         for k in ("bias2", "dvar", "logk"):
             w = base[k].cpu().numpy()
             d = np.abs(out[k].double().cpu().numpy() - w)
             assert np.all(d <= tol.get(k, 4e-5) + 2.0 ** -20 * np.abs(w)), (k, low)
+    if kernel == "stream":  # a row at such a value throughout, the sampled entry too
+        a, b = z.clone().to(DEV), zi.clone().to(DEV)
+        a[0], b[1], a[2] = -1e10, torch.finfo(torch.bfloat16).min, -(2.0 ** 32)
+        out = binding.cis_mismatch_diagnostics(a, b, ids.to(DEV), P)
+        for k, v in out.items():
+            assert bool(torch.isnan(v[:3]).all()) and bool(torch.isfinite(v[3:]).all()), k
 
 
 @pytest.mark.parametrize("T,V,mode", [(700, 1024, "cis"), (400, 2056, "icepop"), (160, 64, "kpop")])
