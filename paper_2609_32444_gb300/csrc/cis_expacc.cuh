@@ -16,14 +16,15 @@
 namespace cis {
 namespace {
 
-// 2^x for 0 <= x < 1, to fp32 rounding.
+// 2^x for -1/8 < x < 9/8, to fp32 rounding.
 __device__ __forceinline__ float exp2_accurate(float x)
 {
     constexpr float ln2_lo = (float)(0.693147180559945309417 - (double)kLn2);
-    const float y = x - 1.0f, h = y * kLn2;  // exact, then 2^x = 2 e^{y ln 2}
+    const bool up = x > 0.5f;
+    const float y = up ? x - 1.0f : x, h = y * kLn2;  // exact, then 2^x = (2) e^{y ln 2}
     float lo;
     const float hi = exp_pair(h, fmaf(y, kLn2, -h) + y * ln2_lo, lo);
-    return 2.0f * (hi + lo);
+    return up ? 2.0f * (hi + lo) : hi + lo;
 }
 
 // Running (m, S[, U]) of one thread in the exponent form above; U = sum e x with
@@ -72,12 +73,13 @@ template <bool kEnt> struct ExpAcc {
             U = fmaf(e, fmaxf(x, -1024.0f), U);
     }
     // As sums of e^{z - m}: m log2e - c is exact (an FMA), between -1 and 0 but
-    // for its rounding.
+    // for the rounding of the product that c was taken from (2^-4 at most): above 0
+    // where that product was rounded down to a whole number.
     __device__ __forceinline__ MaxSumU result() const
     {
         if (m == -INFINITY)
             return {m, 0.0f, 0.0f};
-        const float err = fast() ? fminf(fmaf(m, kLog2e, -c), 0.0f) : 0.0f;
+        const float err = fast() ? fmaf(m, kLog2e, -c) : 0.0f;
         const float f = fast() ? exp2_accurate(-err) : 1.0f;
         return {m, S * f, kEnt ? f * kLn2 * fmaf(-err, S, U) : 0.0f};
     }

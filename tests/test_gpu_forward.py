@@ -6,6 +6,7 @@ the entropy, whose terms are bounded by log V, 2e-5 (1 + log V).
 """
 import math
 
+import numpy as np
 import pytest
 import torch
 
@@ -93,3 +94,37 @@ def test_rows_of_masked_entries(dtype, fill):
         return
     z[3, :5] = 0.25
     _check(z, ids)
+
+
+def _whole_products(lo, hi, n):
+    """fp32 values m in [lo, hi) whose product with log2e rounds down to a whole number,
+    those with the largest remainder."""
+    l2e = np.float32(math.log2(math.e))
+    k = np.arange(int(lo * float(l2e)) + 1, int(hi * float(l2e)), dtype=np.float64)
+    m = (k / np.float64(l2e)).astype(np.float32)
+    best = []
+    for c in (m, np.nextafter(m, np.float32(np.inf)), np.nextafter(m, np.float32(0))):
+        over = c.astype(np.float64) * np.float64(l2e) - k
+        over[(c * l2e).astype(np.float64) != k] = 0
+        best += list(zip(over, c))
+    return [float(c) for _, c in sorted(best)[-n:]]
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_maxima_whose_offset_is_rounded_down(dtype):
+    """16 entries share the maximum, the others are out of reach: log p = -log 16,
+    whatever the maximum (also as p of the diagnostics)."""
+    m = [124928.0, 448512.0]
+    if dtype == torch.float32:
+        m += _whole_products(100, 1000, 3) + _whole_products(1e5, 9e5, 3)
+    V = 2050
+    z = torch.tensor(m, device=DEV).view(-1, 1).expand(len(m), V).to(dtype).contiguous()
+    z[:, 16:] *= 0.5
+    ids = torch.arange(len(m), dtype=torch.int32, device=DEV)
+    lp, lse, ent = binding.cis_token_logprobs(z, ids, want_lse=True, want_entropy=True)
+    p = binding.cis_mismatch_diagnostics(z, z, ids, binding.cis_default_params("cis"))["p"]
+    want = math.log(16)
+    assert bool(((lp + want).abs() <= 2e-5).all()) and bool(((16 * p - 1).abs() <= 2e-5).all())
+    assert bool(((ent - want).abs() <= 2e-5 * (1 + want)).all())
+    x = z[:, 0].double()
+    assert bool(((lse.double() - x - want).abs() <= 2e-5 + 2.0 ** -21 * x).all())
