@@ -33,12 +33,15 @@ template <bool kEnt> struct ExpAcc {
     float m = -INFINITY, c = -INFINITY, S = 0.0f, U = 0.0f;
 
     __device__ __forceinline__ bool fast() const { return fabsf(m) < kHugeLogit; }
-    // Raise the offset to a larger (or NaN) maximum.
+    // Raise the offset to a larger (or NaN) maximum, in whichever of the two forms
+    // each of the maxima has.
     __device__ __forceinline__ void raise(float mx)
     {
         if (mx > m || mx != mx) {
             const float c1 = ceilf(mx * kLog2e);
-            const float d = fast() && fabsf(mx) < kHugeLogit ? c - c1 : (m - mx) * kLog2e;
+            const bool now = fast(), then = fabsf(mx) < kHugeLogit;
+            const float d = now ? (then ? c - c1 : fmaf(-mx, kLog2e, c))
+                                : (then ? fmaf(m, kLog2e, -c1) : (m - mx) * kLog2e);
             const float f = ex2_ftz(d);
             if (kEnt)
                 U = f == 0.0f ? 0.0f : fmaf(d, S, U) * f;
@@ -112,7 +115,7 @@ __device__ __forceinline__ MaxSumU block_exp(const ExpAcc<kEnt> &acc, MaxSumU *r
     MaxSumU t = acc.result();
     float d, f;
     if (all.fast()) {
-        d = acc.fast() ? acc.c - all.c : (acc.m - M) * kLog2e;
+        d = acc.fast() ? acc.c - all.c : fmaf(acc.m, kLog2e, -all.c);
         t.s = acc.S;
         t.u = acc.U;
     } else {

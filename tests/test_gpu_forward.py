@@ -128,3 +128,17 @@ def test_maxima_whose_offset_is_rounded_down(dtype):
     assert bool(((ent - want).abs() <= 2e-5 * (1 + want)).all())
     x = z[:, 0].double()
     assert bool(((lse.double() - x - want).abs() <= 2e-5 + 2.0 ** -21 * x).all())
+
+
+@pytest.mark.parametrize("sign", [1, -1])
+def test_maxima_on_both_sides_of_the_exponents_two_forms(sign):
+    """fp32 rows with entries a step below and above 1e6 (the first or the last part of
+    a row, or every other vector): a thread's maxima, and the threads', cross over."""
+    T, V = 3, 12000
+    lo, hi = (999999.9375, 1000000.0625) if sign > 0 else (-1000000.0625, -999999.9375)
+    z = torch.full((T, V), lo, device=DEV)
+    z[0, V // 2:] = hi
+    z[1, :V // 2] = hi
+    z[2].view(-1, 2, 4)[:, 1] = hi
+    _check(z, torch.tensor([3, 3, 3], dtype=torch.int32, device=DEV))
+    _check(z[:, :1030].contiguous(), torch.tensor([3, 3, 3], dtype=torch.int32, device=DEV))
