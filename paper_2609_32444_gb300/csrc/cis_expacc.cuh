@@ -50,11 +50,13 @@ template <bool kEnt> struct ExpAcc {
             c = c1;
         }
     }
-    // Add 8 entries (those left out are -inf); the offset covers them.
-    __device__ __forceinline__ void add8(const float2 (&z)[4])
+    // The sum of 8 entries (those left out are -inf), as a pair, and of e x in u; the
+    // offset covers them.
+    __device__ __forceinline__ float2 sum8(const float2 (&z)[4], float2 &u) const
     {
         const float2 l2 = make_float2(kLog2e, kLog2e), nc = make_float2(-c, -c);
-        float2 e[4], u = make_float2(0.0f, 0.0f);
+        float2 e[4];
+        u = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float2 x = __ffma2_rn(z[i], l2, nc);
@@ -62,10 +64,25 @@ template <bool kEnt> struct ExpAcc {
             if (kEnt)  // an entry at -inf adds 0, not 0 * -inf
                 u = __ffma2_rn(e[i], make_float2(fmaxf(x.x, -1024.0f), fmaxf(x.y, -1024.0f)), u);
         }
-        const float2 s = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
-        S += s.x + s.y;
+        return __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
+    }
+    // Add N such sums, to each other first: the growing sum is rounded at each addition,
+    // and next to one large entry a thread's many small ones are lost to it, the more the
+    // smaller they come (V=151936, a likely token and another one sampled: log p off by
+    // 1.1e-7 on average; 3.4e-7 a vector at a time).
+    template <int N> __device__ __forceinline__ void grow(float2 (&s)[N], float2 (&u)[N])
+    {
+#pragma unroll
+        for (int w = 1; w < N; w <<= 1)
+#pragma unroll
+            for (int k = 0; k + w < N; k += 2 * w) {
+                s[k] = __fadd2_rn(s[k], s[k + w]);
+                if (kEnt)
+                    u[k] = __fadd2_rn(u[k], u[k + w]);
+            }
+        S += s[0].x + s[0].y;
         if (kEnt)
-            U += u.x + u.y;
+            U += u[0].x + u[0].y;
     }
     // One entry, covered by the offset, in either form.
     __device__ __forceinline__ void add_entry(float z)
@@ -223,6 +240,7 @@ template <int N> __device__ __forceinline__ float vec_max(const Vec<float> (&v)[
 template <bool kEnt, int N>
 __device__ __forceinline__ void add_vecs(ExpAcc<kEnt> &acc, const Vec<__nv_bfloat16> (&v)[N])
 {
+    float2 s[N], u[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const uint4 q = v[k].q;
@@ -230,13 +248,15 @@ __device__ __forceinline__ void add_vecs(ExpAcc<kEnt> &acc, const Vec<__nv_bfloa
                              make_float2(bf16_lo(q.y), bf16_hi(q.y)),
                              make_float2(bf16_lo(q.z), bf16_hi(q.z)),
                              make_float2(bf16_lo(q.w), bf16_hi(q.w))};
-        acc.add8(z);
+        s[k] = acc.sum8(z, u[k]);
     }
+    acc.grow(s, u);
 }
 template <bool kEnt, int N>
 __device__ __forceinline__ void add_vecs(ExpAcc<kEnt> &acc, const Vec<float> (&v)[N])
 {
     const float2 none = make_float2(-INFINITY, -INFINITY);
+    float2 s[(N + 1) / 2], u[(N + 1) / 2];
 #pragma unroll
     for (int k = 0; k < N; k += 2) {
         const uint4 a = v[k].q, b = v[k + 1 < N ? k + 1 : k].q;
@@ -246,8 +266,9 @@ __device__ __forceinline__ void add_vecs(ExpAcc<kEnt> &acc, const Vec<float> (&v
                                        : none,
                              k + 1 < N ? make_float2(__uint_as_float(b.z), __uint_as_float(b.w))
                                        : none};
-        acc.add8(z);
+        s[k / 2] = acc.sum8(z, u[k / 2]);
     }
+    acc.grow(s, u);
 }
 
 template <bool kEnt, int N, typename InT>

@@ -142,3 +142,20 @@ def test_maxima_on_both_sides_of_the_exponents_two_forms(sign):
     z[2].view(-1, 2, 4)[:, 1] = hi
     _check(z, torch.tensor([3, 3, 3], dtype=torch.int32, device=DEV))
     _check(z[:, :1030].contiguous(), torch.tensor([3, 3, 3], dtype=torch.int32, device=DEV))
+
+
+@pytest.mark.parametrize("dtype,z0", [(torch.bfloat16, -19.375), (torch.float32, -18.715)])
+@pytest.mark.parametrize("T", [40, 1300])
+def test_small_entries_next_to_a_large_one(dtype, z0, T):
+    """One entry is 1 and the others so small that a vector of them rounds away against
+    it, but not a batch of four, which is one step of 2^-23 within 3%: a thread's 75
+    batches at most (fp32) lose 75 * 0.03 * 2^-23 = 2.7e-7, and as much again is left for
+    the exponentials; a thread that loses them all loses 4e-6."""
+    V = 151936
+    z = torch.full((T, V), z0, dtype=dtype, device=DEV)
+    z[:, 5] = 0.0
+    ids = torch.full((T,), 9, dtype=torch.int32, device=DEV)
+    lp = binding.cis_token_logprobs(z, ids).double()
+    x = float(z[0, 9])
+    want = x - math.log1p((V - 1) * math.exp(x))
+    assert float((lp - want).abs().max()) <= 5.3e-7 + 2.0 ** -24 * abs(want)
