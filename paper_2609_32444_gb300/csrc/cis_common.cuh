@@ -778,7 +778,8 @@ __device__ __forceinline__ float row_entropy(MaxSumU o, float zy, float lp)
     const float d = u + (ue + dl);  // logit p, as in row_scalars
     // log(1 - p) = -softplus(d)
     const float l1mp = d > 0.0f ? -(d + log1pf(expf(-d))) : -log1pf(expf(d));
-    const float p = expf(lp), q = expf(l1mp);
+    // 1 - p from p where that is small: one rounding, and it scales nearly all of H
+    const float p = expf(lp), q = p < 0.5f ? 1.0f - p : expf(l1mp);
     const float hq = ls - o.u / o.s;
     const float plp = p == 0.0f ? 0.0f : p * lp;      // 0 log 0 = 0
     const float qlq = q == 0.0f ? 0.0f : q * l1mp;
