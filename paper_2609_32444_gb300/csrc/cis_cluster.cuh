@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(kThreads) cis_fused_cluster_kernel(const __gri
         }
         float c, omp, bias_log2, scale = 1.0f;
         DirectRow dw;
-        direct = !has_old && row_direct(o, zy, dw);
+        direct = !has_old && row_direct<(kAll || kRagged)>(o, zy, dw);
         if (direct && !given)
             direct = weight_direct<kAll, kAll || kRagged>(dw, linf, qinv, qinv_lo, kq, a.P, tw.w, tw.trunc);
         if (direct) {

@@ -593,6 +593,8 @@ struct DirectRow {
     float E;    // e^{m' - z_y}
     float p;
 };
+// kFine: p to an ulp (a Newton step), and 1 - p from it where p is small.
+template <bool kFine>
 __device__ __forceinline__ bool row_direct(MaxSum o, float zy, DirectRow &r)
 {
     float dl;
@@ -602,8 +604,11 @@ __device__ __forceinline__ bool row_direct(MaxSum o, float zy, DirectRow &r)
     const float e = expf(dh);
     r.E = fmaf(e, dl, e);
     r.t = o.s * r.E;
-    r.p = __fdividef(1.0f, 1.0f + r.t);
-    r.omp = r.t * r.p;
+    const float x = 1.0f + r.t;
+    r.p = __fdividef(1.0f, x);
+    if (kFine)
+        r.p = fmaf(r.p, fmaf(-x, r.p, 1.0f), r.p);
+    r.omp = kFine && r.t >= 1.0f ? 1.0f - r.p : r.t * r.p;
     return true;
 }
 
@@ -618,9 +623,16 @@ __device__ __forceinline__ bool weight_direct(const DirectRow &d, float linf, fl
 {
     if (!(linf >= -70.0f))
         return false;
-    // log k, which token_weight takes them from, is rounded less often than p / q:
-    // 1 / q as a pair makes up for it (not in the plain aligned form)
-    const float k = kPair ? fmaf(d.p, qinv, d.p * qinv_lo) : d.p * qinv;
+    // log k, which token_weight takes them from, is rounded less often than p / q: 1 / q
+    // as a pair, and p as one where it is above a half (1 - p is the accurate value
+    // there), make up for it (not in the plain aligned form)
+    float k = d.p * qinv;
+    if (kPair) {
+        const bool high = d.t < 1.0f;
+        const float ph = high ? 1.0f - d.omp : d.p;
+        const float pl = high ? (1.0f - ph) - d.omp : 0.0f;
+        k = fmaf(ph, qinv, fmaf(ph, qinv_lo, pl * qinv));
+    }
     trunc = 0;
     w = k;
     switch (P.mode) {

@@ -121,3 +121,34 @@ def test_rows_at_the_lowest_value(dtype, V, low):
                                        torch.ones(1, device=DEV),
                                        binding.cis_default_params("none"))
         assert bool(torch.isnan(out["lp"]).all())
+
+
+def test_weights_and_sampled_gradients_keep_their_roundings():
+    """The weights of likely tokens (p > 0.97) and the sampled entry's gradient of
+    unlikely ones (p < 0.02), formed without logarithms, on fp32 rows.  k = p / q: 1 - p
+    carries a few fp32 roundings, which count by (1 - p) / p < 0.03, 1 / q is a pair, and
+    the product is rounded once: 1.5 roundings.  c (p - 1) with c = 1 / T a power of two:
+    the few roundings of p count by 0.02, and 1 - p is rounded once: 1.2."""
+    T, V = 4096, 1001
+    g = torch.Generator(device=DEV)
+    g.manual_seed(3)
+    z = torch.randn((T, V), generator=g, device=DEV) * 2
+    ids = torch.randint(0, V, (T,), generator=g, device=DEV)
+    r = torch.arange(T, device=DEV)
+    odds = torch.where(r % 2 == 0, 3.6 + 6 * torch.rand(T, generator=g, device=DEV),
+                       -4.0 - 6 * torch.rand(T, generator=g, device=DEV))
+    rest = z.clone()
+    rest[r, ids] = -math.inf
+    z[r, ids] = torch.logsumexp(rest, 1) + odds
+    d = z.double()
+    d[r, ids] = -math.inf
+    lp = -torch.nn.functional.softplus(torch.logsumexp(d, 1) - z[r, ids].double())
+    linf = (lp + 0.1 * torch.randn(T, generator=g, device=DEV)).clamp(max=-1e-4).float()
+    adv = torch.ones(T, device=DEV)
+    high, u = r % 2 == 0, 2.0 ** -24
+    out = binding.cis_loss_fwd_bwd(z, ids.int(), linf, adv, binding.cis_default_params("exact"))
+    k = (lp - linf.double()).exp()
+    assert float(((out["w"].double() - k).abs() / k)[high].max()) <= 1.5 * u
+    out = binding.cis_loss_fwd_bwd(z, ids.int(), linf, adv, binding.cis_default_params("none"))
+    got, want = out["dlogits"][r, ids].double(), torch.expm1(lp) / T
+    assert float(((got - want) / want).abs()[~high].max()) <= 1.2 * u
