@@ -55,7 +55,8 @@
  *       4 dH, 8 dW; default 15) picks the GEMMs that run on 2-CTA clusters
  *       sharing B tiles by multicast, and CIS_LMHEAD_DUAL=0 runs a chunk's
  *       dH and dW as two launches instead of one.  Neither changes a result
- *       bit.  Read at each call.
+ *       bit.  Read at each call.  In a process of a job of several ranks
+ *       (WORLD_SIZE above 1) no GEMM uses multicast, whatever CIS_LMHEAD_MC.
  */
 #ifndef CIS_H
 #define CIS_H

@@ -1259,9 +1259,14 @@ static bool dual_on()
 // Which GEMMs run on 2-CTA multicast clusters: a bit mask over FWD (1), DZ
 // (2), DH (4) and DW (8); all by default, CIS_LMHEAD_MC overrides it.  The
 // results are bit for bit the same either way: each tile's MMAs and epilogue
-// are unchanged, only where half of B comes from differs.
+// are unchanged, only where half of B comes from differs.  Multicast loads are for
+// programs on one GPU (their tensor maps cover that GPU's memory alone): a process
+// of a job of several ranks (WORLD_SIZE above 1) does without, whatever the mask.
 static int mc_mask()
 {
+    const char *w = getenv("WORLD_SIZE");
+    if (w && atol(w) > 1)
+        return 0;
     const char *e = getenv("CIS_LMHEAD_MC");
     return e && e[0] ? (int)strtol(e, nullptr, 0) & 15 : 15;
 }

@@ -182,6 +182,9 @@ def test_lmhead_multicast_clusters_bit_identical(monkeypatch, T, V, H, chunk, gr
             monkeypatch.setenv("CIS_LMHEAD_MC", mc)
             monkeypatch.setenv("CIS_LMHEAD_DUAL", dual)
             outs[mc, dual] = _run(b, grad_dtype=grad, chunk=chunk)
+    monkeypatch.setenv("CIS_LMHEAD_MC", "15")
+    monkeypatch.setenv("WORLD_SIZE", "2")  # one rank of several: single CTAs
+    outs["15", "of two ranks"] = _run(b, grad_dtype=grad, chunk=chunk)
     torch.cuda.synchronize()
     a = outs["15", "1"]
     for key, r in outs.items():
