@@ -47,23 +47,14 @@ namespace {
 constexpr int kDiagThreads = 512;
 constexpr int kNSums = 9;
 
-// The operator's weight for one candidate j in fp32 (a statistic: no fp64
-// decision fallback), from the exponents xp = log2 p_j, xq = log2 q_j, p_j and
+// The weight of IcePop or KPop for one candidate j in fp32 (a statistic: no fp64
+// decision fallback), from the exponents xp = log2 p_j, xq = log2 q_j and
 // k_j = 2^{xp - xq}; MODE is a compile-time cis_mode_t, so the per-candidate
 // loop has no branch on it.
 template <int MODE>
-__device__ __forceinline__ float elem_weight(float xp, float xq, float p, float k,
-                                             const DevParams &P)
+__device__ __forceinline__ float elem_weight(float xp, float xq, float k, const DevParams &P)
 {
-    if (MODE == CIS_MODE_CIS)
-        return fminf(k, fmaf(P.lam_f, fmaxf(1.0f - p, P.kappa_f), 1.0f));
-    if (MODE == CIS_MODE_TIS)
-        return fminf(k, P.tis_cap_f);
-    if (MODE == CIS_MODE_EXACT)
-        return fminf(fmaxf(k, P.exact_lo_f), P.exact_hi_f);
-    if (MODE == CIS_MODE_BAND)
-        return fmaxf(fminf(k, fmaf(P.lam_f, fmaxf(1.0f - p, P.kappa_f), 1.0f)),
-                     0.5f * (1.0f + p));
+    static_assert(MODE == CIS_MODE_ICEPOP || MODE == CIS_MODE_KPOP, "the others are packed");
     if (MODE == CIS_MODE_ICEPOP) {  // log k against the band, in log2 units
         const float lk2 = xp - xq;
         return (lk2 < (float)(P.log_icepop_lo * 1.4426950408889634) ||
@@ -71,28 +62,25 @@ __device__ __forceinline__ float elem_weight(float xp, float xq, float p, float 
                    ? 0.0f
                    : k;
     }
-    if (MODE == CIS_MODE_KPOP) {
-        // binary KL both ways with p, q clamped to [1e-8, 1 - 1e-8], in the
-        // log domain so that 1 - 1e-8 stays representable
-        const float lp = xp * kLn2, lq = xq * kLn2;
-        const float lo = -18.420680743952367f;  // log 1e-8
-        const float hi = -1e-8f;                // log(1 - 1e-8)
-        const float l1p = logf(-expm1f(lp)), l1q = logf(-expm1f(lq));
-        const float a = fminf(fmaxf(lp, lo), hi), b = fminf(fmaxf(lq, lo), hi);
-        const float a1 = fminf(fmaxf(l1p, lo), hi), b1 = fminf(fmaxf(l1q, lo), hi);
-        const float pa = expf(a), qb = expf(b), pa1 = expf(a1), qb1 = expf(b1);
-        const float kpq = pa * (a - b) + pa1 * (a1 - b1);
-        const float kqp = qb * (b - a) + qb1 * (b1 - a1);
-        return fmaxf(kpq, kqp) > (float)P.kpop_phi ? 0.0f : k;
-    }
-    return 1.0f;  // CIS_MODE_NONE
+    // KPop: binary KL both ways with p, q clamped to [1e-8, 1 - 1e-8], in the log
+    // domain so that 1 - 1e-8 stays representable
+    const float lp = xp * kLn2, lq = xq * kLn2;
+    const float lo = -18.420680743952367f;  // log 1e-8
+    const float hi = -1e-8f;                // log(1 - 1e-8)
+    const float l1p = logf(-expm1f(lp)), l1q = logf(-expm1f(lq));
+    const float a = fminf(fmaxf(lp, lo), hi), b = fminf(fmaxf(lq, lo), hi);
+    const float a1 = fminf(fmaxf(l1p, lo), hi), b1 = fminf(fmaxf(l1q, lo), hi);
+    const float pa = expf(a), qb = expf(b), pa1 = expf(a1), qb1 = expf(b1);
+    const float kpq = pa * (a - b) + pa1 * (a1 - b1);
+    const float kqp = qb * (b - a) + qb1 * (b1 - a1);
+    return fmaxf(kpq, kqp) > (float)P.kpop_phi ? 0.0f : k;
 }
 
 // ---------------------------------------------------------------------------
 // Streaming kernel.
 
 // The operator's weight for two candidates at once (f32x2 where the
-// arithmetic allows it); the same values as elem_weight lane by lane.  Where
+// arithmetic allows it).  Where
 // q = 0 the candidate is never drawn and only r = -p counts: every operator
 // here but IcePop and KPop gives a finite f there (k may be inf or NaN, the bounds
 // are finite: finite_bounds), so q (f - 1) = 0 without a test; those two can
@@ -121,9 +109,9 @@ __device__ __forceinline__ float2 elem_weight2(float2 xp, float2 xq, float2 p, f
     if (MODE == CIS_MODE_EXACT)
         return make_float2(fminf(fmaxf(k.x, P.exact_lo_f), P.exact_hi_f),
                            fminf(fmaxf(k.y, P.exact_lo_f), P.exact_hi_f));
-    if (MODE == CIS_MODE_ICEPOP || MODE == CIS_MODE_KPOP)
-        return make_float2(q.x > 0.0f ? elem_weight<MODE>(xp.x, xq.x, p.x, k.x, P) : 1.0f,
-                           q.y > 0.0f ? elem_weight<MODE>(xp.y, xq.y, p.y, k.y, P) : 1.0f);
+    if constexpr (MODE == CIS_MODE_ICEPOP || MODE == CIS_MODE_KPOP)
+        return make_float2(q.x > 0.0f ? elem_weight<MODE>(xp.x, xq.x, k.x, P) : 1.0f,
+                           q.y > 0.0f ? elem_weight<MODE>(xp.y, xq.y, k.y, P) : 1.0f);
     return one;  // CIS_MODE_NONE
 }
 

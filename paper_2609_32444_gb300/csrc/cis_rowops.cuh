@@ -1,6 +1,6 @@
 // cis_rowops.cuh -- row-streaming building blocks of the row kernel
-// (cis_rowwise.cu): a running (max, sum of exponentials) -- optionally with the entropy term -- over the
-// entries j != y of one row, read with 16-byte vector loads.
+// (cis_rowwise.cu): a running (max, sum of exponentials), optionally with the entropy
+// term, over the entries j != y of one row, read with 16-byte vector loads.
 #pragma once
 
 #include "cis_common.cuh"
@@ -64,12 +64,6 @@ __device__ __forceinline__ void ms_update(MaxSumU &acc, const float (&z)[EV], in
     acc.u = u;
 }
 
-template <typename InT, bool kStream>
-__device__ __forceinline__ uint4 load16(const uint4 *p)
-{
-    return kStream ? __ldcs(p) : __ldg(p);
-}
-
 // Unpack one 16-byte vector into floats.
 __device__ __forceinline__ void unpack(uint4 q, float (&z)[8])
 {
@@ -85,7 +79,7 @@ __device__ __forceinline__ void unpack(uint4 q, float (&z)[4])
 }
 
 // This thread's (m, s) -- or (m, s, u) -- over entries j != y of one row.
-template <typename InT, bool kStream, typename Acc = MaxSum, int NT = 256>
+template <typename InT, int NT, typename Acc = MaxSum>
 __device__ Acc row_stats(const InT *row, int64_t V, int64_t y)
 {
     constexpr int EV = 16 / sizeof(InT);
@@ -97,7 +91,7 @@ __device__ Acc row_stats(const InT *row, int64_t V, int64_t y)
         const uint4 *rv = reinterpret_cast<const uint4 *>(row);
         for (int64_t v = threadIdx.x; v < nvec; v += NT) {
             float z[EV];
-            unpack(load16<InT, kStream>(rv + v), z);
+            unpack(__ldg(rv + v), z);
             const int64_t rel = y - v * EV;
             ms_update<EV>(acc, z, (rel >= 0 && rel < EV) ? (int)rel : -1);
         }

@@ -68,10 +68,10 @@ __global__ void __launch_bounds__(kRowThreads) cis_fused_row_kernel(const __grid
     MaxSum o;
     MaxSumU ou{0.0f, 0.0f, 0.0f};
     if constexpr (kEnt) {
-        ou = block_msu<kRowThreads>(row_stats<InT, false, MaxSumU>(row, a.V, y), sh.red);
+        ou = block_msu<kRowThreads>(row_stats<InT, kRowThreads, MaxSumU>(row, a.V, y), sh.red);
         o = MaxSum{ou.m, ou.s};
     } else {
-        o = block_ms<kRowThreads>(row_stats<InT, false>(row, a.V, y), sh.red);
+        o = block_ms<kRowThreads>(row_stats<InT, kRowThreads>(row, a.V, y), sh.red);
     }
     if (threadIdx.x == 0) {
         const RowScalars rs = row_scalars(o, to_f32(row[y]));
