@@ -43,14 +43,23 @@
  *     defaults are the measured best.  Other settings change summation
  *     orders, never the tolerances.
  *       CIS_SLICE_KB (8..200, default 80), CIS_CLUSTER (1..8) and
- *       CIS_CLUSTER_THREADS (128, 256, 384 or 512; default 256) set the
- *       fused pass's slice target, cluster size and CTA width.  By default a
- *       row of 40 to 80 KB runs on two CTAs of 128 threads (CIS_SLICE_KB or
- *       CIS_CLUSTER turns that off).  They are read once per process.
- *       CIS_DIAG_WARPS (16 or 24 with one CTA per SM, 8 with two, 4 with
- *       four; default 16) and CIS_DIAG_SLOT_GROUPS (>= 1) set the diagnostics
- *       kernel's width and ring-slot size, and CIS_DIAG_KERNEL=row selects its
- *       one-CTA kernel.  They are read at each call.
+ *       CIS_CLUSTER_THREADS (128, 256, 384 or 512) set the fused pass's slice
+ *       target, cluster size and CTA width.  By default a CTA has 256 threads,
+ *       or 128 for fp32 rows and for rows of at most 16384 entries in one CTA,
+ *       and a row of 40 to 80 KB runs on two CTAs of 128 threads (CIS_SLICE_KB
+ *       or CIS_CLUSTER turns the last off).  384 and 512 are for 16-byte
+ *       aligned rows with V a multiple of 8, without lp_old and entropy_out,
+ *       under CIS, TIS, EXACT and NONE; other calls take 256 in their place
+ *       (fp32 rows with entropy_out: 128).  They are read once per process.
+ *       CIS_DIAG_KERNEL=row selects the diagnostics' kernel for any row, and
+ *       =stream the streaming one (for bf16, 16-byte aligned rows, V a
+ *       multiple of 8) at any size.  CIS_DIAG_WARPS (16 or 24 with one CTA per
+ *       SM, 8 with two, 4 with four; default 16) and CIS_DIAG_SLOT_GROUPS
+ *       (>= 1) set the streaming kernel's width and ring-slot size, and select
+ *       it as =stream does.  They are read at each call.
+ *       CIS_LMHEAD_PACK=1 leaves masked tokens out of the LM head's products in
+ *       every call of more than 128 tokens, =0 in none (default: from
+ *       T V H = 8e10 on).  Read at each call.
  *       CIS_LMHEAD_MC (a bit mask over the LM head's GEMMs: 1 logits, 2 dz,
  *       4 dH, 8 dW; default 15) picks the GEMMs that run on 2-CTA clusters
  *       sharing B tiles by multicast, and CIS_LMHEAD_DUAL=0 runs a chunk's

@@ -3,14 +3,15 @@ against the fp64 oracle, and at full vocabulary size against closed forms.
 
 Both kernels are covered: the streaming kernel (bf16 rows with V a multiple
 of 8; CIS_DIAG_SLOT_GROUPS shrinks its ring slots so that short rows still
-span many slots, wrap the ring and end in a partial slot) and the one-CTA
+span many slots, wrap the ring and end in a partial slot) and the split
 kernel (fp32 or ragged rows, or bf16 with CIS_DIAG_KERNEL=row).
 
 Tolerances, from the arithmetic: eps and log k come from fp32 row sums (as log
 p does in the token pass: 2e-5 plus 4 ulps).  The bias and the variance
 increase are fp64 combinations of nine sums over the V candidates (P2, R2, RP,
 C1 .. C5, QP: see the kernel), each of fp32 terms summed in fp32 by every
-thread over its n_t candidates, then in fp64.  So each sum S carries
+thread over its n_t candidates and by every warp over its lanes, then in fp64.
+So each sum S carries
   |dS| <= e_c sum_j dterm_j + (n_t + 8) 2^-24 sum_j |term_j|,
 where e_c = (64 + n_t) 2^-24 is one candidate's relative error (its exponent's
 rounding for |exponent| <= 60 -- candidates further out weigh less than 2^-60
@@ -64,8 +65,8 @@ def n_thread(V, slot_groups=2048, threads=512):
     """Most candidates one thread sums in a row: the streaming kernel's ring
     slots of `slot_groups` groups of 8 (each of `threads` threads takes
     ceil(slot_groups / threads) groups of a slot; the defaults are its layout
-    of 16 consumer warps); this also bounds the one-CTA kernel's 512 threads
-    with 8-wide loads."""
+    of 16 consumer warps); this also bounds the split kernel with 512 threads,
+    and with its 128 for rows of at most 5120 entries."""
     groups = -(-V // 8)
     slots = -(-groups // slot_groups)
     return 8 * slots * max(1, -(-slot_groups // threads)) + 8
@@ -311,7 +312,7 @@ def test_diagnostics_slot_sizes_agree(monkeypatch):
     """The same bf16 rows (V=24576: 3072 groups, so every consumer warp holds
     groups in a full slot) through ring slots of 16 and 24 warps, of 8 warps
     in two CTAs per SM and 4 in four, of 64, 7 and 1 groups (the last wraps
-    the ring hundreds of times per pass) and the one-CTA kernel: results
+    the ring hundreds of times per pass) and the split kernel: results
     differ by summation order only."""
     V, T = 24576, 16
     z, zi, ids = _rows(12, T, V, torch.bfloat16)
