@@ -37,6 +37,7 @@ NOMINAL_HBM_GBS = 8000.0
 # the sources of each profiled kernel: a summary's traffic figure is used only
 # while their hash matches the one recorded with it
 FUSED_SOURCES = ["paper_2609_32444_gb300/csrc/cis_cluster.cu",
+                 "paper_2609_32444_gb300/csrc/cis_cluster.cuh",
                  "paper_2609_32444_gb300/csrc/cis_dsmem.cuh",
                  "paper_2609_32444_gb300/csrc/cis_common.cuh"]
 DIAG_SOURCES = ["paper_2609_32444_gb300/csrc/cis_diag.cu",

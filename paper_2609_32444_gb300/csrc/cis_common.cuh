@@ -730,7 +730,7 @@ __device__ __forceinline__ RowScalars row_scalars(MaxSum o, float zy, bool exact
         // every other entry is -inf: p = 1
         r.lp = zy != zy ? zy : 0.0f;
         r.lp_lo = 0.0f;
-        r.omp = 0.0f;
+        r.omp = r.lp;  // 0, or NaN
         r.lse = zy;
         r.m = 0.0f;
         r.bias_log2 = INFINITY;

@@ -152,3 +152,18 @@ def test_weights_and_sampled_gradients_keep_their_roundings():
     out = binding.cis_loss_fwd_bwd(z, ids.int(), linf, adv, binding.cis_default_params("none"))
     got, want = out["dlogits"][r, ids].double(), torch.expm1(lp) / T
     assert float(((got - want) / want).abs()[~high].max()) <= 1.2 * u
+
+
+@pytest.mark.parametrize("dtype", [BF16, F32])
+@pytest.mark.parametrize("T,V", [(3, 1), (3, 8), (3, 9), (3, 1001)])
+def test_nan_sampled_entry_without_others(dtype, T, V):
+    """A NaN logit makes its row's outputs NaN, also where every other entry is at -inf
+    (or there is none); the rows around it are not touched."""
+    z = torch.zeros((T, V), dtype=dtype, device=DEV)
+    z[1, 1:] = -math.inf
+    z[1, 0] = math.nan
+    out = binding.cis_loss_fwd_bwd(z, torch.zeros(T, dtype=torch.int32, device=DEV),
+                                   torch.full((T,), -0.5, device=DEV),
+                                   torch.ones(T, device=DEV), binding.cis_default_params("none"))
+    assert bool(torch.isnan(out["lp"][1])) and bool(torch.isnan(out["dlogits"][1, 0]))
+    assert bool(torch.isfinite(out["dlogits"][::2].float()).all())
