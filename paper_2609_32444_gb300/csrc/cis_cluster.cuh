@@ -39,7 +39,7 @@ struct ClusterPlan {
     int cs;
     int64_t slice;
     size_t smem;
-    int nt;  // CTA width: 0 for the default (CIS_CLUSTER_THREADS, else 256)
+    int nt;  // CTA width: 0 for the default (CIS_CLUSTER_THREADS, else plan_threads)
 };
 
 

@@ -580,10 +580,11 @@ __device__ __forceinline__ MaxSumU block_msu(MaxSumU v, MaxSumU *sh)
 
 // The row's probabilities straight from its statistics, without logarithms.
 // From (m', s') over j != y and z_y, with t = s' e^{m' - z_y} = (1 - p) / p:
-//   p = 1 / (1 + t),   1 - p = t p,
+//   p = 1 / (1 + t),   1 - p = t p  (kFine: 1 - p itself where p <= 1/2),
 // each within ~8 ulp (expf, __fdividef: 2 ulp each), so that k = p e^{-l_inf} (the
 // exponential formed ahead of time) and the bounds it is compared with carry
-// relative errors near 2e-6, inside certain_cmp's 4e-6 (a + b).  False where these forms would leave the normal fp32 range
+// relative errors near 2e-6, inside certain_cmp's 4e-6 (a + b).  False where these
+// forms would leave the normal fp32 range
 // (|m' - z_y| > 70, an empty or non-finite row): the caller then takes the
 // log-domain path (row_scalars, token_weight, token_loss), as it does where a
 // decision is too close to call; that path's fp64 fallback settles it.
