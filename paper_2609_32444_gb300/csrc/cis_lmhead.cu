@@ -771,11 +771,9 @@ struct DualList {
         return false;
     }
 };
-template <bool MC>
-__device__ __forceinline__ DualList dual_list(const GemmArgs &g0, const GemmArgs &g1, int c,
-                                              int G)
+// n0 dH units of k0 K blocks and n1 dW units of k1.
+__host__ __device__ __forceinline__ DualList list_of(int n0, int k0, int n1, int k1, int c, int G)
 {
-    const int n0 = n_tiles<MC>(g0) * g0.splits, n1 = n_tiles<MC>(g1) * g1.splits;
     const int q = n0 / G, r = n0 - q * G;
     DualList d;
     d.c = c;
@@ -783,13 +781,20 @@ __device__ __forceinline__ DualList dual_list(const GemmArgs &g0, const GemmArgs
     d.L = r ? G - r : 0;
     d.pos = c >= r ? c - r : c - r + G;
     d.n_dh = q + (c < r);
-    const int cost1 = g1.ksplit > kDwBlocks ? g1.ksplit : kDwBlocks;
-    const int x = d.L ? g0.ksplit / cost1 : 0;
+    const int cost1 = k1 > kDwBlocks ? k1 : kDwBlocks;
+    const int x = d.L ? k0 / cost1 : 0;
     d.A = d.L * x < n1 ? d.L * x : n1;
     d.n_a = d.pos < d.L && d.A > d.pos ? (d.A - d.pos + d.L - 1) / d.L : 0;
     const int rest = n1 - d.A - d.pos;
     d.n_b = rest > 0 ? (rest + G - 1) / G : 0;
     return d;
+}
+template <bool MC>
+__device__ __forceinline__ DualList dual_list(const GemmArgs &g0, const GemmArgs &g1, int c,
+                                              int G)
+{
+    return list_of(n_tiles<MC>(g0) * g0.splits, g0.ksplit, n_tiles<MC>(g1) * g1.splits, g1.ksplit,
+                   c, G);
 }
 
 // GEMM 0: dH (+)= dz W_c (A = dz K-major, B = W MN-major, EPI0 = kStore on
@@ -1383,7 +1388,42 @@ static int split_count(int64_t T, int64_t w, int64_t Hd)
     S = S < kMaxSplits ? S : kMaxSplits;
     return S > 1 ? (int)S : 1;
 }
-// The chunk and the split for a workspace that holds chunks of `widest` columns.
+// The K blocks of the longest list (cis_lmhead_dual_kernel) that dH and dW of a chunk of w
+// columns give a group: the first group's, or that of the first with a unit of dH less.
+static int64_t dual_blocks(int64_t T, int64_t w, int64_t Hd, int splits)
+{
+    const int64_t nH = Hd / lm::kBN, nM = (T + lm::kBM - 1) / lm::kBM;
+    const int64_t nV = (w + lm::kBM - 1) / lm::kBM;
+    const bool pairs = nM > 1;
+    const int64_t c0 = (w + lm::kBK - 1) / lm::kBK, c1 = (T + lm::kBK - 1) / lm::kBK;
+    const int64_t k0 = (c0 + splits - 1) / splits;
+    const int64_t n0 = (pairs ? (nM + 1) / 2 : nM) * nH * ((c0 + k0 - 1) / k0);
+    const int64_t n1 = (pairs ? (nV + 1) / 2 : nV) * nH;
+    const int64_t G = std::min<int64_t>(pairs ? kSplitSms / 2 : kSplitSms, n0 + n1);
+    int64_t most = 0;
+    for (const int64_t c : {(int64_t)0, n0 % G}) {
+        const lm::DualList l = lm::list_of((int)n0, (int)k0, (int)n1, (int)c1, (int)c, (int)G);
+        most = std::max(most, l.n_dh * k0 + (l.n_a + l.n_b) * std::max<int64_t>(c1, lm::kDwBlocks));
+    }
+    return most;
+}
+// What a plan costs beside the logits' products, in K blocks of 0.34 us: the chunks' lists;
+// 18 us a chunk for its two launches' ends; 0.9 us a MB for dH's products where there are
+// several.  (Fitted to 61 shapes; the lists alone differ from the measured times by these.)
+static double plan_blocks(int64_t T, int64_t V, int64_t Hd, int64_t Vc, int splits)
+{
+    const int64_t whole = V / Vc, w = V - whole * Vc;
+    double b = (double)whole * (54.0 + (double)dual_blocks(T, Vc, Hd, splits));
+    if (w > 0)
+        b += 54.0 + (double)dual_blocks(T, w, Hd, splits);
+    return splits > 1 ? b + 2.7e-6 * 4.0 * (double)T * (double)Hd * (double)splits : b;
+}
+// The chunk and the split for a workspace that holds chunks of `widest` columns.  A split
+// that plan_blocks puts more than 5% above none is not made: with 0.3 units of dH and more a
+// cluster (T=2000, V=8000, H=1024: 166 us against 136; T=6000, V=20000, H=512: 468, 392;
+// T=8192, V=32000, H=256: 689, 604; T=3739, V=45176, H=1024: 990, 925) or short chunks
+// (T=768, V=8000, H=1536: 198, 125).  Up to 5% above, what it leaves out (dz in L2) pays:
+// T=512, V=151936, H=4096 1959 against 2082.
 static Split split_for(int64_t T, int64_t V, int64_t Hd, int64_t widest, size_t bytes)
 {
     if (T <= 0 || split_count(T, widest < V ? widest : V, Hd) == 1)
@@ -1396,8 +1436,11 @@ static Split split_for(int64_t T, int64_t V, int64_t Hd, int64_t widest, size_t 
         const int64_t want = split_count(T, Vc < V ? Vc : V, Hd);
         const int64_t fit = (int64_t)((bytes - base) / (4 * (size_t)T * (size_t)Hd));
         const int64_t S = want < fit ? want : fit;
-        if (S > 1 && 2 * S >= want)
+        if (S > 1 && 2 * S >= want) {
+            if (plan_blocks(T, V, Hd, Vc, (int)S) > 1.05 * plan_blocks(T, V, Hd, widest, 1))
+                break;
             return {Vc, (int)S, base};
+        }
     }
     return {widest, 1, 0};
 }
