@@ -1408,21 +1408,21 @@ static int64_t dual_blocks(int64_t T, int64_t w, int64_t Hd, int splits)
     return most;
 }
 // What a plan costs beside the logits' products, in K blocks of 0.34 us: the chunks' lists;
-// 18 us a chunk for its two launches' ends; 0.9 us a MB for dH's products where there are
-// several.  (Fitted to 61 shapes; the lists alone differ from the measured times by these.)
+// 28 us a chunk for its two launches' ends; 0.5 us a MB for dH's products where there are
+// several.  (Fitted to 106 shapes; the lists alone differ from the measured times by these.)
 static double plan_blocks(int64_t T, int64_t V, int64_t Hd, int64_t Vc, int splits)
 {
     const int64_t whole = V / Vc, w = V - whole * Vc;
-    double b = (double)whole * (54.0 + (double)dual_blocks(T, Vc, Hd, splits));
+    double b = (double)whole * (85.0 + (double)dual_blocks(T, Vc, Hd, splits));
     if (w > 0)
-        b += 54.0 + (double)dual_blocks(T, w, Hd, splits);
-    return splits > 1 ? b + 2.7e-6 * 4.0 * (double)T * (double)Hd * (double)splits : b;
+        b += 85.0 + (double)dual_blocks(T, w, Hd, splits);
+    return splits > 1 ? b + 1.5e-6 * 4.0 * (double)T * (double)Hd * (double)splits : b;
 }
 // The chunk and the split for a workspace that holds chunks of `widest` columns.  A split
 // that plan_blocks puts more than 5% above none is not made: with 0.3 units of dH and more a
 // cluster (T=2000, V=8000, H=1024: 166 us against 136; T=6000, V=20000, H=512: 468, 392;
 // T=8192, V=32000, H=256: 689, 604; T=3739, V=45176, H=1024: 990, 925) or short chunks
-// (T=768, V=8000, H=1536: 198, 125).  Up to 5% above, what it leaves out (dz in L2) pays:
+// (T=768, V=8000, H=1536: 198, 125; T=532, V=7136, H=256: 91, 83).  Up to 5% above, what it leaves out (dz in L2) pays:
 // T=512, V=151936, H=4096 1959 against 2082.
 static Split split_for(int64_t T, int64_t V, int64_t Hd, int64_t widest, size_t bytes)
 {
